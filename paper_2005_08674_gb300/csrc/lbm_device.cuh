@@ -407,10 +407,10 @@ __device__ __forceinline__ float2 v_add(float2 a, float2 b) { return __fadd2_rn(
 __device__ __forceinline__ float v_neg(float a) { return -a; }
 __device__ __forceinline__ double v_neg(double a) { return -a; }
 __device__ __forceinline__ float2 v_neg(float2 a) { return make_float2(-a.x, -a.y); }
-template <typename V>
-__device__ __forceinline__ V v_sub(V a, V b) {
-  return v_add(a, v_neg(b));  // a - b = a + (-b), rounded once
-}
+// a - b rounded once; on two nodes as b * (-1) + a, which rounds alike
+__device__ __forceinline__ float v_sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double v_sub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ float2 v_sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ float v_mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double v_mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float2 v_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
@@ -424,120 +424,139 @@ __device__ __forceinline__ V v_splat(C c) {
   else
     return V(c);
 }
-__device__ __forceinline__ float v_div_rho(float a, float rho) { return div_rho(a, rho); }
-__device__ __forceinline__ double v_div_rho(double a, double rho) { return div_rho(a, rho); }
-__device__ __forceinline__ float2 v_div_rho(float a, float2 rho) {
-  return make_float2(div_rho(a, rho.x), div_rho(a, rho.y));
+// 1 / a for the velocity u = (rho u) / rho.  float: the hardware's
+// approximate reciprocal (within 1 ulp).  double: its gross approximation
+// (about 20 bits) and one third-order step of Householder's iteration,
+// r (1 + e + e^2) with e = 1 - a r, which leaves an error of e^3 (2^-60)
+// before the last rounding: three FP64 operations where the IEEE division
+// takes about nine, on a chip whose FP64 pipe issues one warp instruction
+// in 16 cycles.
+__device__ __forceinline__ float v_rcp(float a) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return r;
 }
-// the moments' sums (as moments() forms them) in this arithmetic
-template <typename V>
-__device__ __forceinline__ void v_moments(const V (&h)[9], V& drho, V& jx, V& jy) {
-  drho = v_add(v_add(v_add(v_add(h[0], h[1]), v_add(h[2], h[3])), v_add(v_add(h[4], h[5]), v_add(h[6], h[7]))),
-               h[8]);
-  const V a = v_sub(h[5], h[6]);
-  jx = v_add(v_add(v_sub(h[1], h[2]), a), v_sub(h[8], h[7]));
-  jy = v_add(v_add(v_sub(h[3], h[4]), a), v_sub(h[7], h[8]));
+__device__ __forceinline__ double v_rcp(double a) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  const double e = __fma_rn(-a, r, 1.0);
+  return __fma_rn(r, __fma_rn(e, e, e), r);
 }
+__device__ __forceinline__ float2 v_rcp(float2 a) { return make_float2(v_rcp(a.x), v_rcp(a.y)); }
 
-// Equilibrium in deviations from the far field: E_i = f_i^eq(rho, u) -
-// f_i^eq(rho0, u0) (Eq. feq_1 at two states, cs^2 = 1/3) times the weight
-// scale ws, from d = rho - rho0, v = u - u0 and the momentum deviation
-// J = rho v (= rho u - rho0 u0 - d u0).  With
-//   P_i(u) = 1 + 3 c_i.u + 4.5 (c_i.u)^2 - 1.5 u.u   (so f_i^eq = w_i rho P_i(u)),
-//   E_i = w_i [ d P_i(u0) + 3 c_i.J + rho Q_i ],
-//   Q_i = 4.5 (c_i.v)(c_i.s) - 1.5 v.s,   s = u + u0 = 2 u0 + v,
-// (rho (P_i(u) - P_i(u0)) = 3 c_i.J + rho Q_i), every term is of the size of
-// the disturbance, so float rounding is relative to it even in a mean flow:
-// forming f^eq(rho, u) and subtracting f^eq(m0) instead rounds terms of the
-// size of the stream's equilibrium (0.04 per population at Ma 0.1) every
-// step, and in a steady flow those roundings -- which do not conserve mass or
-// momentum -- add up step after step.  The first-order term takes J as summed
-// from the populations, not rho times a rounded quotient, so the momentum a
-// BGK relaxation puts back is the node's own to the rounding of each term.
-// For a far field at rest (SHIFT false: rho0 = 1, u0 = 0, P_i(u0) = 1) this
-// is w_i (d + 3 c_i.J + rho (4.5 (c_i.u)^2 - 1.5 u.u)).
+// ---------------------------------------------------------------------------
+// The interior collision, from the pairs of opposite populations.
+//
+// With d = rho - rho0 = sum h, j = sum c h (the momentum's deviation from
+// rho0 u0), J = rho (u - u0) = j - d u0, v = u - u0 = J / rho, the deviation
+// of the equilibrium (Eq. feq_1) from the far field's is
+//   E_i = f_i^eq(rho, u) - f_i^eq(rho0, u0)
+//       = w_i [ d + 3 c_i.j + 4.5 c_i c_i : Pi - 1.5 tr Pi ],
+//   Pi  = rho u u - rho0 u0 u0 = d u0 u0 + J u0 + u0 J + J v,
+// so with a = Pi_xx, b = Pi_yy, c = Pi_xy, q = a + b
+//   E_0     = w_0 [ d - 1.5 q ],
+//   E_{1,2} = w_1 [ d - 1.5 q + 4.5 a +- 3 j_x ],   E_{3,4} with b, j_y,
+//   E_{5,6} = w_5 [ d + 3 q + 9 c +- 3 (j_x + j_y) ],
+//   E_{7,8} = w_5 [ d + 3 q - 9 c +- 3 (j_y - j_x) ].
+// Every term is of the size of the disturbance, so float rounding is
+// relative to it in a mean flow too, and the linear term takes j as summed
+// from the populations.  Everything is held in stored units (times the
+// storage scale s, a power of two): 1 / (s rho) turns s J into v.
+//
+// These kernels are bound by instruction issue (f32 and 16 bit) or by the
+// FP64 pipe (f64), so the operations are what counts: 55 for BGK and 67 for
+// MRT plus the reciprocal.  Forming the nine E_i one by one and relaxing each
+// population took 81 and 138 and an IEEE division in f64.  Every operation
+// is rounded on its own (v_add / v_mul / v_fma), so the shifted form with a
+// zero shift rounds exactly like the plain one, and two nodes at once like
+// one at a time.
+// ---------------------------------------------------------------------------
+template <typename V>
+struct CellSums {
+  V s1, s3, s5, s7;  // h_i + h_opp(i)
+  V t1, t3;          // h_i - h_opp(i)
+  V m, p;            // t5 - t7, t5 + t7
+  V sa, sd;          // s1 + s3, s5 + s7
+  V d, jx, jy;       // moments
+  V a, b, c, q;      // Pi_xx, Pi_yy, Pi_xy, trace
+};
+
 template <bool SHIFT, typename V, typename C>
-__device__ __forceinline__ void equilibrium_dev(V d, V vx, V vy, V jx, V jy, const Shift<C>& z, V (&e)[9],
-                                                C ws = C(1)) {
-  // every operation is rounded on its own (v_add / v_mul / v_fma), so that
-  // the shifted form with a zero shift (rho0 = 1, u0 = 0, P_i(u0) = 1) rounds
-  // exactly like the plain one, and two nodes at once like one at a time
-  V rho, sx, sy;
+__device__ __forceinline__ void cell_sums(const V (&h)[9], const Shift<C>& z, C s, CellSums<V>& o) {
+  o.s1 = v_add(h[1], h[2]);
+  o.t1 = v_sub(h[1], h[2]);
+  o.s3 = v_add(h[3], h[4]);
+  o.t3 = v_sub(h[3], h[4]);
+  o.s5 = v_add(h[5], h[6]);
+  o.s7 = v_add(h[7], h[8]);
+  const V t5 = v_sub(h[5], h[6]), t7 = v_sub(h[7], h[8]);
+  o.m = v_sub(t5, t7);
+  o.p = v_add(t5, t7);
+  o.sa = v_add(o.s1, o.s3);
+  o.sd = v_add(o.s5, o.s7);
+  o.d = v_add(v_add(o.sa, o.sd), h[0]);
+  o.jx = v_add(o.t1, o.m);
+  o.jy = v_add(o.t3, o.p);
   if constexpr (SHIFT) {
-    rho = v_add(v_splat<V>(z.rho0), d);
-    sx = v_fma(v_splat<V>(C(2)), v_splat<V>(z.u0[0]), vx);
-    sy = v_fma(v_splat<V>(C(2)), v_splat<V>(z.u0[1]), vy);
+    const C ux = z.u0[0], uy = z.u0[1];
+    const V inv = v_rcp(v_add(v_splat<V>(mul_rn(s, z.rho0)), o.d));
+    const V Jx = v_fma(v_splat<V>(-ux), o.d, o.jx), Jy = v_fma(v_splat<V>(-uy), o.d, o.jy);
+    const V vx = v_mul(Jx, inv), vy = v_mul(Jy, inv);
+    // s = 2 u0 + v and u0 + v as multiply-adds: a paired addition that takes a
+    // paired product may be fused with it, and would then round differently
+    const V one = v_splat<V>(C(1)), two = v_splat<V>(C(2)), u = v_splat<V>(ux), w = v_splat<V>(uy);
+    const V sx = v_fma(two, u, vx), sy = v_fma(two, w, vy);
+    o.a = v_fma(o.d, v_splat<V>(mul_rn(ux, ux)), v_mul(Jx, sx));
+    o.b = v_fma(o.d, v_splat<V>(mul_rn(uy, uy)), v_mul(Jy, sy));
+    o.c = v_fma(u, Jy, v_fma(o.d, v_splat<V>(mul_rn(ux, uy)), v_mul(Jx, v_fma(one, w, vy))));
   } else {
-    rho = v_add(v_splat<V>(C(1)), d);
-    sx = vx;
-    sy = vy;
+    const V inv = v_rcp(v_add(v_splat<V>(s), o.d));
+    const V vx = v_mul(o.jx, inv), vy = v_mul(o.jy, inv);
+    o.a = v_mul(o.jx, vx);
+    o.b = v_mul(o.jy, vy);
+    o.c = v_mul(o.jx, vy);
   }
-  V dp[9];  // d P_i(u0)
-#pragma unroll
-  for (int i = 0; i < 9; ++i) dp[i] = SHIFT ? v_mul(d, v_splat<V>(z.p0[i])) : d;
-  const V vs = v_mul(v_splat<V>(C(1.5)), v_fma(vx, sx, v_mul(vy, sy)));
-  const V nvs = v_neg(vs);
-  const V w0 = v_splat<V>(wt<C>(0) * ws), wa = v_splat<V>(wt<C>(1) * ws), wd = v_splat<V>(wt<C>(5) * ws);
-  const V c45 = v_splat<V>(C(4.5)), c3 = v_splat<V>(C(3));
-  e[0] = v_mul(w0, v_fma(v_neg(rho), vs, dp[0]));
-  // axis directions: c.v = +-vx, +-vy
-  {
-    const V q = v_fma(v_mul(c45, vx), sx, nvs), b = v_mul(c3, jx);
-    e[1] = v_mul(wa, v_add(v_fma(rho, q, dp[1]), b));
-    e[2] = v_mul(wa, v_sub(v_fma(rho, q, dp[2]), b));
-  }
-  {
-    const V q = v_fma(v_mul(c45, vy), sy, nvs), b = v_mul(c3, jy);
-    e[3] = v_mul(wa, v_add(v_fma(rho, q, dp[3]), b));
-    e[4] = v_mul(wa, v_sub(v_fma(rho, q, dp[4]), b));
-  }
-  {
-    const V cv = v_add(vx, vy), cs = v_add(sx, sy);  // c_5 = -c_6 = (1, 1)
-    const V q = v_fma(v_mul(c45, cv), cs, nvs), b = v_mul(c3, v_add(jx, jy));
-    e[5] = v_mul(wd, v_add(v_fma(rho, q, dp[5]), b));
-    e[6] = v_mul(wd, v_sub(v_fma(rho, q, dp[6]), b));
-  }
-  {
-    const V cv = v_sub(vy, vx), cs = v_sub(sy, sx);  // c_7 = -c_8 = (-1, 1)
-    const V q = v_fma(v_mul(c45, cv), cs, nvs), b = v_mul(c3, v_sub(jy, jx));
-    e[7] = v_mul(wd, v_add(v_fma(rho, q, dp[7]), b));
-    e[8] = v_mul(wd, v_sub(v_fma(rho, q, dp[8]), b));
-  }
+  o.q = v_add(o.a, o.b);
 }
 
 // BGK collision, Eq. (lbe_1) with dt = 1, on shifted populations held as
-// s * h (s = storage scale; the relaxation is linear in h, only the moments
-// need 1/s).  Written as h* = (1 - omega) h + omega h^eq with omega folded
-// into the equilibrium weights: one fused multiply-add per population.
-// With a storage shift (SHIFT: a far field not at rest) the velocity enters
-// as its deviation v = u - u0 = (sum c h - d u0) / rho and the equilibrium as
-// its deviation from f^eq(m0) (equilibrium_dev), so no term of the size of
-// the stream's equilibrium is ever rounded.  The relaxation is one explicitly
-// rounded fused multiply-add per population in both forms, and the shifted
-// form with a zero shift gives the same bits as the plain one.
+// s * h: h* = (1 - omega) h + omega E, by pairs: with S = (h*_i + h*_opp) / 2
+// and T = (h*_i - h*_opp) / 2,
+//   S_i = keep/2 s_i + omega w_i [ ... ],   X = T_5 - T_7, Y = T_5 + T_7,
+// and what the relaxation conserves closes the rest: T_1 = j_x / 2 - X,
+// T_3 = j_y / 2 - Y, h*_0 = d - 2 (S_1 + S_3 + S_5 + S_7).  Mass and momentum
+// are then kept to the rounding of each sum; relaxing every population with
+// its own rounded omega w_i lost up to 1e-7 of the disturbance per step (the
+// rounded weights do not add up to omega), which after 100 steps was the
+// whole f32 error.
 template <bool SHIFT, typename V, typename C>
 __device__ __forceinline__ void collide_bgk(V (&h)[9], const Rates<C>& r, C s = C(1)) {
-  const C omega = r.omega;
-  V sd, sjx, sjy;
-  v_moments(h, sd, sjx, sjy);
-  const C is = C(1) / s;
-  const V vis = v_splat<V>(is);
-  const V d = v_mul(sd, vis);  // rho - rho0
-  V e[9];
-  if constexpr (SHIFT) {
-    // J = rho (u - u0) = sum c h - d u0 and v = J / rho, from small quantities only
-    const V inv = v_div_rho(is, v_add(v_splat<V>(r.z.rho0), d));
-    const V nsd = v_neg(sd);
-    const V jx = v_fma(nsd, v_splat<V>(r.z.u0[0]), sjx), jy = v_fma(nsd, v_splat<V>(r.z.u0[1]), sjy);
-    equilibrium_dev<true>(d, v_mul(jx, inv), v_mul(jy, inv), v_mul(jx, vis), v_mul(jy, vis), r.z, e, s * omega);
-  } else {
-    const V inv = v_div_rho(is, v_add(v_splat<V>(C(1)), d));
-    equilibrium_dev<false>(d, v_mul(sjx, inv), v_mul(sjy, inv), v_mul(sjx, vis), v_mul(sjy, vis), r.z, e,
-                           s * omega);
-  }
-  const V keep = v_splat<V>(C(1) - omega);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) h[i] = v_fma(keep, h[i], e[i]);
+  CellSums<V> n;
+  cell_sums<SHIFT>(h, r.z, s, n);
+  const C omega = r.omega, k2c = mul_rn(C(0.5), sub_rn(C(1), omega));
+  const C wa = mul_rn(omega, wt<C>(1)), wd = mul_rn(C(0.25), wa);
+  const V k2 = v_splat<V>(k2c);
+  const V ba = v_fma(v_splat<V>(mul_rn(C(-1.5), wa)), n.q, v_mul(v_splat<V>(wa), n.d));
+  const V bd = v_fma(v_splat<V>(mul_rn(C(3), wd)), n.q, v_mul(v_splat<V>(wd), n.d));
+  const V wa45 = v_splat<V>(mul_rn(C(4.5), wa));
+  const V S1 = v_fma(k2, n.s1, v_fma(wa45, n.a, ba));
+  const V S3 = v_fma(k2, n.s3, v_fma(wa45, n.b, ba));
+  const V S5 = v_fma(k2, n.s5, v_fma(v_splat<V>(mul_rn(C(9), wd)), n.c, bd));
+  const V S7 = v_fma(k2, n.s7, v_fma(v_splat<V>(mul_rn(C(-9), wd)), n.c, bd));
+  const V wd6 = v_splat<V>(mul_rn(C(6), wd));
+  const V X = v_fma(k2, n.m, v_mul(wd6, n.jx)), Y = v_fma(k2, n.p, v_mul(wd6, n.jy));
+  const V half = v_splat<V>(C(0.5)), mhalf = v_splat<V>(C(-0.5));
+  const V T1 = v_fma(half, n.jx, v_neg(X)), T3 = v_fma(half, n.jy, v_neg(Y));
+  const V U5 = v_add(X, Y), U7 = v_sub(Y, X);  // 2 T_5, 2 T_7
+  h[0] = v_fma(v_splat<V>(C(-2)), v_add(v_add(S1, S3), v_add(S5, S7)), n.d);
+  h[1] = v_add(S1, T1);
+  h[2] = v_sub(S1, T1);
+  h[3] = v_add(S3, T3);
+  h[4] = v_sub(S3, T3);
+  h[5] = v_fma(half, U5, S5);
+  h[6] = v_fma(mhalf, U5, S5);
+  h[7] = v_fma(half, U7, S7);
+  h[8] = v_fma(mhalf, U7, S7);
 }
 
 // ---------------------------------------------------------------------------
@@ -552,53 +571,47 @@ __device__ __forceinline__ void collide_bgk(V (&h)[9], const Rates<C>& r, C s = 
 //   pxy = ( 0,  0,  0,  0,  0,  1,  1, -1, -1)   |pxy|^2 = 4
 // The rows are orthogonal, so M^-1 = M^T diag(1/|row|^2); a row scale does
 // not change M^-1 S M.  The conserved moments of f - f^eq vanish, so their
-// rates (C_rho, C_jx, C_jy) never enter.  The stress rate is 1/tau.
+// rates (C_rho, C_jx, C_jy) never enter.  The stress rate is 1/tau.  The
+// moments of E (above) are e: -2 d + 3 q, eps: d - 3 q, q: -j, pxx: a - b,
+// pxy: c, so the non-equilibrium moments need no equilibrium populations:
+//   e   : -2 h0 + sa + 4 sd - 3 q      eps : 3 (h0 - sa + q)
+//   qx  : 2 m - t1                     qy  : 2 p - t3
+//   pxx : (s1 - s3) - (a - b)          pxy : (s5 - s7) - c
 // ---------------------------------------------------------------------------
-
-template <bool SHIFT, typename C>
-__device__ __forceinline__ void collide_mrt(C (&h)[9], const Rates<C>& r, C s = C(1)) {
-  C sd, sjx, sjy;
-  moments(h, sd, sjx, sjy);
-  const C is = C(1) / s;
-  const C dr = sd * is;  // rho - rho0
-  C e[9];
-  if constexpr (SHIFT) {
-    const C inv = div_rho(is, r.z.rho0 + dr);
-    const C jx = fma_rn(-sd, r.z.u0[0], sjx), jy = fma_rn(-sd, r.z.u0[1], sjy);
-    equilibrium_dev<true>(dr, jx * inv, jy * inv, jx * is, jy * is, r.z, e, s);
-  } else {
-    const C inv = div_rho(is, C(1) + dr);
-    equilibrium_dev<false>(dr, sjx * inv, sjy * inv, sjx * is, sjy * is, r.z, e, s);
-  }
-  C n[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) n[i] = sub_rn(h[i], e[i]);
-  const C ax = n[1] + n[2], ay = n[3] + n[4], d = (n[5] + n[6]) + (n[7] + n[8]);
-  const C me = C(-4) * n[0] - (ax + ay) + C(2) * d;
-  const C mep = C(4) * n[0] - C(2) * (ax + ay) + d;
-  const C mqx = C(-2) * (n[1] - n[2]) + ((n[5] - n[6]) + (n[8] - n[7]));
-  const C mqy = C(-2) * (n[3] - n[4]) + ((n[5] - n[6]) + (n[7] - n[8]));
-  const C mxx = ax - ay;
-  const C mxy = (n[5] + n[6]) - (n[7] + n[8]);
-  const C re = r.s_e * me * C(1.0 / 36.0), rep = r.s_eps * mep * C(1.0 / 36.0);
-  const C rqx = r.s_q * mqx * C(1.0 / 12.0), rqy = r.s_q * mqy * C(1.0 / 12.0);
-  const C rxx = r.omega * mxx * C(0.25), rxy = r.omega * mxy * C(0.25);
-  const C a0 = C(-1) * re - C(2) * rep;  // e/eps part of the axis columns
-  const C a1 = C(2) * re + rep;          // e/eps part of the diagonal columns
-  h[0] -= C(4) * (rep - re);
-  h[1] -= a0 - C(2) * rqx + rxx;
-  h[2] -= a0 + C(2) * rqx + rxx;
-  h[3] -= a0 - C(2) * rqy - rxx;
-  h[4] -= a0 + C(2) * rqy - rxx;
-  h[5] -= a1 + rqx + rqy + rxy;
-  h[6] -= a1 - rqx - rqy + rxy;
-  h[7] -= a1 - rqx + rqy - rxy;
-  h[8] -= a1 + rqx - rqy - rxy;
+template <bool SHIFT, typename V, typename C>
+__device__ __forceinline__ void collide_mrt(V (&h)[9], const Rates<C>& r, C s = C(1)) {
+  CellSums<V> n;
+  cell_sums<SHIFT>(h, r.z, s, n);
+  const V two = v_splat<V>(C(2)), mtwo = v_splat<V>(C(-2));
+  const V me = v_fma(v_splat<V>(C(-3)), n.q, v_fma(v_splat<V>(C(4)), n.sd, v_fma(mtwo, h[0], n.sa)));
+  const V mep = v_add(v_sub(h[0], n.sa), n.q);  // a third of it
+  const V mqx = v_fma(two, n.m, v_neg(n.t1)), mqy = v_fma(two, n.p, v_neg(n.t3));
+  const V mxx = v_sub(v_sub(n.s1, n.s3), v_sub(n.a, n.b));
+  const V mxy = v_sub(v_sub(n.s5, n.s7), n.c);
+  const V kw = v_splat<V>(mul_rn(r.omega, C(0.25))), kq = v_splat<V>(mul_rn(r.s_q, C(1.0 / 12.0)));
+  const V re = v_mul(v_splat<V>(mul_rn(r.s_e, C(1.0 / 36.0))), me);
+  const V rep = v_mul(v_splat<V>(mul_rn(r.s_eps, C(1.0 / 12.0))), mep);
+  const V rqx = v_mul(kq, mqx), rqy = v_mul(kq, mqy);
+  const V rxx = v_mul(kw, mxx), rxy = v_mul(kw, mxy);
+  const V a0 = v_fma(mtwo, rep, v_neg(re));  // e/eps part of the axis columns
+  const V a1 = v_fma(two, re, rep);          // e/eps part of the diagonal columns
+  const V ax = v_add(a0, rxx), ay = v_sub(a0, rxx);
+  const V d5 = v_add(a1, rxy), d7 = v_sub(a1, rxy);
+  const V q5 = v_add(rqx, rqy), q7 = v_sub(rqy, rqx);
+  h[0] = v_fma(v_splat<V>(C(-4)), v_sub(rep, re), h[0]);
+  h[1] = v_sub(h[1], v_fma(mtwo, rqx, ax));
+  h[2] = v_sub(h[2], v_fma(two, rqx, ax));
+  h[3] = v_sub(h[3], v_fma(mtwo, rqy, ay));
+  h[4] = v_sub(h[4], v_fma(two, rqy, ay));
+  h[5] = v_sub(h[5], v_add(d5, q5));
+  h[6] = v_sub(h[6], v_sub(d5, q5));
+  h[7] = v_sub(h[7], v_add(d7, q7));
+  h[8] = v_sub(h[8], v_sub(d7, q7));
 }
 
 // Collision model: 0 = BGK (Eq. lbe_1), 1 = MRT (Eq. mrt_lbe).
-template <int MODEL, bool SHIFT, typename C>
-__device__ __forceinline__ void collide(C (&h)[9], const Rates<C>& r, C s = C(1)) {
+template <int MODEL, bool SHIFT, typename V, typename C>
+__device__ __forceinline__ void collide(V (&h)[9], const Rates<C>& r, C s = C(1)) {
   if constexpr (MODEL == 1)
     collide_mrt<SHIFT>(h, r, s);
   else
@@ -606,20 +619,20 @@ __device__ __forceinline__ void collide(C (&h)[9], const Rates<C>& r, C s = C(1)
 }
 
 // The collision of N nodes held as h[i][k] (population i of node k): with
-// PAIRED, in float BGK, two nodes per paired instruction (half the
-// arithmetic instructions, at the price of register pairs: worth it where
-// the kernel is bound by instruction issue and has registers to spare),
-// otherwise one after another; the bits of each node are those of collide()
-// on it alone either way.
+// PAIRED, in float, two nodes per paired instruction (half the arithmetic
+// instructions, at the price of register pairs: worth it where the kernel is
+// bound by instruction issue and has registers to spare), otherwise one
+// after another; the bits of each node are those of collide() on it alone
+// either way.
 template <int MODEL, bool SHIFT, bool PAIRED, typename C, int N>
 __device__ __forceinline__ void collide_nodes(C (&h)[9][N], const Rates<C>& r, C s = C(1)) {
-  if constexpr (PAIRED && MODEL == 0 && std::is_same<C, float>::value && N % 2 == 0) {
+  if constexpr (PAIRED && std::is_same<C, float>::value && N % 2 == 0) {
 #pragma unroll
     for (int k = 0; k < N; k += 2) {
       float2 p[9];
 #pragma unroll
       for (int i = 0; i < 9; ++i) p[i] = make_float2(h[i][k], h[i][k + 1]);
-      collide_bgk<SHIFT>(p, r, s);
+      collide<MODEL, SHIFT>(p, r, s);
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
         h[i][k] = p[i].x;

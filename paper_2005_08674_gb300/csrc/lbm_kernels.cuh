@@ -137,9 +137,11 @@ __device__ __forceinline__ void bulk_row(const T* __restrict__ A, T* __restrict_
   }
 }
 
+// f32: 64 registers (32 resident warps); at 72 (28 warps), which the compiler
+// takes if left free, a 1024^2 step loses 3 %.
 template <typename T, int BX, int MODEL, bool SHIFT = false>
-__global__ void __launch_bounds__(BX) bulk_kernel(const T* __restrict__ A, T* __restrict__ B, Geom g,
-                                                  Rates<typename Store<T>::C> rates, int rows, int pf) {
+__global__ void __launch_bounds__(BX, sizeof(T) == 4 && !SHIFT ? 1024 / BX : 0)
+    bulk_kernel(const T* __restrict__ A, T* __restrict__ B, Geom g, Rates<typename Store<T>::C> rates, int rows, int pf) {
   constexpr int V = Store<T>::V;
   const int lane = threadIdx.x & 31;
   const int x0 = (blockIdx.x * BX + threadIdx.x) * V;
