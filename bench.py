@@ -31,6 +31,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "D2Q9+NSBC MLUPS"
 UNIT = "MLUPS"
+PASS_STEPS = 4  # time steps of one launch of the multi-step pass
 BYTES_PER_CELL = {"f64": 144, "f32": 72, "f16": 36, "bf16": 36}
 CPU_SAMPLE_N = 2048
 
@@ -144,7 +145,7 @@ def measured_peak_gbs():
 
 def kernel_source_sha() -> str:
     h = hashlib.sha256()
-    for name in ("lbm_kernels.cuh", "lbm_device.cuh", "lbm_staged.cuh", "lbm_twostep.cuh"):
+    for name in ("lbm_kernels.cuh", "lbm_device.cuh", "lbm_staged.cuh", "lbm_multistep.cuh"):
         with open(os.path.join(ROOT, "paper_2005_08674_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -154,12 +155,12 @@ def step_kernel(sim, nx, ny):
     """(kernel description, traffic summary file stem, nodes whose state one
     timed launch reads and writes once) of the kernel that carries the step:
     the staged kernel updates every node, the bulk kernel the interior (the
-    NSBC kernel the perimeter, beside it); a two-step pass moves every node's
-    state once for two steps (one launch)."""
+    NSBC kernel the perimeter, beside it); a multi-step pass moves every
+    node's state once for four steps (one launch)."""
     if sim.twostep:
-        return ("two-step pass: pass_kernel, one launch per two steps (step n+1 on the width-3 frame into a "
-                "frame buffer, steps n+1 and n+2 on nodes 2..n-3 by warps rolling down 128-column strips with "
-                "step n+1 in registers, step n+2 on the width-2 frame)", "twostep_traffic", nx * ny)
+        return ("multi-step pass: pass_kernel, one launch per four steps (the nodes at distance 4 or more by warps "
+                "rolling down 64-column strips with the steps in between in registers, the frame as tiles in "
+                "shared memory)", "multistep_traffic", nx * ny)
     if sim.staged:
         return ("batch_ws_kernel (staged step: interior tiles by bulk copies + NSBC chunks, "
                 f"{sim.staged} stages)", "staged_step_traffic", nx * ny)
@@ -458,11 +459,11 @@ def run_ours(args, rank, world, local_rank):
                          "dram_frac": traffic / (bulk_avg * 1e-3) / 1e9 / peak if traffic else None,
                          "kernel": kname,
                          "bytes_per_cell": BYTES_PER_CELL[args.storage], "cells_per_launch": kcells,
-                         "steps_per_launch": 2 if sim.twostep else 1,
+                         "steps_per_launch": PASS_STEPS if sim.twostep else 1,
                          "avg_launch_ms": bulk_avg, "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)",
                          "nsbc_avg_launch_ms": nsbc_avg if nn else None,
                          "timing": f"per-launch CUDA events over {kprof} steps after the timed region"},
-            "gpu_launches": (args.steps // 2 + 2 * (args.steps % 2) if sim.twostep else
+            "gpu_launches": (-(-args.steps // PASS_STEPS) if sim.twostep else
                              (1 if sim.staged or sim.fused else 2) * args.steps),
             "clocks": clk,
         }

@@ -47,7 +47,7 @@ extern "C" {
  * relative to it even in a mean flow.  binary16 holds it scaled by 2^12.
  * Arithmetic: LBM_F64 computes in double everywhere; the other three
  * collide and apply the NSBC in float, with the NSBC gradient extrapolation
- * and far-field blend (Eqs. nes_2, nes_3) in double. */
+ * and far-field blend (Eqs. nes_2, nes_3) as pairs of floats (48 bits). */
 #define LBM_F64 0
 #define LBM_F32 1
 #define LBM_F16 2  /* IEEE binary16, round-to-nearest-even */
@@ -158,10 +158,14 @@ int lbm_init(lbm_t* h, const double* rho, const double* ux, const double* uy);
 /* As lbm_init, from DEVICE fields [ny][nx] double; asynchronous. */
 int lbm_init_device(lbm_t* h, const double* d_rho, const double* d_ux, const double* d_uy);
 
-/* Advance n >= 0 steps, asynchronously on the stream.  Steps are replayed
- * from a CUDA graph of a fixed number of steps captured on first use (and
- * recaptured after lbm_set_nsbc / lbm_set_stream); the remainder is
- * launched directly. */
+/* Advance n >= 0 steps, asynchronously on the stream.  Until lbm_set_launch,
+ * lbm_set_fused, lbm_set_staged, lbm_set_twostep or lbm_autotune chooses, the
+ * launch form goes by size and storage: several steps per launch on small
+ * domains (tiles in shared memory) and on large ones (the pass of
+ * lbm_set_twostep), one launch or the kernel pair per step between; all forms
+ * give the same bits.  Forms of one step are replayed from a CUDA graph of a
+ * fixed number of steps captured on first use (and recaptured after
+ * lbm_set_nsbc / lbm_set_stream); everything else is launched directly. */
 int lbm_step(lbm_t* h, int32_t n);
 
 /* Number of steps taken since the last lbm_init* / lbm_set_populations. */
@@ -267,26 +271,22 @@ int32_t lbm_get_staged(const lbm_t* h);
  * NULL handle. */
 int lbm_set_fused(lbm_t* h, int32_t enable);
 int32_t lbm_get_fused(const lbm_t* h);
-/* Two steps per pass (temporal blocking), in one launch whose warps take, in
- * turn, three kinds of work: step n + 1 on the frame of nodes within
- * distance 2 of an edge (the NSBC and the interior collision) into a small
- * frame buffer; steps n + 1 and n + 2 on the nodes at distance 2 or more,
- * each warp rolling down a strip of 128 columns, staging the state rows by
- * bulk copies and keeping step n + 1 in registers; and, once all of the first
- * kind is done (a bounded wait on a counter), step n + 2 on the frame from
- * the frame buffer.  Every node runs the same device arithmetic as the
- * single-step kernels and step n + 1 is rounded to the storage type as a
- * single step stores it, so the results are bit-identical to the kernel
- * pair, while the state crosses device memory once per two steps.
- * lbm_step(n) runs n / 2 passes (graphs of 16 steps) and, for odd n, one
- * step of the kernel pair.  enable != 0 turns it on (and the staged and fused
- * kernels off); lbm_set_launch, lbm_set_staged and lbm_set_fused turn it off;
- * lbm_autotune times it against the other forms.  LBM_EINVAL when enabling
- * it on an f64 handle, a handle with a periodic axis or fewer than 8 x 8
- * nodes.  A bounded wait that gives up makes lbm_status report LBM_ETIMEOUT.
- * Device memory: a frame buffer of 9 x (6 (nx + ny) - 36) populations,
- * allocated when first enabled.  lbm_get_twostep: 1 if on, 0 if off,
- * LBM_EINVAL for NULL. */
+/* Several steps per pass (temporal blocking; four, and two or three where
+ * fewer are left), one launch each: the nodes at distance 4 or more from every
+ * edge by warps that roll down strips of 64 columns, staging the state rows
+ * by bulk copies and carrying the steps in between in registers; the frame of
+ * nodes nearer to an edge (the NSBC among them) as tiles that blocks advance
+ * in shared memory.  No work item waits for another.  Every node runs the
+ * same device arithmetic as the single-step kernels and the steps in between
+ * are rounded to the storage type as single steps store them, so the results
+ * are bit-identical to the kernel pair, while the state crosses device memory
+ * once per pass.  A lone step is one of the kernel pair.  enable != 0 turns it
+ * on (and the staged and fused kernels off); lbm_set_launch, lbm_set_staged
+ * and lbm_set_fused turn it off; lbm_autotune times it against the other
+ * forms.  LBM_EINVAL when enabling it on an f64 handle, a handle with a
+ * periodic axis or fewer than 8 x 8 nodes.  A bounded wait that gives up makes
+ * lbm_status report LBM_ETIMEOUT.  No device memory of its own.
+ * lbm_get_twostep: 1 if on, 0 if off, LBM_EINVAL for NULL. */
 int lbm_set_twostep(lbm_t* h, int32_t enable);
 int32_t lbm_get_twostep(const lbm_t* h);
 /* LBM_ETIMEOUT if a bounded wait of the staged kernel gave up (the state is
@@ -294,8 +294,8 @@ int32_t lbm_get_twostep(const lbm_t* h);
 int lbm_status(lbm_t* h);
 
 /* Time every compiled bulk launch shape and prefetch distance (as the
- * kernel pair and as the fused one-launch step), and the staged kernel with
- * 3 and 4 stages, on this handle's own buffers (a few whole steps each,
+ * kernel pair and as the fused one-launch step), the staged kernel with 3 and
+ * 4 stages and the forms of several steps, on this handle's own buffers (a few whole steps each,
  * CUDA events on the stream) and keep the fastest; the state is restored
  * afterwards (through a temporary device copy from cudaMallocAsync).  Writes
  * the bulk shape, and the time per step in milliseconds of the winner, to
@@ -433,22 +433,22 @@ int lbm_batch_unstable_nodes(lbm_batch_t* b, int32_t k, int64_t* count);
  * shape not compiled. */
 int lbm_batch_set_launch(lbm_batch_t* b, int32_t threads_x, int32_t rows, int32_t blocks, int32_t prefetch_rows,
                          int32_t split, int32_t tma_tile);
-/* Two steps per pass for every instance (the pass lbm_set_twostep describes,
- * here in three launches over all instances: step n + 1 on every frame, the
- * rolling items in bands of at most 64 output rows, claimed by warps from a
- * counter, largest instance first, beside the frame launches on a side
- * stream, then step n + 2 on every frame; each instance's frame buffer after
- * the last).  Bit-identical to two batched steps.  lbm_batch_step(n) runs n / 2
- * passes (graphs of 16 steps) and, for odd n, one batched step of the launch
- * shape set.  enable != 0 turns it on; lbm_batch_set_launch turns it off;
- * lbm_batch_autotune times it against the other forms.  LBM_EINVAL when
- * enabling it on f64 storage, with a periodic axis, or with an instance
- * smaller than 8 x 8.  lbm_batch_get_twostep: 1 on, 0 off, LBM_EINVAL for
- * NULL. */
+/* Several steps per pass for every instance (the pass lbm_set_twostep
+ * describes, in one launch over all instances: their frame tiles, then the
+ * rolling items, claimed by warps from a counter, largest instance first).
+ * Bit-identical to batched single steps.  lbm_batch_step(n) runs passes of
+ * four steps (graphs of 16 steps), of two or three where fewer are left, and
+ * for a lone step one batched step of the launch shape set.  enable != 0 turns
+ * it on; lbm_batch_set_launch turns it off; a batch for which neither was
+ * called takes passes when it is stored in f32 and has a million nodes or
+ * more (lbm_batch_get_twostep then still reports 0).  lbm_batch_autotune times
+ * it against the other forms.  LBM_EINVAL when enabling it on f64 storage,
+ * with a periodic axis, or with an instance smaller than 8 x 8.
+ * lbm_batch_get_twostep: 1 on, 0 off, LBM_EINVAL for NULL. */
 int lbm_batch_set_twostep(lbm_batch_t* b, int32_t enable);
 int32_t lbm_batch_get_twostep(const lbm_batch_t* b);
 /* Time every compiled tile shape, grid size, prefetch setting and split, the
- * shared-memory paths and the two-step pass, on the batch's own state
+ * shared-memory paths and the multi-step pass, on the batch's own state
  * (restored afterwards, through a temporary device copy from
  * cudaMallocAsync) and keep the fastest. */
 int lbm_batch_autotune(lbm_batch_t* b, int32_t* threads_x, int32_t* rows, int32_t* blocks, int32_t* prefetch_rows,

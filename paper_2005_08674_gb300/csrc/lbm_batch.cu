@@ -34,10 +34,10 @@
 #include "lbm.h"
 #include "lbm_aux.cuh"
 #include "lbm_kernels.cuh"
+#include "lbm_multistep.cuh"
 #include "lbm_staged.cuh"
 #include "lbm_trace.h"
 #include "lbm_tune_cache.h"
-#include "lbm_twostep.cuh"
 
 int lbm_internal_fail(int code, const char* msg);
 // the autotuner cache of lbm_runtime.cu (lbm_set_tune_cache)
@@ -79,6 +79,7 @@ using lbmk::mbar_wait;
 using lbmk::smem_u32;
 
 constexpr int kBatchGraphSteps = 16;
+static_assert(kBatchGraphSteps % (2 * lbmk::kPassSteps) == 0, "a graph returns the pools to their roles");
 constexpr int kBatchBX[] = {64, 128, 256};
 constexpr int kBatchRows[] = {1, 2, 4};
 
@@ -116,15 +117,13 @@ struct lbm_batch {
   int wave = 1;                        // resident blocks on the device for the current shape
   int tile = 128;                      // > 0: bulk tiles of this many vectors staged by bulk copies
   int* d_err = nullptr;                // [0] work counter, [1] blocks done, [2] a bounded wait gave up
-  // two-step passes (lbm_batch_set_twostep): the rolling kernel's items and
-  // grid, the frame launches' items (step n + 1 on the width-3 frames, step
-  // n + 2 on the width-2 frames) and the instances' frame buffers
+  // multi-step passes (lbm_batch_set_twostep): the frame tiles, the rolling
+  // items and the grid
   bool twostep = false, ts_dirty = true;
+  bool form_auto = true;  // no launch form was asked for: passes where they serve the batch
   int4* d_roll = nullptr;
-  int4* d_frame1 = nullptr;
-  int4* d_frame2 = nullptr;
-  void* d_frame = nullptr;
-  int n_roll = 0, n_frame1 = 0, n_frame2 = 0, roll_grid = 0;
+  int4* d_tiles = nullptr;
+  int n_roll = 0, n_tiles = 0, roll_grid = 0;
   bool items_dirty = true;
   std::vector<char> initialised;
   int cur = 0;
@@ -233,22 +232,16 @@ __global__ void __launch_bounds__(BX) batch_step_kernel(const T* __restrict__ A,
 // next tile is in flight while the current one is collided, so the bytes in
 // flight are bounded by shared memory, not by registers.
 // ---------------------------------------------------------------------------
-// A wait on a barrier nothing ever arrives on, then a wait on a counter
-// nothing ever increments (the two-step pass's wait for its first-frame
-// chunks): each must give up after its budget; *flag = 1 if both did (the
-// kernel then returns normally), 2 otherwise.
-__global__ void wait_selftest_kernel(long long budget, int* flag, const int* counter) {
+// A wait on a barrier nothing ever arrives on must give up after its budget;
+// *flag = 1 if it did (the kernel then returns normally), 2 otherwise.
+__global__ void wait_selftest_kernel(long long budget, int* flag) {
   __shared__ __align__(8) uint64_t bar;
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const bool a = mbar_wait(&bar, 0u, budget);
-    const bool b = lbmk::wait_count(counter, 1, budget);
-    *flag = (!a && !b) ? 1 : 2;
-  }
+  if (threadIdx.x == 0) *flag = !mbar_wait(&bar, 0u, budget) ? 1 : 2;
 }
 
 // The whole step of every instance in ONE persistent launch: blocks take
@@ -610,19 +603,32 @@ int build_items(lbm_batch_t* b) {
   return LBM_OK;
 }
 
-// The two-step pass serves the batch: 16- or 32-bit storage, no periodic
+// The multi-step pass serves the batch: 16- or 32-bit storage, no periodic
 // axis, every instance 8 x 8 nodes or more.
-bool batch_twostep_ok(const lbm_batch_t* b) {
+bool batch_pass_ok(const lbm_batch_t* b) {
   if (b->storage == LBM_F64 || b->nsbc.periodic_x || b->nsbc.periodic_y) return false;
   for (const InstDev& d : b->inst)
-    if (d.nx < 8 || d.ny < 8) return false;
+    if (d.nx < 2 * lbmk::kPassSteps || d.ny < 2 * lbmk::kPassSteps) return false;
   return true;
 }
 
-// Work lists of the two-step pass, largest instance first: rolling items in
-// bands of at most 64 output rows, all strips of a band side by side;
-// frame items of 128 threads; each instance's frame buffer after the last.
-int build_twostep(lbm_batch_t* b) {
+// Whether the next steps are taken in passes: as asked for, else f32 batches
+// of kPassCells nodes or more (us a step, staged / pass: 0.34 M nodes 8.7 /
+// 9.1, 2.1 M 30 / 21, 3.9 M 53 / 37, 13.9 M 157 / 85; f16 13.9 M 95 / 104:
+// the 16-bit pass is bound by instructions, not by the traffic it saves).
+constexpr long long kPassCells = 1000000;
+bool batch_passes(const lbm_batch_t* b) {
+  const bool want = b->form_auto ? b->storage == LBM_F32 && b->cells >= kPassCells : b->twostep;
+  return want && batch_pass_ok(b);
+}
+
+// Work lists of the multi-step pass, largest instance first: rolling items in
+// bands of rows, all strips of a band side by side; frame tiles.  The items
+// cover the rows and columns of the shortest pass (two steps); the kernel
+// clips them.  Bands of half a warp's share of the rows, 16 to 64 of them
+// (us a step in f32, bands of 16 / 32 / 64: 2.1 M nodes 21 / 21 / 26, 3.7 M
+// 31 / 33 / 34, 10.4 M 72 / 65 / 67, 13.9 M 95 / 87 / 85).
+int build_passes(lbm_batch_t* b) {
   if (!b->ts_dirty) return LBM_OK;
   const int out = b->storage == LBM_F32 ? lbmk::Roll<float>::OUT : lbmk::Roll<__half>::OUT;
   std::vector<int> order(b->count);
@@ -630,41 +636,7 @@ int build_twostep(lbm_batch_t* b) {
   std::stable_sort(order.begin(), order.end(), [&](int i, int j) {
     return (long long)b->inst[i].nx * b->inst[i].ny > (long long)b->inst[j].nx * b->inst[j].ny;
   });
-  std::vector<int4> roll, f1, f2;
-  long long foff = 0;
-  for (int k : order) {
-    const InstDev& d = b->inst[k];
-    const int strips = (d.nx - 4 + out - 1) / out, iy = d.ny - 4;
-    // bands of at most 64 rows: more, smaller items balance the warps better
-    // (measured on the 256-instance batch, band caps 128 / 64 / 32 / 16:
-    // f32 115k / 123k / 124k / 122k MLUPS, f16 144k / 149k / 149k / 144k)
-    const int nb = (iy + 63) / 64, band = (iy + nb - 1) / nb;
-    for (int y = 2; y < d.ny - 2; y += band)
-      for (int j = 0; j < strips; ++j) roll.push_back(make_int4(k, j * out, y, std::min(y + band, d.ny - 2)));
-    if (foff > INT32_MAX - 9LL * lbmk::ring_offset(d.nx, d.ny, lbmk::kFrameWidth))
-      return bfail(LBM_EINVAL, "lbm_batch: frame buffers beyond 2^31 elements");
-    for (int t0 = 0; t0 < lbmk::frame_threads(d.nx, d.ny, lbmk::kFrameWidth); t0 += 128)
-      f1.push_back(make_int4(k, t0, (int)foff, 0));
-    for (int t0 = 0; t0 < lbmk::frame_threads(d.nx, d.ny, 2); t0 += 128) f2.push_back(make_int4(k, t0, (int)foff, 0));
-    foff += 9LL * lbmk::ring_offset(d.nx, d.ny, lbmk::kFrameWidth);
-  }
-  for (int4** p : {&b->d_roll, &b->d_frame1, &b->d_frame2}) {
-    cudaFree(*p);
-    *p = nullptr;
-  }
-  cudaFree(b->d_frame);
-  b->d_frame = nullptr;
-  BATCH_CUDA(cudaMalloc(&b->d_frame, (size_t)foff * b->elt));
-  BATCH_CUDA(cudaMalloc(&b->d_roll, roll.size() * sizeof(int4)));
-  BATCH_CUDA(cudaMalloc(&b->d_frame1, f1.size() * sizeof(int4)));
-  BATCH_CUDA(cudaMalloc(&b->d_frame2, f2.size() * sizeof(int4)));
-  BATCH_CUDA(cudaMemcpy(b->d_roll, roll.data(), roll.size() * sizeof(int4), cudaMemcpyHostToDevice));
-  BATCH_CUDA(cudaMemcpy(b->d_frame1, f1.data(), f1.size() * sizeof(int4), cudaMemcpyHostToDevice));
-  BATCH_CUDA(cudaMemcpy(b->d_frame2, f2.data(), f2.size() * sizeof(int4), cudaMemcpyHostToDevice));
-  b->n_roll = (int)roll.size();
-  b->n_frame1 = (int)f1.size();
-  b->n_frame2 = (int)f2.size();
-  // the rolling kernel's shared memory, and one resident wave of its blocks
+  // the kernel's shared memory, and one resident wave of its blocks
   int per_sm = 0, sms = 0;
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
   bdispatch(b->storage, [&](auto tag) {
@@ -672,58 +644,63 @@ int build_twostep(lbm_batch_t* b) {
     if constexpr (!std::is_same<T, double>::value) {
       const int smem = (int)lbmk::Roll<T>::kSmem;
       for (const void* k :
-           {(const void*)lbmk::roll_batch_kernel<T, 0, false>, (const void*)lbmk::roll_batch_kernel<T, 0, true>,
-            (const void*)lbmk::roll_batch_kernel<T, 1, false>, (const void*)lbmk::roll_batch_kernel<T, 1, true>})
+           {(const void*)lbmk::pass_batch_kernel<T, 0, false>, (const void*)lbmk::pass_batch_kernel<T, 0, true>,
+            (const void*)lbmk::pass_batch_kernel<T, 1, false>, (const void*)lbmk::pass_batch_kernel<T, 1, true>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
       if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbmk::roll_batch_kernel<T, 1, true>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbmk::pass_batch_kernel<T, 1, true>,
                                                           lbmk::kRollThreads, smem);
     }
   });
-  if (e != cudaSuccess) return bfail(LBM_ECUDA, "lbm_batch: two-step kernel setup: %s", cudaGetErrorString(e));
-  if (per_sm <= 0) return bfail(LBM_ECUDA, "lbm_batch: no two-step block fits on an SM");
+  if (e != cudaSuccess) return bfail(LBM_ECUDA, "lbm_batch: multi-step kernel setup: %s", cudaGetErrorString(e));
+  if (per_sm <= 0) return bfail(LBM_ECUDA, "lbm_batch: no multi-step block fits on an SM");
   const int warps = lbmk::Roll<float>::WARPS;
-  b->roll_grid = std::max(1, std::min(per_sm * sms, (b->n_roll + warps - 1) / warps));
+  long long rows = 0;
+  for (const InstDev& d : b->inst) rows += (long long)((d.nx - 4 + out - 1) / out) * (d.ny - 4);
+  int max_band = (int)std::min<long long>(64, std::max<long long>(16, rows / (2LL * warps * per_sm * sms)));
+  std::vector<int4> roll, tiles;
+  for (int k : order) {
+    const InstDev& d = b->inst[k];
+    const int strips = (d.nx - 4 + out - 1) / out, iy = d.ny - 4;
+    const int nb = (iy + max_band - 1) / max_band, band = (iy + nb - 1) / nb;
+    for (int y = 2; y < d.ny - 2; y += band)
+      for (int j = 0; j < strips; ++j) roll.push_back(make_int4(k, j * out, y, std::min(y + band, d.ny - 2)));
+    for (int t = 0; t < lbmk::frame_tiles(d.nx, d.ny); ++t) tiles.push_back(make_int4(k, t, 0, 0));
+  }
+  for (int4** p : {&b->d_roll, &b->d_tiles}) {
+    cudaFree(*p);
+    *p = nullptr;
+  }
+  BATCH_CUDA(cudaMalloc(&b->d_roll, roll.size() * sizeof(int4)));
+  BATCH_CUDA(cudaMalloc(&b->d_tiles, tiles.size() * sizeof(int4)));
+  BATCH_CUDA(cudaMemcpy(b->d_roll, roll.data(), roll.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  BATCH_CUDA(cudaMemcpy(b->d_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  b->n_roll = (int)roll.size();
+  b->n_tiles = (int)tiles.size();
+  b->roll_grid = std::max(1, std::min(per_sm * sms, std::max((b->n_roll + warps - 1) / warps, b->n_tiles)));
   b->ts_dirty = false;
   return LBM_OK;
 }
 
-// Two steps from pool `from` to 1 - from: three launches.
-void enqueue_batch_twostep(const lbm_batch_t* b, int from, cudaStream_t s) {
+// `steps` (2 .. kPassSteps) steps from pool `from` to 1 - from: one launch.
+void enqueue_batch_pass(const lbm_batch_t* b, int from, int steps, cudaStream_t s) {
   bdispatch(b->storage, [&](auto tag) {
     using T = decltype(tag);
     if constexpr (!std::is_same<T, double>::value) {
-      using C = typename lbmk::Store<T>::C;
       const T* A = static_cast<const T*>(b->pool[from]);
       T* B = static_cast<T*>(b->pool[1 - from]);
-      T* F = static_cast<T*>(b->d_frame);
-      const auto* zs = static_cast<const lbmk::Shift<C>*>(b->d_shift);
+      const auto* zs = static_cast<const lbmk::Shift<typename lbmk::Store<T>::C>*>(b->d_shift);
       with_shift(b->shift, [&](auto zc) {
         constexpr bool Z = decltype(zc)::value;
-        // the frame launches on the side stream, beside the rolling kernel
-        // (whose warps claim items, so blocks that start late take fewer)
-        cudaStream_t fs = b->side ? b->side : s;
-        auto go = [&](auto mc) {
-          constexpr int M = decltype(mc)::value;
-          if (fs != s) {
-            cudaEventRecord(b->ev_fork, s);
-            cudaStreamWaitEvent(fs, b->ev_fork, 0);
-          }
-          lbmk::frame_batch_kernel<T, M, Z, true><<<b->n_frame1, 128, 0, fs>>>(A, B, F, b->d_inst, zs, b->d_frame1,
-                                                                               b->nsbc, b->s_e, b->s_eps, b->s_q);
-          lbmk::roll_batch_kernel<T, M, Z><<<b->roll_grid, lbmk::kRollThreads, lbmk::Roll<T>::kSmem, s>>>(
-              A, B, b->d_inst, zs, b->d_roll, b->n_roll, b->s_e, b->s_eps, b->s_q, b->d_err);
-          lbmk::frame_batch_kernel<T, M, Z, false><<<b->n_frame2, 128, 0, fs>>>(A, B, F, b->d_inst, zs, b->d_frame2,
-                                                                                b->nsbc, b->s_e, b->s_eps, b->s_q);
-          if (fs != s) {
-            cudaEventRecord(b->ev_join, fs);
-            cudaStreamWaitEvent(s, b->ev_join, 0);
-          }
+        auto go = [&](auto kernel) {
+          kernel<<<b->roll_grid, lbmk::kRollThreads, lbmk::Roll<T>::kSmem, s>>>(
+              A, B, b->d_inst, zs, b->d_tiles, b->n_tiles, b->d_roll, b->n_roll, steps, b->nsbc, b->s_e, b->s_eps,
+              b->s_q, b->d_err);
         };
         if (b->collision == 1)
-          go(std::integral_constant<int, 1>{});
+          go(lbmk::pass_batch_kernel<T, 1, Z>);
         else
-          go(std::integral_constant<int, 0>{});
+          go(lbmk::pass_batch_kernel<T, 0, Z>);
       });
     }
   });
@@ -813,11 +790,7 @@ lbm_batch_t* lbm_batch_create(int32_t count, const lbm_instance_desc* descs, int
   b->count = count;
   b->storage = storage;
   b->elt = storage == LBM_F64 ? 8 : (storage == LBM_F32 ? 4 : 2);
-  b->nsbc.gamma = 0.6;
-  b->nsbc.beta = 0.0;
-  b->nsbc.kappa = 3.0;
-  b->nsbc.order = 1;
-  b->nsbc.corner = 0;
+  b->nsbc.set(0.6, 0.0, 3.0, 0, 1);
   long long off = 0;
   for (int k = 0; k < count; ++k) {
     const lbm_instance_desc& s = descs[k];
@@ -870,9 +843,7 @@ void lbm_batch_destroy(lbm_batch_t* b) {
   cudaFree(b->d_items);
   cudaFree(b->d_err);
   cudaFree(b->d_roll);
-  cudaFree(b->d_frame1);
-  cudaFree(b->d_frame2);
-  cudaFree(b->d_frame);
+  cudaFree(b->d_tiles);
   if (b->cap) cudaStreamDestroy(b->cap);
   if (b->side) cudaStreamDestroy(b->side);
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
@@ -925,11 +896,7 @@ int lbm_batch_set_nsbc(lbm_batch_t* b, double gamma, double beta, double kappa, 
       (corner_mode != LBM_CORNER_DIAGONAL && corner_mode != LBM_CORNER_MEAN))
     return bfail(LBM_EINVAL,
                  "lbm_batch_set_nsbc: need finite gamma, beta, kappa, corner_mode 0 or 1 and grad_order 1 or 2");
-  b->nsbc.gamma = gamma;
-  b->nsbc.beta = beta;
-  b->nsbc.kappa = kappa;
-  b->nsbc.order = grad_order;
-  b->nsbc.corner = corner_mode;
+  b->nsbc.set(gamma, beta, kappa, corner_mode, grad_order);
   drop_batch_graphs(b);
   return LBM_OK;
 }
@@ -1006,9 +973,9 @@ int lbm_batch_step(lbm_batch_t* b, int32_t n) {
   if (rc) return rc;
   rc = ensure_batch_streams(b);
   if (rc) return rc;
-  const bool two = b->twostep && batch_twostep_ok(b);
-  if (two) {
-    rc = build_twostep(b);
+  const bool passes = batch_passes(b);
+  if (passes) {
+    rc = build_passes(b);
     if (rc) return rc;
   }
   int left = n;
@@ -1016,8 +983,9 @@ int lbm_batch_step(lbm_batch_t* b, int32_t n) {
     if (!b->graph[b->cur]) {
       cudaGraph_t g = nullptr;
       BATCH_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-      if (two)  // kBatchGraphSteps / 2 passes: an even number of pool swaps
-        for (int s = 0; s < kBatchGraphSteps / 2; ++s) enqueue_batch_twostep(b, (b->cur + s) & 1, b->cap);
+      if (passes)  // an even number of pool swaps
+        for (int s = 0; s < kBatchGraphSteps / lbmk::kPassSteps; ++s)
+          enqueue_batch_pass(b, (b->cur + s) & 1, lbmk::kPassSteps, b->cap);
       else
         for (int s = 0; s < kBatchGraphSteps; ++s) enqueue_batch_step(b, (b->cur + s) & 1, b->cap);
       cudaError_t e = cudaStreamEndCapture(b->cap, &g);
@@ -1031,9 +999,12 @@ int lbm_batch_step(lbm_batch_t* b, int32_t n) {
       left -= kBatchGraphSteps;
     }
   }
-  for (; two && left >= 2; left -= 2) {
-    enqueue_batch_twostep(b, b->cur, b->stream);
+  while (passes && left >= 2) {
+    int take = std::min(lbmk::kPassSteps, left);
+    if (left - take == 1 && take > 2) --take;  // five are three and two: a pass takes two steps at least
+    enqueue_batch_pass(b, b->cur, take, b->stream);
     b->cur ^= 1;
+    left -= take;
   }
   for (; left > 0; --left) {
     enqueue_batch_step(b, b->cur, b->stream);
@@ -1119,6 +1090,7 @@ int lbm_batch_set_launch(lbm_batch_t* b, int32_t threads_x, int32_t rows, int32_
   b->split = tma_tile == 0 && split != 0;
   b->tile = tma_tile;
   b->twostep = false;
+  b->form_auto = false;
   b->items_dirty = true;
   drop_batch_graphs(b);
   return LBM_OK;
@@ -1126,10 +1098,11 @@ int lbm_batch_set_launch(lbm_batch_t* b, int32_t threads_x, int32_t rows, int32_
 
 int lbm_batch_set_twostep(lbm_batch_t* b, int32_t enable) {
   if (!b) return bfail(LBM_EINVAL, "lbm_batch_set_twostep: NULL handle");
-  if (enable && !batch_twostep_ok(b))
+  if (enable && !batch_pass_ok(b))
     return bfail(LBM_EINVAL, "lbm_batch_set_twostep: needs f32, f16 or bf16 storage, no periodic axis and every "
                              "instance 8 x 8 nodes or more");
   b->twostep = enable != 0;
+  b->form_auto = false;
   drop_batch_graphs(b);
   return LBM_OK;
 }
@@ -1183,6 +1156,7 @@ int lbm_batch_autotune(lbm_batch_t* b, int32_t* threads_x, int32_t* rows, int32_
   int bb = b->bx, br = b->rows, bk = b->blocks, bp = b->pf, bt = b->tile;
   bool bs = b->split, bts = false;
   b->twostep = false;
+  b->form_auto = false;
   int rc = LBM_OK;
   auto time_it = [&]() -> float {
     for (int s = 0; s < 2; ++s) enqueue_batch_step(b, s & 1, b->stream);
@@ -1255,19 +1229,19 @@ int lbm_batch_autotune(lbm_batch_t* b, int32_t* threads_x, int32_t* rows, int32_
       if (rc) break;
       keep(time_it());
     }
-  // two-step passes (their odd steps, if any, take the best single step)
-  if (!rc && batch_twostep_ok(b)) {
-    rc = build_twostep(b);
+  // multi-step passes (a lone odd step, if any, takes the best single step)
+  if (!rc && batch_pass_ok(b)) {
+    rc = build_passes(b);
     if (!rc) {
-      for (int s = 0; s < 2; ++s) enqueue_batch_twostep(b, s & 1, b->stream);
+      for (int s = 0; s < 2; ++s) enqueue_batch_pass(b, s & 1, lbmk::kPassSteps, b->stream);
       cudaEventRecord(e0, b->stream);
-      const int passes = std::max(2, reps / 2);
-      for (int s = 0; s < passes; ++s) enqueue_batch_twostep(b, s & 1, b->stream);
+      const int passes = std::max(2, reps / lbmk::kPassSteps);
+      for (int s = 0; s < passes; ++s) enqueue_batch_pass(b, s & 1, lbmk::kPassSteps, b->stream);
       cudaEventRecord(e1, b->stream);
       float ms = 1e30f;
       if (cudaEventSynchronize(e1) == cudaSuccess) {
         cudaEventElapsedTime(&ms, e0, e1);
-        ms /= 2.0f * passes;
+        ms /= (float)(lbmk::kPassSteps * passes);
       }
       if (ms < best) {
         best = ms;
@@ -1335,12 +1309,12 @@ int lbm_partition_instances(int32_t count, const int64_t* cells, int32_t ranks, 
 int lbm_wait_selftest(int64_t budget_cycles) {
   if (budget_cycles <= 0 || budget_cycles > 4000000000LL)
     return bfail(LBM_EINVAL, "lbm_wait_selftest: budget %lld outside (0, 4e9] cycles", (long long)budget_cycles);
-  int* d = nullptr;  // [0] the flag, [1] a counter that stays 0
-  BATCH_CUDA(cudaMalloc(&d, 2 * sizeof(int)));
-  cudaError_t e = cudaMemset(d, 0, 2 * sizeof(int));
+  int* d = nullptr;
+  BATCH_CUDA(cudaMalloc(&d, sizeof(int)));
+  cudaError_t e = cudaMemset(d, 0, sizeof(int));
   int h = 0;
   if (e == cudaSuccess) {
-    wait_selftest_kernel<<<1, 32>>>(budget_cycles, d, d + 1);
+    wait_selftest_kernel<<<1, 32>>>(budget_cycles, d);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpy(&h, d, sizeof h, cudaMemcpyDeviceToHost);

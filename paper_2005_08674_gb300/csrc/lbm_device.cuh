@@ -407,10 +407,10 @@ __device__ __forceinline__ float2 v_add(float2 a, float2 b) { return __fadd2_rn(
 __device__ __forceinline__ float v_neg(float a) { return -a; }
 __device__ __forceinline__ double v_neg(double a) { return -a; }
 __device__ __forceinline__ float2 v_neg(float2 a) { return make_float2(-a.x, -a.y); }
-// a - b rounded once; on two nodes as b * (-1) + a, which rounds alike
+// a - b rounded once (negating a paired operand costs no instruction)
 __device__ __forceinline__ float v_sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ double v_sub(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ float2 v_sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 v_sub(float2 a, float2 b) { return v_add(a, v_neg(b)); }
 __device__ __forceinline__ float v_mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double v_mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float2 v_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
@@ -442,6 +442,13 @@ __device__ __forceinline__ double v_rcp(double a) {
   const double e = __fma_rn(-a, r, 1.0);
   return __fma_rn(r, __fma_rn(e, e, e), r);
 }
+// 1 / a to the last bit but for rare ties (one Newton step in float; the
+// iteration above in double)
+__device__ __forceinline__ float rcp_full(float a) {
+  const float r = v_rcp(a);
+  return __fmaf_rn(r, __fmaf_rn(-a, r, 1.f), r);
+}
+__device__ __forceinline__ double rcp_full(double a) { return v_rcp(a); }
 __device__ __forceinline__ float2 v_rcp(float2 a) { return make_float2(v_rcp(a.x), v_rcp(a.y)); }
 
 // ---------------------------------------------------------------------------
@@ -478,11 +485,12 @@ struct CellSums {
   V m, p;            // t5 - t7, t5 + t7
   V sa, sd;          // s1 + s3, s5 + s7
   V d, jx, jy;       // moments
-  V a, b, c, q;      // Pi_xx, Pi_yy, Pi_xy, trace
+  V Jx, Jy, wy;      // J, u_y: Pi_xy = J_x u_y + u0_x (J_y + d u0_y)
+  V a, b, q, r;      // Pi_xx, Pi_yy, a + b, a - b
 };
 
 template <bool SHIFT, typename V, typename C>
-__device__ __forceinline__ void cell_sums(const V (&h)[9], const Shift<C>& z, C s, CellSums<V>& o) {
+__device__ __forceinline__ void cell_sums(const V (&h)[9], const Shift<C>& z, C s, V vs, CellSums<V>& o) {
   o.s1 = v_add(h[1], h[2]);
   o.t1 = v_sub(h[1], h[2]);
   o.s3 = v_add(h[3], h[4]);
@@ -497,26 +505,101 @@ __device__ __forceinline__ void cell_sums(const V (&h)[9], const Shift<C>& z, C 
   o.d = v_add(v_add(o.sa, o.sd), h[0]);
   o.jx = v_add(o.t1, o.m);
   o.jy = v_add(o.t3, o.p);
+  // No sum takes a product here: a paired sum of a paired product may be
+  // contracted by the compiler, and would then round differently from the
+  // scalar form.
   if constexpr (SHIFT) {
     const C ux = z.u0[0], uy = z.u0[1];
     const V inv = v_rcp(v_add(v_splat<V>(mul_rn(s, z.rho0)), o.d));
-    const V Jx = v_fma(v_splat<V>(-ux), o.d, o.jx), Jy = v_fma(v_splat<V>(-uy), o.d, o.jy);
-    const V vx = v_mul(Jx, inv), vy = v_mul(Jy, inv);
-    // s = 2 u0 + v and u0 + v as multiply-adds: a paired addition that takes a
-    // paired product may be fused with it, and would then round differently
-    const V one = v_splat<V>(C(1)), two = v_splat<V>(C(2)), u = v_splat<V>(ux), w = v_splat<V>(uy);
-    const V sx = v_fma(two, u, vx), sy = v_fma(two, w, vy);
-    o.a = v_fma(o.d, v_splat<V>(mul_rn(ux, ux)), v_mul(Jx, sx));
-    o.b = v_fma(o.d, v_splat<V>(mul_rn(uy, uy)), v_mul(Jy, sy));
-    o.c = v_fma(u, Jy, v_fma(o.d, v_splat<V>(mul_rn(ux, uy)), v_mul(Jx, v_fma(one, w, vy))));
+    const V u = v_splat<V>(ux), w = v_splat<V>(uy), one = v_splat<V>(C(1)), two = v_splat<V>(C(2));
+    const V uyy = v_splat<V>(mul_rn(uy, uy)), uxx = v_splat<V>(mul_rn(ux, ux));
+    o.Jx = v_fma(v_neg(u), o.d, o.jx);
+    o.Jy = v_fma(v_neg(w), o.d, o.jy);
+    const V vx = v_mul(o.Jx, inv), vy = v_mul(o.Jy, inv);
+    const V sx = v_fma(two, u, vx), sy = v_fma(two, w, vy);  // s = 2 u0 + v
+    o.wy = v_fma(one, w, vy);
+    o.a = v_fma(o.d, uxx, v_mul(o.Jx, sx));
+    o.b = v_fma(o.d, uyy, v_mul(o.Jy, sy));
+    o.q = v_fma(o.Jx, sx, v_fma(o.d, uxx, o.b));
+    o.r = v_fma(v_neg(o.Jy), sy, v_fma(v_neg(o.d), uyy, o.a));
   } else {
-    const V inv = v_rcp(v_add(v_splat<V>(s), o.d));
-    const V vx = v_mul(o.jx, inv), vy = v_mul(o.jy, inv);
+    const V inv = v_rcp(v_add(vs, o.d));
+    const V vx = v_mul(o.jx, inv);
+    o.Jx = o.jx;
+    o.Jy = o.jy;
+    o.wy = v_mul(o.jy, inv);
     o.a = v_mul(o.jx, vx);
-    o.b = v_mul(o.jy, vy);
-    o.c = v_mul(o.jx, vy);
+    o.b = v_mul(o.jy, o.wy);
+    o.q = v_fma(o.jx, vx, o.b);
+    o.r = v_fma(v_neg(o.jy), o.wy, o.a);
   }
-  o.q = v_add(o.a, o.b);
+}
+
+// Pi_xy, and x - Pi_xy
+template <bool SHIFT, typename V, typename C>
+__device__ __forceinline__ V pi_xy(const CellSums<V>& n, const Shift<C>& z) {
+  V c = v_mul(n.Jx, n.wy);
+  if constexpr (SHIFT)
+    c = v_fma(v_splat<V>(z.u0[0]), n.Jy, v_fma(v_splat<V>(mul_rn(z.u0[0], z.u0[1])), n.d, c));
+  return c;
+}
+template <bool SHIFT, typename V, typename C>
+__device__ __forceinline__ V less_pi_xy(const CellSums<V>& n, const Shift<C>& z, V x) {
+  if constexpr (SHIFT) {
+    x = v_fma(v_splat<V>(-z.u0[0]), n.Jy, x);
+    x = v_fma(v_splat<V>(-mul_rn(z.u0[0], z.u0[1])), n.d, x);
+  }
+  return v_fma(v_neg(n.Jx), n.wy, x);
+}
+
+// The constants of the collision of two nodes or one, formed once per kernel.
+// PIN (pairs): the compiler would rather rebuild a pair of equal constants
+// before each use than keep its two registers; an empty asm it cannot see
+// through keeps them.
+template <typename V, bool PIN>
+__device__ __forceinline__ V v_const(typename std::conditional<std::is_same<V, double>::value, double, float>::type c) {
+  V v = v_splat<V>(c);
+  if constexpr (PIN && std::is_same<V, float2>::value) {
+    unsigned long long u;
+    memcpy(&u, &v, 8);
+    asm volatile("" : "+l"(u));
+    memcpy(&v, &u, 8);
+  }
+  return v;
+}
+
+template <typename V>
+struct CellConst {
+  V s, two, half;                     // storage scale, 2, 1/2
+  V k2, wa, wa15, wa45, wd, wd3, wd6, wd9;  // BGK
+  V three, four, ke, kep, kq, kw;     // MRT
+};
+
+template <int MODEL, bool PIN, typename V, typename C>
+__device__ __forceinline__ CellConst<V> cell_const(const Rates<C>& r, C s) {
+  CellConst<V> k;
+  k.s = v_const<V, PIN>(s);
+  k.two = v_const<V, PIN>(C(2));
+  if constexpr (MODEL == 1) {
+    k.three = v_const<V, PIN>(C(3));
+    k.four = v_const<V, PIN>(C(4));
+    k.ke = v_const<V, PIN>(mul_rn(r.s_e, C(1.0 / 36.0)));
+    k.kep = v_const<V, PIN>(mul_rn(r.s_eps, C(1.0 / 12.0)));
+    k.kq = v_const<V, PIN>(mul_rn(r.s_q, C(1.0 / 12.0)));
+    k.kw = v_const<V, PIN>(mul_rn(r.omega, C(0.25)));
+  } else {
+    const C wa = mul_rn(r.omega, wt<C>(1)), wd = mul_rn(C(0.25), wa);
+    k.half = v_const<V, PIN>(C(0.5));
+    k.k2 = v_const<V, PIN>(mul_rn(C(0.5), sub_rn(C(1), r.omega)));
+    k.wa = v_const<V, PIN>(wa);
+    k.wa15 = v_const<V, PIN>(mul_rn(C(1.5), wa));
+    k.wa45 = v_const<V, PIN>(mul_rn(C(4.5), wa));
+    k.wd = v_const<V, PIN>(wd);
+    k.wd3 = v_const<V, PIN>(mul_rn(C(3), wd));
+    k.wd6 = v_const<V, PIN>(mul_rn(C(6), wd));
+    k.wd9 = v_const<V, PIN>(mul_rn(C(9), wd));
+  }
+  return k;
 }
 
 // BGK collision, Eq. (lbe_1) with dt = 1, on shifted populations held as
@@ -530,33 +613,28 @@ __device__ __forceinline__ void cell_sums(const V (&h)[9], const Shift<C>& z, C 
 // rounded weights do not add up to omega), which after 100 steps was the
 // whole f32 error.
 template <bool SHIFT, typename V, typename C>
-__device__ __forceinline__ void collide_bgk(V (&h)[9], const Rates<C>& r, C s = C(1)) {
+__device__ __forceinline__ void collide_bgk(V (&h)[9], const Rates<C>& r, C s, const CellConst<V>& k) {
   CellSums<V> n;
-  cell_sums<SHIFT>(h, r.z, s, n);
-  const C omega = r.omega, k2c = mul_rn(C(0.5), sub_rn(C(1), omega));
-  const C wa = mul_rn(omega, wt<C>(1)), wd = mul_rn(C(0.25), wa);
-  const V k2 = v_splat<V>(k2c);
-  const V ba = v_fma(v_splat<V>(mul_rn(C(-1.5), wa)), n.q, v_mul(v_splat<V>(wa), n.d));
-  const V bd = v_fma(v_splat<V>(mul_rn(C(3), wd)), n.q, v_mul(v_splat<V>(wd), n.d));
-  const V wa45 = v_splat<V>(mul_rn(C(4.5), wa));
-  const V S1 = v_fma(k2, n.s1, v_fma(wa45, n.a, ba));
-  const V S3 = v_fma(k2, n.s3, v_fma(wa45, n.b, ba));
-  const V S5 = v_fma(k2, n.s5, v_fma(v_splat<V>(mul_rn(C(9), wd)), n.c, bd));
-  const V S7 = v_fma(k2, n.s7, v_fma(v_splat<V>(mul_rn(C(-9), wd)), n.c, bd));
-  const V wd6 = v_splat<V>(mul_rn(C(6), wd));
-  const V X = v_fma(k2, n.m, v_mul(wd6, n.jx)), Y = v_fma(k2, n.p, v_mul(wd6, n.jy));
-  const V half = v_splat<V>(C(0.5)), mhalf = v_splat<V>(C(-0.5));
-  const V T1 = v_fma(half, n.jx, v_neg(X)), T3 = v_fma(half, n.jy, v_neg(Y));
+  cell_sums<SHIFT>(h, r.z, s, k.s, n);
+  const V ba = v_fma(v_neg(k.wa15), n.q, v_mul(k.wa, n.d));
+  const V bd = v_fma(k.wd3, n.q, v_mul(k.wd, n.d));
+  const V c = pi_xy<SHIFT>(n, r.z);
+  const V S1 = v_fma(k.k2, n.s1, v_fma(k.wa45, n.a, ba));
+  const V S3 = v_fma(k.k2, n.s3, v_fma(k.wa45, n.b, ba));
+  const V S5 = v_fma(k.k2, n.s5, v_fma(k.wd9, c, bd));
+  const V S7 = v_fma(k.k2, n.s7, v_fma(v_neg(k.wd9), c, bd));
+  const V X = v_fma(k.k2, n.m, v_mul(k.wd6, n.jx)), Y = v_fma(k.k2, n.p, v_mul(k.wd6, n.jy));
+  const V T1 = v_fma(k.half, n.jx, v_neg(X)), T3 = v_fma(k.half, n.jy, v_neg(Y));
   const V U5 = v_add(X, Y), U7 = v_sub(Y, X);  // 2 T_5, 2 T_7
-  h[0] = v_fma(v_splat<V>(C(-2)), v_add(v_add(S1, S3), v_add(S5, S7)), n.d);
+  h[0] = v_fma(v_neg(k.two), v_add(v_add(S1, S3), v_add(S5, S7)), n.d);
   h[1] = v_add(S1, T1);
   h[2] = v_sub(S1, T1);
   h[3] = v_add(S3, T3);
   h[4] = v_sub(S3, T3);
-  h[5] = v_fma(half, U5, S5);
-  h[6] = v_fma(mhalf, U5, S5);
-  h[7] = v_fma(half, U7, S7);
-  h[8] = v_fma(mhalf, U7, S7);
+  h[5] = v_fma(k.half, U5, S5);
+  h[6] = v_fma(v_neg(k.half), U5, S5);
+  h[7] = v_fma(k.half, U7, S7);
+  h[8] = v_fma(v_neg(k.half), U7, S7);
 }
 
 // ---------------------------------------------------------------------------
@@ -579,26 +657,24 @@ __device__ __forceinline__ void collide_bgk(V (&h)[9], const Rates<C>& r, C s = 
 //   pxx : (s1 - s3) - (a - b)          pxy : (s5 - s7) - c
 // ---------------------------------------------------------------------------
 template <bool SHIFT, typename V, typename C>
-__device__ __forceinline__ void collide_mrt(V (&h)[9], const Rates<C>& r, C s = C(1)) {
+__device__ __forceinline__ void collide_mrt(V (&h)[9], const Rates<C>& r, C s, const CellConst<V>& k) {
   CellSums<V> n;
-  cell_sums<SHIFT>(h, r.z, s, n);
-  const V two = v_splat<V>(C(2)), mtwo = v_splat<V>(C(-2));
-  const V me = v_fma(v_splat<V>(C(-3)), n.q, v_fma(v_splat<V>(C(4)), n.sd, v_fma(mtwo, h[0], n.sa)));
+  cell_sums<SHIFT>(h, r.z, s, k.s, n);
+  const V two = k.two, mtwo = v_neg(k.two);
+  const V me = v_fma(v_neg(k.three), n.q, v_fma(k.four, n.sd, v_fma(mtwo, h[0], n.sa)));
   const V mep = v_add(v_sub(h[0], n.sa), n.q);  // a third of it
   const V mqx = v_fma(two, n.m, v_neg(n.t1)), mqy = v_fma(two, n.p, v_neg(n.t3));
-  const V mxx = v_sub(v_sub(n.s1, n.s3), v_sub(n.a, n.b));
-  const V mxy = v_sub(v_sub(n.s5, n.s7), n.c);
-  const V kw = v_splat<V>(mul_rn(r.omega, C(0.25))), kq = v_splat<V>(mul_rn(r.s_q, C(1.0 / 12.0)));
-  const V re = v_mul(v_splat<V>(mul_rn(r.s_e, C(1.0 / 36.0))), me);
-  const V rep = v_mul(v_splat<V>(mul_rn(r.s_eps, C(1.0 / 12.0))), mep);
-  const V rqx = v_mul(kq, mqx), rqy = v_mul(kq, mqy);
-  const V rxx = v_mul(kw, mxx), rxy = v_mul(kw, mxy);
+  const V mxx = v_sub(v_sub(n.s1, n.s3), n.r);
+  const V mxy = less_pi_xy<SHIFT>(n, r.z, v_sub(n.s5, n.s7));
+  const V re = v_mul(k.ke, me), rep = v_mul(k.kep, mep);
+  const V rqx = v_mul(k.kq, mqx), rqy = v_mul(k.kq, mqy);
+  const V rxx = v_mul(k.kw, mxx), rxy = v_mul(k.kw, mxy);
   const V a0 = v_fma(mtwo, rep, v_neg(re));  // e/eps part of the axis columns
   const V a1 = v_fma(two, re, rep);          // e/eps part of the diagonal columns
   const V ax = v_add(a0, rxx), ay = v_sub(a0, rxx);
   const V d5 = v_add(a1, rxy), d7 = v_sub(a1, rxy);
   const V q5 = v_add(rqx, rqy), q7 = v_sub(rqy, rqx);
-  h[0] = v_fma(v_splat<V>(C(-4)), v_sub(rep, re), h[0]);
+  h[0] = v_fma(v_neg(k.four), v_sub(rep, re), h[0]);
   h[1] = v_sub(h[1], v_fma(mtwo, rqx, ax));
   h[2] = v_sub(h[2], v_fma(two, rqx, ax));
   h[3] = v_sub(h[3], v_fma(mtwo, rqy, ay));
@@ -611,11 +687,15 @@ __device__ __forceinline__ void collide_mrt(V (&h)[9], const Rates<C>& r, C s = 
 
 // Collision model: 0 = BGK (Eq. lbe_1), 1 = MRT (Eq. mrt_lbe).
 template <int MODEL, bool SHIFT, typename V, typename C>
-__device__ __forceinline__ void collide(V (&h)[9], const Rates<C>& r, C s = C(1)) {
+__device__ __forceinline__ void collide(V (&h)[9], const Rates<C>& r, C s, const CellConst<V>& k) {
   if constexpr (MODEL == 1)
-    collide_mrt<SHIFT>(h, r, s);
+    collide_mrt<SHIFT>(h, r, s, k);
   else
-    collide_bgk<SHIFT>(h, r, s);
+    collide_bgk<SHIFT>(h, r, s, k);
+}
+template <int MODEL, bool SHIFT, typename V, typename C>
+__device__ __forceinline__ void collide(V (&h)[9], const Rates<C>& r, C s = C(1)) {
+  collide<MODEL, SHIFT>(h, r, s, cell_const<MODEL, false, V>(r, s));
 }
 
 // The collision of N nodes held as h[i][k] (population i of node k): with
@@ -660,6 +740,11 @@ struct Geom {
   long long plane;  // elements between population planes
 };
 
+// A number as the unevaluated sum of two floats (48 bits together).
+struct FloatPair {
+  float h, l;
+};
+
 struct Nsbc {
   double gamma, beta, kappa;
   double m0[3];  // far-field (rho, ux, uy)
@@ -668,6 +753,27 @@ struct Nsbc {
   int periodic_x, periodic_y;  // axes closed periodically instead of by NSBC edges
   int vel[4];                  // edges (left, right, bottom, top) with a prescribed velocity
   double uw[4][2];             // that velocity
+  // the same settings as the float kernels use them (set())
+  float kappa_f;
+  FloatPair step[2];  // gamma / |n| along an edge's normal and along a corner's diagonal, halved for order 2
+  FloatPair keep;     // 1 - beta
+
+  void set(double gamma_, double beta_, double kappa_, int corner_, int order_) {
+    gamma = gamma_;
+    beta = beta_;
+    kappa = kappa_;
+    corner = corner_;
+    order = order_;
+    auto pair = [](double v) {
+      const float h = (float)v;
+      return FloatPair{h, (float)(v - (double)h)};
+    };
+    const double g = order == 2 ? 0.5 * gamma : gamma;
+    kappa_f = (float)kappa;
+    step[0] = pair(g);
+    step[1] = pair(g * 0.70710678118654752);
+    keep = pair(1.0 - beta);
+  }
 };
 
 // Node k of the perimeter (k < 2 nx + 2 (ny - 2)) -> coordinates and outward
@@ -722,13 +828,13 @@ __device__ __forceinline__ void dmoments_of(const C (&h)[9], C rho0, C u0x, C u0
   moments(h, d, jx, jy);
   m[0] = d;
   if constexpr (SHIFT) {
-    const C inv = C(1) / (rho0 + d);
-    m[1] = fma_rn(-d, u0x, jx) * inv;
-    m[2] = fma_rn(-d, u0y, jy) * inv;
+    const C inv = rcp_full(rho0 + d);
+    m[1] = mul_rn(fma_rn(-d, u0x, jx), inv);
+    m[2] = mul_rn(fma_rn(-d, u0y, jy), inv);
   } else {
-    const C inv = C(1) / (C(1) + d);
-    m[1] = jx * inv;
-    m[2] = jy * inv;
+    const C inv = rcp_full(C(1) + d);
+    m[1] = mul_rn(jx, inv);
+    m[2] = mul_rn(jy, inv);
   }
 }
 

@@ -298,11 +298,11 @@ __device__ __forceinline__ void pair_collide(const QuadPair& pr, int q, C& hp, C
   pair_moments<SHIFT>(pr, hp, hm, h0, r.z, quad, d, sjx, sjy);
   C jx = sjx, jy = sjy, inv;
   if constexpr (SHIFT) {
-    inv = div_rho(C(1), r.z.rho0 + d);
+    inv = v_rcp(r.z.rho0 + d);
     jx = fma_rn(-d, r.z.u0[0], sjx);
     jy = fma_rn(-d, r.z.u0[1], sjy);
   } else {
-    inv = div_rho(C(1), C(1) + d);
+    inv = v_rcp(C(1) + d);
   }
   C ep, em, e0;
   if constexpr (MODEL == 1) {
@@ -338,28 +338,48 @@ __device__ __forceinline__ void pair_collide(const QuadPair& pr, int q, C& hp, C
 // Eq. (nes_2): m_p = m_b - gamma d_n m, d_n along the outward unit normal by
 // the one-sided difference of the given order (1 / |n| = 1/sqrt(2) along a
 // corner's diagonal); Eq. (nes_3): m_c = (1 - beta) m_p + beta m_0, which
-// for the deviation m - m_0 is (1 - beta) (m_p - m_0).  Component c of the
-// deviation (rho - rho0, u - u0) from its values at b, b - n, b - 2n, in FP64
-// with every rounding explicit (no contraction left to the compiler), so that
-// every caller gets the same bits.  GB300's FP64 divide is slow: no divides.
+// for the deviation m - m_0 is (1 - beta) (m_p - m_0).  One component of the
+// deviation (rho - rho0, u - u0) from its values at b, b - n, b - 2n, with
+// every rounding explicit (no contraction left to the compiler), so that
+// every caller gets the same bits.  f64 storage: in FP64.  Otherwise as pairs
+// of floats (exact differences and products by Knuth's and Dekker's error
+// terms, 48 bits): the chip's FP64 pipe takes one warp instruction in about
+// 15 cycles per SM, and eight of them per warp -- four conversions among
+// them -- were half of a boundary tile's step.
 // The settings Eqs. nes_2 and nes_3 use, and the far field in the compute
 // type: small values passed by value (also to the out-of-line corner pass,
 // where a reference would move the caller's structures to local memory).
-struct Predict {
+template <typename C>
+struct Predict;
+template <>
+struct Predict<double> {
   double gamma, beta;
+  int order;
+};
+template <>
+struct Predict<float> {
+  FloatPair step[2], keep;
   int order;
 };
 template <typename C>
 struct Far {
   C rho0, u0x, u0y;
 };
-__device__ __forceinline__ Predict predict_of(const Nsbc& p) { return Predict{p.gamma, p.beta, p.order}; }
+template <typename C>
+__device__ __forceinline__ Predict<C> predict_of(const Nsbc& p) {
+  if constexpr (std::is_same<C, double>::value)
+    return Predict<double>{p.gamma, p.beta, p.order};
+  else
+    return Predict<float>{{p.step[0], p.step[1]}, p.keep, p.order};
+}
 template <typename C>
 __device__ __forceinline__ Far<C> far_of(const Shift<C>& z) { return Far<C>{z.rho0, z.u0[0], z.u0[1]}; }
 
+// a prediction before its rounding to the compute type
 template <typename C>
-__device__ __forceinline__ double edge_predict(C vb, C v1, C v2, bool diagonal, Predict p) {
-  const double mb = (double)vb, m1 = (double)v1, m2 = (double)v2;
+using Predicted = typename std::conditional<std::is_same<C, double>::value, double, FloatPair>::type;
+
+__device__ __forceinline__ double edge_predict(double mb, double m1, double m2, bool diagonal, Predict<double> p) {
   const double inv_len = diagonal ? 0.70710678118654752 : 1.0;
   const double dn = p.order == 2 ? __dmul_rn(__fma_rn(3.0, mb, __fma_rn(-4.0, m1, m2)), 0.5 * inv_len)
                                  : __dmul_rn(__dsub_rn(mb, m1), inv_len);
@@ -367,13 +387,47 @@ __device__ __forceinline__ double edge_predict(C vb, C v1, C v2, bool diagonal, 
   return __dmul_rn(1.0 - p.beta, mp);
 }
 
+// a - b = s + e exactly (Knuth, TAOCP vol. 2, 4.2.2)
+__device__ __forceinline__ FloatPair exact_diff(float a, float b) {
+  const float s = __fsub_rn(a, b), t = __fsub_rn(s, a);
+  return FloatPair{s, __fsub_rn(__fsub_rn(a, __fsub_rn(s, t)), __fadd_rn(b, t))};
+}
+
+__device__ __forceinline__ FloatPair edge_predict(float mb, float m1, float m2, bool diagonal, Predict<float> p) {
+  FloatPair d = exact_diff(mb, m1);
+  if (p.order == 2) {  // 3 m_b - 4 m_1 + m_2 = 3 (m_b - m_1) - (m_1 - m_2)
+    const FloatPair e = exact_diff(m1, m2);
+    const float t = __fmul_rn(3.f, d.h);
+    const FloatPair q = exact_diff(t, e.h);
+    const float low = __fadd_rn(__fmaf_rn(3.f, d.h, -t), __fmaf_rn(3.f, d.l, -e.l));
+    d = FloatPair{q.h, __fadd_rn(q.l, low)};
+  }
+  const float gh = diagonal ? p.step[1].h : p.step[0].h, gl = diagonal ? p.step[1].l : p.step[0].l;
+  const float t = __fmul_rn(gh, d.h);
+  const float tl = __fmaf_rn(gl, d.h, __fmaf_rn(gh, d.l, __fmaf_rn(gh, d.h, -t)));
+  const FloatPair m = exact_diff(mb, t);
+  const float ml = __fsub_rn(m.l, tl);
+  const float r = __fmul_rn(p.keep.h, m.h);
+  return FloatPair{r, __fmaf_rn(p.keep.h, ml, __fmaf_rn(p.keep.l, m.h, __fmaf_rn(p.keep.h, m.h, -r)))};
+}
+
+__device__ __forceinline__ double predicted_mean(double a, double b) { return __dmul_rn(0.5, __dadd_rn(a, b)); }
+__device__ __forceinline__ FloatPair predicted_mean(FloatPair a, FloatPair b) {
+  const FloatPair s = exact_diff(a.h, -b.h);
+  return FloatPair{__fmul_rn(0.5f, s.h), __fmul_rn(0.5f, __fadd_rn(s.l, __fadd_rn(a.l, b.l)))};
+}
+__device__ __forceinline__ double predicted_value(double a) { return a; }
+__device__ __forceinline__ float predicted_value(FloatPair a) { return __fadd_rn(a.h, a.l); }
+
 // Lane q of a quad: the deviations (rho - rho0, u - u0) of node b - q n (zeros for
 // lanes beyond the difference order), transposed across the quad so that
 // lane c (c < 3) gets component c at b, b - n, b - 2n, predicted and blended
-// in FP64 by edge_predict.  All four lanes call this together.
+// by edge_predict.  All four lanes call this together.
 template <typename T, bool SHIFT>
-__device__ __forceinline__ double quad_predict(const typename Store<T>::C (&v)[9], Far<typename Store<T>::C> z,
-                                               unsigned quad, int cq, bool diagonal, Predict p) {
+__device__ __forceinline__ Predicted<typename Store<T>::C> quad_predict(const typename Store<T>::C (&v)[9],
+                                                                        Far<typename Store<T>::C> z, unsigned quad,
+                                                                        int cq, bool diagonal,
+                                                                        Predict<typename Store<T>::C> p) {
   using C = typename Store<T>::C;
   C mq[3];
   dmoments_of<SHIFT>(v, z.rho0, z.u0x, z.u0y, mq);  // lanes that loaded nothing get unused values
@@ -453,7 +507,8 @@ __device__ __forceinline__ void quad_finish(const Dst& B, const Geom& g, const N
       d_jx = fma_rn(-rho_c, mc[1], jx);
       d_jy = fma_rn(-rho_c, mc[2], jy);
     }
-    const C t = C(p.kappa) * (C(pr.cx) * d_jx + C(pr.cy) * d_jy);
+    const C kappa = std::is_same<C, double>::value ? C(p.kappa) : C(p.kappa_f);
+    const C t = kappa * (C(pr.cx) * d_jx + C(pr.cy) * d_jy);
     const C w = pr.diag ? wt<C>(5) : wt<C>(1);
     hp -= w * (d_rho + t);
     hm -= w * (d_rho - t);
@@ -472,8 +527,10 @@ __device__ __forceinline__ void quad_finish(const Dst& B, const Geom& g, const N
 // horizontal edge's normal (0, nyn).  Kept out of line: only the quads that
 // hold a corner call it, and inlined it would cost every NSBC node registers.
 template <typename T, bool SHIFT, typename Src>
-__device__ __noinline__ double corner_second_prediction(Src A, int x, int y, Far<typename Store<T>::C> z,
-                                                        unsigned quad, int q, Predict p) {
+__device__ __noinline__ Predicted<typename Store<T>::C> corner_second_prediction(Src A, int x, int y,
+                                                                                 Far<typename Store<T>::C> z,
+                                                                                 unsigned quad, int q,
+                                                                                 Predict<typename Store<T>::C> p) {
   typename Store<T>::C w[9];
   load_node<T>(A, x, y, q <= p.order, w);
   return quad_predict<T, SHIFT>(w, z, quad, q < 3 ? q : 0, false, p);
@@ -494,21 +551,18 @@ __device__ __noinline__ double corner_second_prediction(Src A, int x, int y, Far
 // and gets the mean of the two blended states; the second pass runs only in
 // the quads that hold a corner.
 template <typename T, int MODEL, int K, bool SHIFT = false, typename Src, typename Dst>
-__device__ __forceinline__ void nsbc_nodes(const Src& A, const Dst& B, const Geom& g, const Nsbc& p,
-                                           const Rates<typename Store<T>::C>& rates, const int (&node)[K],
-                                           const bool (&valid)[K], int q) {
+__device__ __forceinline__ void nsbc_edge_nodes(const Src& A, const Dst& B, const Geom& g, const Nsbc& p,
+                                                const Rates<typename Store<T>::C>& rates, const EdgeNode (&en)[K],
+                                                const bool (&valid)[K], int q) {
   using S = Store<T>;
   using C = typename S::C;
   const unsigned quad = 0xFu << ((threadIdx.x & 31) & ~3);
   const QuadPair pr = quad_pair(q);
-  EdgeNode en[K];
   C hp[K], hm[K], h0[K], v[K][9];
   bool kp[K], km[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    en[k] = edge_node(node[k], g, p);
+  for (int k = 0; k < K; ++k)
     quad_pull<T>(A, g, p, en[k], pr, hp[k], hm[k], h0[k], kp[k], km[k]);  // this lane's pulled pair
-  }
 #pragma unroll
   for (int k = 0; k < K; ++k) {  // lane q: the node b - q n (zeros if not needed)
     const bool split = p.corner == 1 && en[k].nxn != 0 && en[k].nyn != 0;
@@ -521,12 +575,11 @@ __device__ __forceinline__ void nsbc_nodes(const Src& A, const Dst& B, const Geo
   for (int k = 0; k < K; ++k) {
     const bool corner = en[k].nxn != 0 && en[k].nyn != 0;
     const bool split = p.corner == 1 && corner;  // the same for all four lanes of the quad
-    double mine = quad_predict<T, SHIFT>(v[k], far_of(rates.z), quad, cq, corner && !split, predict_of(p));
+    Predicted<C> mine = quad_predict<T, SHIFT>(v[k], far_of(rates.z), quad, cq, corner && !split, predict_of<C>(p));
     if (split)
-      mine = __dmul_rn(0.5, __dadd_rn(mine, corner_second_prediction<T, SHIFT>(A, en[k].x, en[k].y - q * en[k].nyn,
-                                                                              far_of(rates.z), quad, q,
-                                                                              predict_of(p))));
-    const C mcq = C(mine);
+      mine = predicted_mean(mine, corner_second_prediction<T, SHIFT>(A, en[k].x, en[k].y - q * en[k].nyn,
+                                                                    far_of(rates.z), quad, q, predict_of<C>(p)));
+    const C mcq = predicted_value(mine);
 #pragma unroll
     for (int c = 0; c < 3; ++c) mc[k][c] = __shfl_sync(quad, mcq, c, 4);
   }
@@ -534,6 +587,17 @@ __device__ __forceinline__ void nsbc_nodes(const Src& A, const Dst& B, const Geo
   for (int k = 0; k < K; ++k)
     quad_finish<T, MODEL, SHIFT>(B, g, p, rates, en[k], pr, q, quad, hp[k], hm[k], h0[k], kp[k], km[k], mc[k],
                                  valid[k]);
+}
+
+// The same for perimeter nodes given by their index (perimeter_node's order).
+template <typename T, int MODEL, int K, bool SHIFT = false, typename Src, typename Dst>
+__device__ __forceinline__ void nsbc_nodes(const Src& A, const Dst& B, const Geom& g, const Nsbc& p,
+                                           const Rates<typename Store<T>::C>& rates, const int (&node)[K],
+                                           const bool (&valid)[K], int q) {
+  EdgeNode en[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) en[k] = edge_node(node[k], g, p);
+  nsbc_edge_nodes<T, MODEL, K, SHIFT>(A, B, g, p, rates, en, valid, q);
 }
 
 template <typename T, int MODEL, bool SHIFT = false>

@@ -20,9 +20,9 @@
 #include "lbm.h"
 #include "lbm_aux.cuh"
 #include "lbm_kernels.cuh"
+#include "lbm_multistep.cuh"
 #include "lbm_staged.cuh"
 #include "lbm_trace.h"
-#include "lbm_twostep.cuh"
 #include "lbm_tune_cache.h"
 
 namespace lbmk {
@@ -85,6 +85,13 @@ constexpr int kGraphSteps = 16;  // steps per captured graph (even: buffers retu
 constexpr int kReduceThreads = 256;
 constexpr int kReduceBlocks = 1216;  // 8 x 152 SMs
 constexpr int kNsbcThreads = 128;
+// where pick_form() draws the lines
+constexpr long long kPassNodes32 = 1200000, kPassNodes16 = 2800000, kTileNodes = 110000, kFusedNodes = 800000;
+constexpr long long kTileCells = 1 << 21;  // largest domain the autotuner tries as tiles
+
+// How lbm_step launches steps: the bulk and NSBC kernel pair, both in one
+// launch, the staged kernel, the multi-step pass, or tiles.
+enum class Form { Pair, Fused, Staged, Pass, Tiles };
 
 // launch shapes compiled for the bulk kernel: threads per block along x
 constexpr int kShapesBX[] = {64, 128, 256, 512};
@@ -124,18 +131,22 @@ struct lbm {
   // fused step kernel (lbm_set_fused): the bulk grid of the current shape and
   // the NSBC quads in one launch per step
   bool fused = false;
-  // two-step pass (lbm_set_twostep): two steps per pass, the step in between
-  // kept on chip except on the frame of width 3 (in d_frame, fn nodes);
-  // the rolling kernel's strips, bands, rows per band, bands per wave,
-  // waves and persistent grid, and the device's SM count
+  // multi-step pass (lbm_set_twostep): several steps per launch, the steps in
+  // between kept on chip; the rolling items' strips, bands, rows per band,
+  // bands per wave, waves and persistent grid, and the device's SM count
   bool twostep = false;
   int ts_strips = 0, ts_bands = 0, ts_band = 0, ts_wave_bands = 0, ts_waves = 0, ts_grid = 0, sms = 0;
-  void* d_frame = nullptr;
-  int frame_fn = 0;
+  // tiles (small domains): several steps per launch of tile_kernel
+  bool tiles = false;
+  int tl_gx = 0, tl_gy = 0, tl_steps = 0, tl_smem = 0;
+  // no launch form was asked for: lbm_step takes the one pick_form() names
+  bool form_auto = true;
+  Form form = Form::Pair;  // what prepare_form() settled on
+  bool form_ready = false;
+  bool sched_clear = false;  // the counters have been zeroed
   int4* d_items = nullptr;
   lbmk::InstDev* d_inst = nullptr;
   void* d_shift = nullptr;  // the far field's storage shift in the compute type (staged kernel)
-  int* d_sched = nullptr;  // work counter, blocks done, give-up flag
   int n_items = 0, items_storage = -1, staged_grid = 0;
   // per-launch timing (lbm_profile): an event pair around every launch, and
   // which kernel it was (0 = bulk or staged step kernel, 1 = NSBC)
@@ -159,6 +170,13 @@ double* scratch_field(lbm_t* h, int c) {
 }
 double* scratch_partials(lbm_t* h) { return scratch_field(h, 3); }
 double* scratch_out(lbm_t* h) { return scratch_partials(h) + kReduceBlocks * 4; }
+// work counter, warps or blocks done, give-up flag of the kernels that claim
+// work: the last bytes of the area, which its rounding to 256 bytes leaves
+constexpr size_t kScratchTail = (kReduceBlocks * 4 + 4) * sizeof(double);
+static_assert((kScratchTail + 255) / 256 * 256 - kScratchTail >= 16, "no room for the counters");
+int* sched(const lbm_t* h) {
+  return reinterpret_cast<int*>(static_cast<char*>(h->scratch) + lbm_scratch_bytes(h) - 16);
+}
 
 void drop_graphs(lbm_t* h) {
   for (auto& g : h->graph)
@@ -167,6 +185,7 @@ void drop_graphs(lbm_t* h) {
       g = nullptr;
     }
   h->staged_grid = 0;  // the staged kernel's residency may have changed too
+  h->form_ready = false;
 }
 
 int ensure_memory(lbm_t* h) {
@@ -182,6 +201,15 @@ int ensure_memory(lbm_t* h) {
   lbmk::check_add(h->buf[1], bb);
   h->owns_memory = true;
   h->bound = true;
+  return LBM_OK;
+}
+
+// Zero the work counters once the memory is there (each launch that uses them
+// leaves them at zero).
+int clear_sched(lbm_t* h) {
+  if (h->sched_clear) return LBM_OK;
+  LBM_CUDA(cudaMemsetAsync(sched(h), 0, 4 * sizeof(int), h->stream));
+  h->sched_clear = true;
   return LBM_OK;
 }
 
@@ -286,10 +314,13 @@ void launch_fused_bx(const lbm_t* h, const void* a, void* b, int rows, cudaStrea
   });
 }
 
+// (picked by lbm_step itself: blocks of 64, which spread the boundary's quads
+// over twice as many SMs -- 200^2 f64 10.6 against 13.5 us a step, 400^2 f32
+// 3.6 against 3.9)
 template <typename T>
 void launch_fused(const lbm_t* h, const void* a, void* b, cudaStream_t s) {
-  switch (h->bx) {
-    case 64: launch_fused_bx<T, 64>(h, a, b, h->rows, s); break;
+  switch (h->form_auto ? 64 : h->bx) {
+    case 64: launch_fused_bx<T, 64>(h, a, b, h->form_auto ? 1 : h->rows, s); break;
     case 256: launch_fused_bx<T, 256>(h, a, b, h->rows, s); break;
     case 512: launch_fused_bx<T, 512>(h, a, b, h->rows, s); break;
     default: launch_fused_bx<T, 128>(h, a, b, h->rows, s); break;
@@ -328,7 +359,7 @@ void launch_staged(const lbm_t* h, const void* a, void* b, cudaStream_t s) {
   auto go = [&](auto kernel) {
     kernel<<<grid, block, smem, s>>>(A, B, h->d_inst,
                                      static_cast<const lbmk::Shift<typename lbmk::Store<T>::C>*>(h->d_shift),
-                                     h->d_items, h->n_items, h->nsbc, h->s_e, h->s_eps, h->s_q, h->d_sched);
+                                     h->d_items, h->n_items, h->nsbc, h->s_e, h->s_eps, h->s_q, sched(h));
   };
   with_shift(h, [&](auto zc) {
     constexpr bool Z = decltype(zc)::value;
@@ -346,93 +377,109 @@ void launch_staged(const lbm_t* h, const void* a, void* b, cudaStream_t s) {
   });
 }
 
-// Two-step pass: the rolling items are strips of Roll::OUT output columns
-// times bands of ts_band rows, taken with the frame chunks by a persistent
-// grid of as many blocks as fit on the device at once; each wave of items is
-// all strips of ts_wave_bands bands.  Bands of 16 rows (a restart costs four
-// staged and two computed rows) unless the domain gives every resident warp
-// more than 16 (f32) or 8 (16-bit) items: measured on pulse-2048 / 4096 /
-// 8192, f32 bands of 16 gave 128k / 147k / 162k MLUPS against 58-100k /
-// 111-147k / 157-160k for bands of 24-48, and 16-bit storage, bound by
-// instruction issue, gains from the longer bands at 8192^2 (29 rows: 207k
-// against 198k for 16).  Items that would fill one wave of warps and a bit
-// of a second are cut to one wave instead (f32 at 2048^2: 102k -> 128k).
+// Multi-step pass: the rolling items are strips of Roll::OUT output columns
+// times bands of rows, taken after the frame's tiles by a persistent grid of
+// as many blocks as fit on the device at once; each wave of items is all
+// strips of ts_wave_bands bands.
 template <typename T>
-void twostep_grid(lbm_t* h, int per_sm) {
+void pass_grid(lbm_t* h, int per_sm) {
   using R = lbmk::Roll<T>;
-  const int interior_x = h->nx - 4, interior_y = h->ny - 4;  // output nodes [2, n - 2)
-  h->ts_strips = (interior_x + R::OUT - 1) / R::OUT;
+  const int rows = std::max(1, h->ny - 4);  // of the shortest pass (two steps)
+  h->ts_strips = (std::max(h->nx - 4, 1) + R::OUT - 1) / R::OUT;
   const int warps = std::max(1, per_sm * h->sms * R::WARPS);
   const int per_wave = std::max(1, warps / h->ts_strips);  // bands side by side
-  const int items_per_warp = sizeof(T) == 4 ? 16 : 8;
-  const int want = std::max(1, std::min(items_per_warp * per_wave, interior_y));
-  h->ts_band = std::max(std::min(16, interior_y), (interior_y + want - 1) / want);
-  const long long items = (long long)h->ts_strips * ((interior_y + h->ts_band - 1) / h->ts_band);
-  if (items > warps && items < 2LL * warps && per_wave * h->ts_strips <= warps)
-    h->ts_band = std::max(h->ts_band, (interior_y + per_wave - 1) / per_wave);
-  h->ts_bands = (interior_y + h->ts_band - 1) / h->ts_band;
+  // rows per band, 24 / 48 / 64 / 96 / 128 at 8192^2: f32 267 / 242 / 237 / 238 / 247 us a step,
+  // f16 299 / 270 / 263 / 258 / 255 (4096^2 alike): a restart costs the rows above the band
+  // (2 K of them), a long band the lines neighbouring strips share
+  int want = sizeof(T) == 4 ? 64 : 96;
+  const int waves = std::max(1, (rows + per_wave * want / 2) / (per_wave * want));
+  h->ts_band = std::max(4, (rows + per_wave * waves - 1) / (per_wave * waves));
+  h->ts_bands = (rows + h->ts_band - 1) / h->ts_band;
   h->ts_wave_bands = std::min(per_wave, h->ts_bands);
   h->ts_waves = (h->ts_bands + h->ts_wave_bands - 1) / h->ts_wave_bands;
-  h->ts_grid = std::max(1, per_sm * h->sms);  // frame chunks as well as rolling items: every resident warp
-}
-
-template <typename T, int MODEL, bool SHIFT>
-void launch_twostep_k(const lbm_t* h, const T* A, T* B, cudaStream_t s) {
-  using C = typename lbmk::Store<T>::C;
-  const lbmk::Geom g{h->nx, h->ny, h->pitch, h->plane};
-  const lbmk::Rates<C> r = rates<C>(h);
-  // one launch: the frame chunks of step n + 1, the rolling items, the frame
-  // chunks of step n + 2 (32 frame threads per chunk)
-  const int n_f1 = (lbmk::frame_threads(h->nx, h->ny, lbmk::kFrameWidth) + 31) / 32;
-  const int n_f3 = (lbmk::frame_threads(h->nx, h->ny, 2) + 31) / 32;
-  lbmk::pass_kernel<T, MODEL, SHIFT><<<h->ts_grid, lbmk::kRollThreads, lbmk::Roll<T>::kSmem, s>>>(
-      A, B, static_cast<T*>(h->d_frame), g, h->nsbc, r, h->ts_strips, h->ts_band, h->ts_bands, h->ts_wave_bands,
-      h->ts_waves, n_f1, n_f3, h->d_sched);
+  h->ts_grid = std::max(1, per_sm * h->sms);
 }
 
 template <typename T>
-void launch_twostep(const lbm_t* h, const void* a, void* b, cudaStream_t s) {
+void launch_pass(const lbm_t* h, const void* a, void* b, int steps, cudaStream_t s) {
+  using C = typename lbmk::Store<T>::C;
   const T* A = static_cast<const T*>(a);
   T* B = static_cast<T*>(b);
+  const int n_tiles = lbmk::frame_tiles(h->nx, h->ny);
   with_shift(h, [&](auto zc) {
     constexpr bool Z = decltype(zc)::value;
+    auto go = [&](auto kernel) {
+      kernel<<<h->ts_grid, lbmk::kRollThreads, lbmk::Roll<T>::kSmem, s>>>(
+          A, B, geom(h), h->nsbc, rates<C>(h), steps, n_tiles, h->ts_strips, h->ts_band, h->ts_bands,
+          h->ts_wave_bands, h->ts_waves, sched(h));
+    };
     if (h->collision == 1)
-      launch_twostep_k<T, 1, Z>(h, A, B, s);
+      go(lbmk::pass_kernel<T, 1, Z>);
     else
-      launch_twostep_k<T, 0, Z>(h, A, B, s);
+      go(lbmk::pass_kernel<T, 0, Z>);
   });
 }
 
-// the two-step kernel serves this handle (f32 / f16 / bf16, no periodic axis, 8 x 8 nodes or more)
-bool twostep_ok(const lbm_t* h) {
-  return h->storage != LBM_F64 && !h->nsbc.periodic_x && !h->nsbc.periodic_y && h->nx >= 8 && h->ny >= 8;
+// the multi-step pass serves this handle (f32 / f16 / bf16, no periodic axis, 8 x 8 nodes or more)
+bool pass_ok(const lbm_t* h) {
+  return h->storage != LBM_F64 && !h->nsbc.periodic_x && !h->nsbc.periodic_y && h->nx >= 2 * lbmk::kPassSteps &&
+         h->ny >= 2 * lbmk::kPassSteps;
 }
 
 template <typename T>
-int twostep_prepare(lbm_t* h) {
-  if (!h->d_sched) {  // the give-up flag of the bounded waits (lbm_status reads it)
-    LBM_CUDA(cudaMalloc(&h->d_sched, 4 * sizeof(int)));
-    LBM_CUDA(cudaMemset(h->d_sched, 0, 4 * sizeof(int)));
-  }
-  if (!h->d_frame) {
-    h->frame_fn = lbmk::ring_offset(h->nx, h->ny, lbmk::kFrameWidth);
-    LBM_CUDA(cudaMalloc(&h->d_frame, (size_t)9 * h->frame_fn * sizeof(T)));
-  }
+int pass_prepare(lbm_t* h) {
   const int smem = (int)lbmk::Roll<T>::kSmem;
   cudaError_t e = cudaSuccess;
-  int per_sm = 0, sms = 0;
+  int per_sm = 0;
   for (const void* k : {(const void*)lbmk::pass_kernel<T, 0, false>, (const void*)lbmk::pass_kernel<T, 0, true>,
                         (const void*)lbmk::pass_kernel<T, 1, false>, (const void*)lbmk::pass_kernel<T, 1, true>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbmk::pass_kernel<T, 1, true>, lbmk::kRollThreads,
                                                       smem);
   if (e != cudaSuccess)
-    return fail(LBM_ECUDA, "two-step kernel: %d bytes of shared memory refused: %s", smem, cudaGetErrorString(e));
-  if (per_sm <= 0) return fail(LBM_ECUDA, "two-step kernel: no block fits on an SM");
-  h->sms = sms;
-  twostep_grid<T>(h, per_sm);
+    return fail(LBM_ECUDA, "multi-step pass: %d bytes of shared memory refused: %s", smem, cudaGetErrorString(e));
+  if (per_sm <= 0) return fail(LBM_ECUDA, "multi-step pass: no block fits on an SM");
+  pass_grid<T>(h, per_sm);
+  return LBM_OK;
+}
+
+// ---- tiles of a small domain -----------------------------------------------
+// tiles serve this handle at all (every form of it is covered: storage,
+// collision, edges); false for domains too narrow to cut
+bool tiles_ok(const lbm_t* h) { return h->nx >= 8 && h->ny >= 8; }
+
+template <typename T>
+void launch_tiles(const lbm_t* h, const void* a, void* b, int steps, cudaStream_t s) {
+  using C = typename lbmk::Store<T>::C;
+  with_shift(h, [&](auto zc) {
+    constexpr bool Z = decltype(zc)::value;
+    auto go = [&](auto kernel) {
+      kernel<<<h->tl_gx * h->tl_gy, lbmk::kTileThreads, h->tl_smem, s>>>(static_cast<const T*>(a), static_cast<T*>(b),
+                                                                        geom(h), h->nsbc, rates<C>(h), h->tl_gx,
+                                                                        h->tl_gy, steps);
+    };
+    if (h->collision == 1)
+      go(lbmk::tile_kernel<T, 1, Z>);
+    else
+      go(lbmk::tile_kernel<T, 0, Z>);
+  });
+}
+
+template <typename T>
+int tiles_prepare(lbm_t* h) {
+  lbmk::TilePlan p = lbmk::plan_tiles(h->nx, h->ny, h->storage == LBM_F64, h->nsbc.periodic_x, h->nsbc.periodic_y, h->sms);
+  if (p.steps == 0) return fail(LBM_EINVAL, "tiles: no plan");
+  h->tl_gx = p.gx;
+  h->tl_gy = p.gy;
+  h->tl_steps = p.steps;
+  h->tl_smem = p.smem;
+  cudaError_t e = cudaSuccess;
+  for (const void* k : {(const void*)lbmk::tile_kernel<T, 0, false>, (const void*)lbmk::tile_kernel<T, 0, true>,
+                        (const void*)lbmk::tile_kernel<T, 1, false>, (const void*)lbmk::tile_kernel<T, 1, true>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbmk::kTileRoom);
+  if (e != cudaSuccess)
+    return fail(LBM_ECUDA, "tiles: %d bytes of shared memory refused: %s", (int)lbmk::kTileRoom, cudaGetErrorString(e));
   return LBM_OK;
 }
 
@@ -478,10 +525,6 @@ int ensure_staged(lbm_t* h) {
       if (cudaMemcpy(h->d_shift, &z, sizeof z, cudaMemcpyHostToDevice) != cudaSuccess) rcz = LBM_ECUDA;
     });
     if (rcz) return fail(rcz, "staged step kernel: shift copy failed");
-    if (!h->d_sched) {
-      LBM_CUDA(cudaMalloc(&h->d_sched, 4 * sizeof(int)));
-      LBM_CUDA(cudaMemset(h->d_sched, 0, 4 * sizeof(int)));
-    }
     h->n_items = (int)items.size();
     h->items_storage = h->storage;
   }
@@ -519,27 +562,76 @@ void enqueue_macros_rows(const lbm_t* h, double* d_rho, double* d_ux, double* d_
   });
 }
 
-// One step from buffer `from` to 1 - from.  With `fork`, the NSBC kernel runs
-// on the side stream concurrently with the bulk kernel (both only read
-// buffer `from` and write disjoint nodes of the other buffer).
-// Two-step launches need the kernels' shared-memory attribute and the grid
-// (once the storage is fixed); 0 when the two-step kernel is off.
-int ensure_twostep(lbm_t* h) {
-  if (!h->twostep || !twostep_ok(h)) return LBM_OK;
+// The launch form lbm_step takes when none was asked for, by size and storage
+// (microseconds per step on a GB300, BGK):
+//   nodes            200^2   300^2   400^2   600^2  1024^2  1200^2  1700^2  2048^2  4096^2
+//   f32   one launch  3.1     3.3     3.6     5.7     9.0    14.2    33.4    46.1     181
+//         tiles       2.3     2.8     3.8     6.6    14.4
+//         pass                        5.2     7.2     9.8    11.3    15.8    19.0      65
+//   f16   one launch                  4.0     5.6     7.4    11.0    19.8    28.5     107
+//         pass                        6.8     7.5    11.5    14.3    19.2    23.6      75
+// A pass is a chain of rows, so it needs enough of them to fill the chip; a
+// tile's halo grows with the steps it takes.
+Form pick_form(const lbm_t* h) {
+  const long long nodes = (long long)h->nx * h->ny;
+  if (pass_ok(h) && nodes >= (h->elt == 4 ? kPassNodes32 : kPassNodes16)) return Form::Pass;
+  if (h->storage != LBM_F64 && tiles_ok(h) && nodes <= kTileNodes) return Form::Tiles;
+  return nodes <= kFusedNodes ? Form::Fused : Form::Pair;
+}
+
+// The form of the next steps, its grid and its kernels' attributes (nothing
+// is allocated).
+int prepare_form(lbm_t* h) {
+  if (h->form_ready) return LBM_OK;
+  if (!h->sms) {
+    int sms = 0;
+    LBM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    h->sms = sms;
+  }
+  h->form = h->form_auto ? (h->profiling ? Form::Pair : pick_form(h))
+            : h->staged                ? Form::Staged
+            : h->fused                 ? Form::Fused
+            : h->twostep && pass_ok(h) ? Form::Pass
+            : h->tiles && tiles_ok(h)  ? Form::Tiles
+                                       : Form::Pair;
   int rc = LBM_OK;
-  dispatch(h->storage, [&](auto tag) {
-    using T = decltype(tag);
-    if constexpr (!std::is_same<T, double>::value) rc = twostep_prepare<T>(h);
-  });
+  if (h->form == Form::Pass || h->form == Form::Tiles)
+    dispatch(h->storage, [&](auto tag) {
+      using T = decltype(tag);
+      if (h->form == Form::Tiles) {
+        rc = tiles_prepare<T>(h);
+      } else if constexpr (!std::is_same<T, double>::value) {
+        rc = pass_prepare<T>(h);
+      }
+    });
+  h->form_ready = rc == LBM_OK;
   return rc;
 }
 
-// Two steps from buffer `from` to 1 - from (one launch of the pass kernel).
-void enqueue_twostep(const lbm_t* h, int from, cudaStream_t s) {
-  dispatch(h->storage, [&](auto tag) {
-    using T = decltype(tag);
-    if constexpr (!std::is_same<T, double>::value) launch_twostep<T>(h, h->buf[from], h->buf[1 - from], s);
-  });
+int steps_per_launch(const lbm_t* h) {
+  return h->form == Form::Pass ? lbmk::kPassSteps : (h->form == Form::Tiles ? h->tl_steps : 1);
+}
+
+// One step from buffer `from` to 1 - from.  With `fork`, the NSBC kernel runs
+// on the side stream concurrently with the bulk kernel (both only read
+// buffer `from` and write disjoint nodes of the other buffer).
+void enqueue_step(const lbm_t* h, int from, cudaStream_t s, bool fork);
+
+// One launch of `steps` steps (the form's own number or fewer) from buffer
+// `from` to 1 - from; the forms of one step take one.
+void enqueue_launch(const lbm_t* h, int from, int steps, cudaStream_t s, bool fork) {
+  if (h->form == Form::Tiles || (h->form == Form::Pass && steps > 1)) {
+    dispatch(h->storage, [&](auto tag) {
+      using T = decltype(tag);
+      if (h->form == Form::Tiles) {
+        launch_tiles<T>(h, h->buf[from], h->buf[1 - from], steps, s);
+      } else if constexpr (!std::is_same<T, double>::value) {
+        launch_pass<T>(h, h->buf[from], h->buf[1 - from], steps, s);
+      }
+    });
+  } else {
+    enqueue_step(h, from, s, fork);
+  }
 }
 
 void enqueue_step(const lbm_t* h, int from, cudaStream_t s, bool fork) {
@@ -551,7 +643,7 @@ void enqueue_step(const lbm_t* h, int from, cudaStream_t s, bool fork) {
       launch_staged<T>(h, a, b, s);
       return;
     }
-    if (h->fused) {
+    if (h->form == Form::Fused) {
       launch_fused<T>(h, a, b, s);
       return;
     }
@@ -572,12 +664,7 @@ void enqueue_step(const lbm_t* h, int from, cudaStream_t s, bool fork) {
 int capture_graph(lbm_t* h, int from) {
   cudaGraph_t g = nullptr;
   LBM_CUDA(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-  if (h->twostep && twostep_ok(h)) {
-    // kGraphSteps / 2 launches of two steps: an even number of buffer swaps
-    for (int k = 0; k < kGraphSteps / 2; ++k) enqueue_twostep(h, (from + k) & 1, h->cap);
-  } else {
-    for (int k = 0; k < kGraphSteps; ++k) enqueue_step(h, (from + k) & 1, h->cap, true);
-  }
+  for (int k = 0; k < kGraphSteps; ++k) enqueue_step(h, (from + k) & 1, h->cap, true);
   cudaError_t e = cudaStreamEndCapture(h->cap, &g);
   if (e != cudaSuccess) return fail(LBM_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
   e = cudaGraphInstantiate(&h->graph[from], g, 0);
@@ -629,14 +716,14 @@ int enqueue_step_profiled(lbm_t* h, int from) {
   return LBM_OK;
 }
 
-// A two-step pass with an event pair around its launch (counted as one bulk
-// launch; it carries two steps).
-int enqueue_twostep_profiled(lbm_t* h, int from) {
+// A launch of several steps with an event pair around it (counted as one bulk
+// launch).
+int enqueue_launch_profiled(lbm_t* h, int from, int steps) {
   cudaEvent_t e[2];
   int rc = profiled_pair(h, 0, e);
   if (rc) return rc;
   cudaEventRecord(e[0], h->stream);
-  enqueue_twostep(h, from, h->stream);
+  enqueue_launch(h, from, steps, h->stream, false);
   cudaEventRecord(e[1], h->stream);
   return LBM_OK;
 }
@@ -681,11 +768,7 @@ lbm_t* lbm_create(int32_t nx, int32_t ny, double tau, double farfield_rho, const
   h->nx = nx;
   h->ny = ny;
   h->tau = tau;
-  h->nsbc.gamma = 0.6;
-  h->nsbc.beta = 0.0;
-  h->nsbc.kappa = 3.0;
-  h->nsbc.order = 1;
-  h->nsbc.corner = 0;
+  h->nsbc.set(0.6, 0.0, 3.0, 0, 1);
   h->nsbc.m0[0] = farfield_rho;
   h->nsbc.m0[1] = farfield_u[0];
   h->nsbc.m0[2] = farfield_u[1];
@@ -710,8 +793,6 @@ void lbm_destroy(lbm_t* h) {
   if (h->d_items) cudaFree(h->d_items);
   if (h->d_inst) cudaFree(h->d_inst);
   if (h->d_shift) cudaFree(h->d_shift);
-  if (h->d_sched) cudaFree(h->d_sched);
-  if (h->d_frame) cudaFree(h->d_frame);
   if (h->cap) {
     cudaStreamDestroy(h->cap);
     cudaStreamDestroy(h->side);
@@ -727,11 +808,7 @@ int lbm_set_nsbc(lbm_t* h, double gamma, double beta, double kappa, int32_t corn
   if (!std::isfinite(gamma) || !std::isfinite(beta) || !std::isfinite(kappa) || (grad_order != 1 && grad_order != 2) ||
       (corner_mode != LBM_CORNER_DIAGONAL && corner_mode != LBM_CORNER_MEAN))
     return fail(LBM_EINVAL, "lbm_set_nsbc: need finite gamma, beta, kappa, corner_mode 0 or 1 and grad_order 1 or 2");
-  h->nsbc.gamma = gamma;
-  h->nsbc.beta = beta;
-  h->nsbc.kappa = kappa;
-  h->nsbc.order = grad_order;
-  h->nsbc.corner = corner_mode;
+  h->nsbc.set(gamma, beta, kappa, corner_mode, grad_order);
   drop_graphs(h);
   return LBM_OK;
 }
@@ -888,6 +965,8 @@ int lbm_init_device(lbm_t* h, const double* d_rho, const double* d_ux, const dou
   int rc = ensure_memory(h);
   if (rc) return rc;
   h->cur = 0;
+  rc = clear_sched(h);
+  if (rc) return rc;
   enqueue_init_rows(h, d_rho, d_ux, d_uy, 0, h->ny);
   rc = check_launch();
   if (rc) return rc;
@@ -902,6 +981,7 @@ int lbm_init(lbm_t* h, const double* rho, const double* ux, const double* uy) {
   int rc = ensure_memory(h);
   if (rc) return rc;
   rc = ensure_streams(h);
+  if (!rc) rc = clear_sched(h);
   if (rc) return rc;
   // the copy of row chunk c (side stream, copy engine) overlaps the
   // initialisation of chunk c - 1 (the handle's stream)
@@ -934,24 +1014,12 @@ int lbm_step(lbm_t* h, int32_t n) {
   if (n < 0) return fail(LBM_EINVAL, "lbm_step: n=%d < 0", n);
   if (!h->initialised) return fail(LBM_ESTATE, "lbm_step: call lbm_init first");
   int rc = ensure_streams(h);
+  if (!rc) rc = prepare_form(h);
   if (!rc) rc = ensure_staged(h);
-  if (!rc) rc = ensure_twostep(h);
   if (rc) return rc;
-  const bool two = h->twostep && twostep_ok(h);
+  const int per = steps_per_launch(h);
   int left = n;
-  if (h->profiling) {
-    for (; two && left >= 2; left -= 2) {
-      rc = enqueue_twostep_profiled(h, h->cur);
-      if (rc) return rc;
-      h->cur ^= 1;
-    }
-    for (; left > 0; --left) {
-      rc = enqueue_step_profiled(h, h->cur);
-      if (rc) return rc;
-      h->cur ^= 1;
-    }
-  }
-  if (left >= kGraphSteps) {
+  if (!h->profiling && per == 1 && left >= kGraphSteps) {
     if (!h->graph[h->cur]) {
       rc = capture_graph(h, h->cur);
       if (rc) return rc;
@@ -961,13 +1029,19 @@ int lbm_step(lbm_t* h, int32_t n) {
       left -= kGraphSteps;  // kGraphSteps is even: h->cur is unchanged
     }
   }
-  for (; two && left >= 2; left -= 2) {
-    enqueue_twostep(h, h->cur, h->stream);
+  while (left > 0) {
+    int take = std::min(per, left);
+    // a pass takes at least two steps: five are three and two, not four and one
+    if (h->form == Form::Pass && left - take == 1 && take > 2) --take;
+    // the last tile launches share what is left evenly
+    if (h->form == Form::Tiles) take = (left + (left + per - 1) / per - 1) / ((left + per - 1) / per);
+    if (!h->profiling)
+      enqueue_launch(h, h->cur, take, h->stream, false);
+    else
+      rc = take > 1 ? enqueue_launch_profiled(h, h->cur, take) : enqueue_step_profiled(h, h->cur);
+    if (rc) return rc;
     h->cur ^= 1;
-  }
-  for (; left > 0; --left) {  // an odd last step: the kernel pair
-    enqueue_step(h, h->cur, h->stream, false);
-    h->cur ^= 1;
+    left -= take;
   }
   rc = check_launch();
   if (rc) return rc;
@@ -1054,6 +1128,7 @@ int lbm_get_populations(lbm_t* h, double* f) {
 int lbm_set_populations(lbm_t* h, const double* f) {
   if (!h || !f) return fail(LBM_EINVAL, "lbm_set_populations: NULL argument");
   int rc = ensure_memory(h);
+  if (!rc) rc = clear_sched(h);
   if (rc) return rc;
   const long long n = (long long)h->nx * h->ny;
   h->cur = 0;
@@ -1133,6 +1208,7 @@ int lbm_load_state(lbm_t* h, const void* host, size_t bytes) {
                   hd.m0[0], hd.m0[1], hd.m0[2]);
   if (hd.steps < 0) return fail(LBM_EINVAL, "lbm_load_state: step count %lld < 0", (long long)hd.steps);
   int rc = ensure_memory(h);
+  if (!rc) rc = clear_sched(h);
   if (rc) return rc;
   h->cur = 0;
   const size_t bb = lbm_buffer_bytes(h);
@@ -1173,6 +1249,7 @@ int lbm_reduce(lbm_t* h, const double* ref_rho, const double* ref_ux, const doub
 int lbm_profile(lbm_t* h, int32_t enable) {
   if (!h) return fail(LBM_EINVAL, "lbm_profile: NULL handle");
   h->profiling = enable != 0;
+  drop_graphs(h);  // the form lbm_step picks by itself depends on it
   h->ev_used = 0;
   return LBM_OK;
 }
@@ -1211,6 +1288,8 @@ int lbm_set_launch(lbm_t* h, int32_t threads_x, int32_t rows, int32_t prefetch_r
   h->staged = 0;
   h->fused = false;
   h->twostep = false;
+  h->tiles = false;
+  h->form_auto = false;
   drop_graphs(h);
   return LBM_OK;
 }
@@ -1218,9 +1297,11 @@ int lbm_set_launch(lbm_t* h, int32_t threads_x, int32_t rows, int32_t prefetch_r
 int lbm_set_fused(lbm_t* h, int32_t enable) {
   if (!h) return fail(LBM_EINVAL, "lbm_set_fused: NULL handle");
   h->fused = enable != 0;
+  h->form_auto = false;
   if (h->fused) {
     h->staged = 0;
     h->twostep = false;
+    h->tiles = false;
   }
   drop_graphs(h);
   return LBM_OK;
@@ -1233,9 +1314,11 @@ int lbm_set_staged(lbm_t* h, int32_t stages) {
   if (stages != 0 && stages != 3 && stages != 4)
     return fail(LBM_EINVAL, "lbm_set_staged: stages=%d (0 = off, 3 or 4)", stages);
   h->staged = stages;
+  h->form_auto = false;
   if (stages) {
     h->fused = false;
     h->twostep = false;
+    h->tiles = false;
   }
   drop_graphs(h);
   return LBM_OK;
@@ -1245,12 +1328,14 @@ int32_t lbm_get_staged(const lbm_t* h) { return h ? h->staged : LBM_EINVAL; }
 
 int lbm_set_twostep(lbm_t* h, int32_t enable) {
   if (!h) return fail(LBM_EINVAL, "lbm_set_twostep: NULL handle");
-  if (enable && !twostep_ok(h))
+  if (enable && !pass_ok(h))
     return fail(LBM_EINVAL, "lbm_set_twostep: needs f32, f16 or bf16 storage, no periodic axis and 8 x 8 nodes or more");
   h->twostep = enable != 0;
+  h->form_auto = false;
   if (h->twostep) {
     h->staged = 0;
     h->fused = false;
+    h->tiles = false;
   }
   drop_graphs(h);
   return LBM_OK;
@@ -1260,11 +1345,11 @@ int32_t lbm_get_twostep(const lbm_t* h) { return h ? (h->twostep ? 1 : 0) : LBM_
 
 int lbm_status(lbm_t* h) {
   if (!h) return fail(LBM_EINVAL, "lbm_status: NULL handle");
-  if (!h->d_sched) return LBM_OK;
+  if (!h->sched_clear) return LBM_OK;
   int flag = 0;
-  LBM_CUDA(cudaMemcpyAsync(&flag, h->d_sched + 2, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  LBM_CUDA(cudaMemcpyAsync(&flag, sched(h) + 2, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(cudaStreamSynchronize(h->stream));
-  if (flag) return fail(LBM_ETIMEOUT, "lbm_status: a bounded wait of the staged step kernel gave up");
+  if (flag) return fail(LBM_ETIMEOUT, "lbm_status: a bounded wait of a step kernel gave up");
   return LBM_OK;
 }
 
@@ -1280,13 +1365,14 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
   if (!tune_path.empty()) {
     tune_key = lbm_internal_tune_key("domain", h->storage, h->collision, zshift(h).on, {h->nx, h->ny});
     lbmtune::Entry e;
-    double bx = 0, r = 0, pf = 0, st = -1, fz = -1, ts = -1, ms = 0;
+    double bx = 0, r = 0, pf = 0, st = -1, fz = -1, ts = -1, tl = -1, ms = 0;
     if (lbmtune::lookup(tune_path, tune_key, &e) && e.get("threads_x", &bx) && e.get("rows", &r) &&
         e.get("prefetch_rows", &pf) && e.get("staged", &st) && e.get("fused", &fz) && e.get("twostep", &ts) &&
-        e.get("ms_per_step", &ms) && (st == 0 || st == 3 || st == 4) && (fz == 0 || fz == 1) &&
-        (ts == 0 || ts == 1) && lbm_set_launch(h, (int32_t)bx, (int32_t)r, (int32_t)pf) == LBM_OK &&
+        e.get("tiles", &tl) && e.get("ms_per_step", &ms) && (st == 0 || st == 3 || st == 4) && (fz == 0 || fz == 1) &&
+        (ts == 0 || ts == 1) && (tl == 0 || (tl == 1 && tiles_ok(h))) && lbm_set_launch(h, (int32_t)bx, (int32_t)r, (int32_t)pf) == LBM_OK &&
         (st == 0 || lbm_set_staged(h, (int32_t)st) == LBM_OK) && (fz == 0 || lbm_set_fused(h, 1) == LBM_OK) &&
         (ts == 0 || lbm_set_twostep(h, 1) == LBM_OK)) {
+      h->tiles = tl == 1;
       lbm_internal_tune_count(true);
       if (threads_x) *threads_x = h->bx;
       if (rows) *rows = h->rows;
@@ -1307,10 +1393,13 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
   const int reps = (int)std::max<long long>(4, std::min<long long>(64, (1LL << 28) / std::max(cells, 1LL)));
   float best = 1e30f;
   int best_bx = h->bx, best_rows = h->rows, best_pf = h->pf, best_staged = h->staged;
-  bool best_fused = h->fused, best_twostep = false;
-  h->twostep = false;
+  bool best_fused = h->fused, best_twostep = false, best_tiles = false;
+  const bool profiling = h->profiling;
+  h->twostep = h->tiles = h->form_auto = h->profiling = false;
   // whole steps as the graphs run them (NSBC kernel on the forked branch)
   auto time_steps = [&]() -> float {
+    h->form_ready = false;
+    if (prepare_form(h) != LBM_OK) return 1e30f;
     for (int k = 0; k < 2; ++k) enqueue_step(h, k & 1, h->stream, true);
     cudaEventRecord(e0, h->stream);
     for (int k = 0; k < reps; ++k) enqueue_step(h, k & 1, h->stream, true);
@@ -1327,8 +1416,7 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
   const bool use_graph = cells <= (1LL << 22);
   auto time_graph = [&]() -> float {
     drop_graphs(h);
-    if (h->staged && ensure_staged(h) != LBM_OK) return 1e30f;
-    if (h->twostep && ensure_twostep(h) != LBM_OK) return 1e30f;
+    if (prepare_form(h) != LBM_OK || ensure_staged(h) != LBM_OK) return 1e30f;
     if (capture_graph(h, 0) != LBM_OK) return 1e30f;
     const int n = std::max(1, reps / kGraphSteps);
     cudaGraphLaunch(h->graph[0], h->stream);
@@ -1379,33 +1467,33 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
       best_twostep = false;
     }
   }
-  // the two-step kernel: two steps per launch
+  // the forms of several steps per launch, launched as lbm_step does
   h->staged = 0;
-  if (twostep_ok(h)) {
-    h->twostep = true;
-    if (ensure_twostep(h) == LBM_OK) {
+  for (bool tiles : {false, true}) {
+    if (tiles ? !tiles_ok(h) || cells > kTileCells : !pass_ok(h)) continue;
+    h->twostep = !tiles;
+    h->tiles = tiles;
+    drop_graphs(h);
+    if (prepare_form(h) == LBM_OK) {
+      const int per = steps_per_launch(h), launches = std::max(4, reps / per);
+      for (int k = 0; k < 2; ++k) enqueue_launch(h, k & 1, per, h->stream, false);
+      cudaEventRecord(e0, h->stream);
+      for (int k = 0; k < launches; ++k) enqueue_launch(h, k & 1, per, h->stream, false);
+      cudaEventRecord(e1, h->stream);
       float ms = 1e30f;
-      if (use_graph) {
-        ms = time_graph();
-      } else {
-        const int launches = std::max(2, reps / 2);
-        for (int k = 0; k < 2; ++k) enqueue_twostep(h, k & 1, h->stream);
-        cudaEventRecord(e0, h->stream);
-        for (int k = 0; k < launches; ++k) enqueue_twostep(h, k & 1, h->stream);
-        cudaEventRecord(e1, h->stream);
-        if (cudaEventSynchronize(e1) == cudaSuccess) {
-          cudaEventElapsedTime(&ms, e0, e1);
-          ms /= 2.0f * launches;
-        }
+      if (cudaEventSynchronize(e1) == cudaSuccess) {
+        cudaEventElapsedTime(&ms, e0, e1);
+        ms /= (float)(per * launches);
       }
       if (ms < best) {
         best = ms;
-        best_twostep = true;
+        best_twostep = !tiles;
+        best_tiles = tiles;
         best_staged = 0;
         best_fused = false;
       }
     }
-    h->twostep = false;
+    h->twostep = h->tiles = false;
   }
   rc = check_launch();
   h->bx = best_bx;
@@ -1413,7 +1501,9 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
   h->pf = best_pf;
   h->staged = best_staged;
   h->fused = best_fused && !best_staged;
-  h->twostep = best_twostep && !best_staged && !h->fused;
+  h->twostep = best_twostep;
+  h->tiles = best_tiles;
+  h->profiling = profiling;
   drop_graphs(h);
   LBM_CUDA(cudaMemcpyAsync(h->buf[h->cur], backup, bb, cudaMemcpyDeviceToDevice, h->stream));
   LBM_CUDA(cudaFreeAsync(backup, h->stream));
@@ -1426,7 +1516,7 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
     lbmtune::Entry e{tune_key,
                      {{"threads_x", best_bx}, {"rows", best_rows}, {"prefetch_rows", best_pf},
                       {"staged", h->staged}, {"fused", h->fused ? 1 : 0}, {"twostep", h->twostep ? 1 : 0},
-                      {"ms_per_step", best}}};
+                      {"tiles", h->tiles ? 1 : 0}, {"ms_per_step", best}}};
     lbmtune::store(tune_path, e);  // a cache that cannot be written is only not reused
   }
   if (threads_x) *threads_x = best_bx;

@@ -76,15 +76,19 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 // clock cycles have passed without the phase completing.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long budget = kTmaWaitCycles) {
   const uint32_t a = smem_u32(bar);
-  const long long t0 = clock64();
-  do {
-    uint32_t done;
+  auto done = [&] {
+    uint32_t d;
     asm volatile(
         "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(done)
+        : "=r"(d)
         : "r"(a), "r"(parity)
         : "memory");
-    if (done) return true;
+    return d != 0;
+  };
+  if (done()) return true;  // the usual case: no clock is read
+  const long long t0 = clock64();
+  do {
+    if (done()) return true;
   } while (clock64() - t0 < budget);
   return false;
 }

@@ -534,7 +534,7 @@ class Simulation:
         return lbm_get_fused(self.h) == 1
 
     def set_twostep(self, enable=True):
-        """Two steps per launch, the step in between kept on chip (see lbm_set_twostep)."""
+        """Several steps per launch, the steps in between kept on chip (see lbm_set_twostep)."""
         lbm_set_twostep(self.h, enable)
         return self
 
@@ -748,7 +748,7 @@ class Batch:
         return lbm_batch_status(self.b)
 
     def set_twostep(self, enable=True):
-        """Two steps per pass for every instance (see lbm_batch_set_twostep)."""
+        """Several steps per pass for every instance (see lbm_batch_set_twostep)."""
         lbm_batch_set_twostep(self.b, enable)
         return self
 
