@@ -294,7 +294,13 @@ struct Roll {
   // and strips start OUT apart, a multiple of 16 bytes for the copies
   static constexpr int OUT = (W - 2 * K) / (16 / (int)sizeof(T)) * (16 / (int)sizeof(T));
   static constexpr int DEPTH = 6;  // ring rows: three read, the others in flight
-  static constexpr int BLOCKS = 3;  // resident blocks per SM
+  // resident blocks per SM.  The kernel waits on its own chain of operations
+  // (57 % of issue slots used with three blocks), so what counts is how many
+  // warps the registers allow.  f32 carries 54 registers: three blocks (168).
+  // 16 bits carried as stored pairs are 27: four (128), 8192^2 f16 259 -> 247
+  // us a step, 3001 x 1777 bf16 29.7 -> 27.1; a fifth (96) spills and gives
+  // 245 and 27.3, but 273 against 262 in a mean flow.
+  static constexpr int BLOCKS = sizeof(T) == 4 ? 3 : 4;
   static constexpr int ROWE = 9 * W;
   static constexpr int WARPS = 4;  // independent warps per block
   static constexpr size_t kRing = (size_t)WARPS * DEPTH * ROWE * sizeof(T);
@@ -313,14 +319,29 @@ __device__ __forceinline__ float2 roll_lds(const __half* p) {
 __device__ __forceinline__ float2 roll_lds(const __nv_bfloat16* p) {
   return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
 }
-// two values rounded to the storage type, as a single step stores them
-__device__ __forceinline__ float2 roll_round(float2 v, const float*) { return v; }
-__device__ __forceinline__ float2 roll_round(float2 v, const __half*) {
-  return __half22float2(__floats2half2_rn(v.x, v.y));
-}
-__device__ __forceinline__ float2 roll_round(float2 v, const __nv_bfloat16*) {
-  return __bfloat1622float2(__floats2bfloat162_rn(v.x, v.y));
-}
+// What an item carries of two neighbouring nodes' values of one population
+// from row to row: the values rounded to the storage type, as a single step
+// stores them, 16-bit ones as the pair they are stored as.
+template <typename T>
+struct RollPair;
+template <>
+struct RollPair<float> {
+  float2 v;
+  static __device__ __forceinline__ RollPair of(float2 a) { return {a}; }
+  __device__ __forceinline__ float2 get() const { return v; }
+};
+template <>
+struct RollPair<__half> {
+  __half2 v;
+  static __device__ __forceinline__ RollPair of(float2 a) { return {__floats2half2_rn(a.x, a.y)}; }
+  __device__ __forceinline__ float2 get() const { return __half22float2(v); }
+};
+template <>
+struct RollPair<__nv_bfloat16> {
+  __nv_bfloat162 v;
+  static __device__ __forceinline__ RollPair of(float2 a) { return {__floats2bfloat162_rn(a.x, a.y)}; }
+  __device__ __forceinline__ float2 get() const { return __bfloat1622float2(v); }
+};
 // two neighbouring nodes' values of one population to device memory
 __device__ __forceinline__ void roll_st(float* p, float2 v) {
   if (in_bounds(p, 8)) __stcs(reinterpret_cast<float2*>(p), v);
@@ -352,6 +373,21 @@ __device__ __forceinline__ void shift_x(int c, float2& v) {
     const float l = __shfl_down_sync(0xffffffffu, v.x, 1);
     v.x = v.y;
     v.y = l;
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void shift_x(int c, RollPair<T>& p) {
+  if constexpr (sizeof(T) == 4) {
+    shift_x(c, p.v);
+  } else {
+    unsigned v;
+    memcpy(&v, &p.v, 4);
+    if (c > 0)
+      v = __byte_perm(__shfl_up_sync(0xffffffffu, v, 1), v, 0x5432);  // {left's second, first}
+    else if (c < 0)
+      v = __byte_perm(v, __shfl_down_sync(0xffffffffu, v, 1), 0x5432);  // {second, right's first}
+    memcpy(&p.v, &v, 4);
   }
 }
 
@@ -389,8 +425,9 @@ struct RollStage {
 // What a rolling item carries from row to row for step n + j, j = 1 .. K - 1,
 // all already pulled along x: of the newest row r the c_y = 0 (mid) and c_y =
 // +1 (up1) populations, and of row r - 1 the c_y = +1 ones (up2).
+template <typename T>
 struct RollCarry {
-  float2 up2[kPassSteps - 1][3], mid[kPassSteps - 1][3], up1[kPassSteps - 1][3];
+  RollPair<T> up2[kPassSteps - 1][3], mid[kPassSteps - 1][3], up1[kPassSteps - 1][3];
 };
 
 // State row s (ring slot `slot`) has arrived: step n + j of row s - j for j =
@@ -402,7 +439,7 @@ struct RollCarry {
 template <bool FULL, typename T, int MODEL, bool SHIFT>
 __device__ __forceinline__ void roll_row(RollStage<T>& stage, T*& out, const Geom& g,
                                          const Rates<typename Store<T>::C>& r, int K, int x0, int s0, int s, int s1,
-                                         int slot, const T* ring, int lo, int hi, bool whole, bool some, RollCarry& c,
+                                         int slot, const T* ring, int lo, int hi, bool whole, bool some, RollCarry<T>& c,
                                          const CellConst<float2>& k) {
   using R = Roll<T>;
   using S = Store<T>;
@@ -429,26 +466,27 @@ __device__ __forceinline__ void roll_row(RollStage<T>& stage, T*& out, const Geo
   for (int j = 1; j < KM; ++j) {
     if (FULL || (live && j < K)) {
       // h: step n + j of row s - j
+      RollPair<T> n[9];
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
-        h[i] = roll_round(h[i], ring);
-        shift_x(cx(i), h[i]);
+        n[i] = RollPair<T>::of(h[i]);
+        shift_x(cx(i), n[i]);
       }
       float2 o[9];
-      o[0] = c.mid[j - 1][0];
-      o[1] = c.mid[j - 1][1];
-      o[2] = c.mid[j - 1][2];
-      o[3] = c.up2[j - 1][0];
-      o[5] = c.up2[j - 1][1];
-      o[7] = c.up2[j - 1][2];
-      o[4] = h[4];
-      o[6] = h[6];
-      o[8] = h[8];
+      o[0] = c.mid[j - 1][0].get();
+      o[1] = c.mid[j - 1][1].get();
+      o[2] = c.mid[j - 1][2].get();
+      o[3] = c.up2[j - 1][0].get();
+      o[5] = c.up2[j - 1][1].get();
+      o[7] = c.up2[j - 1][2].get();
+      o[4] = n[4].get();
+      o[6] = n[6].get();
+      o[8] = n[8].get();
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         c.up2[j - 1][a] = c.up1[j - 1][a];
-        c.up1[j - 1][a] = h[3 + 2 * a];
-        c.mid[j - 1][a] = h[a];
+        c.up1[j - 1][a] = n[3 + 2 * a];
+        c.mid[j - 1][a] = n[a];
       }
       if (!FULL) live = s >= s0 + 2 * (j + 1);  // the rows above exist from here on
       if (FULL || live) {
@@ -494,11 +532,11 @@ __device__ __forceinline__ bool roll_item(const T* __restrict__ A, T* __restrict
                      (uint32_t)(min(X0 + R::W, g.pitch) - X0) * (uint32_t)sizeof(T), smem_u32(bar),
                      smem_u32(ring) + lane * (uint32_t)(R::W * sizeof(T)), g.pitch, lane};
   for (int k = 0; k < min(R::DEPTH, s1 - s0 + 1); ++k) stage.row(k);
-  RollCarry c;
+  RollCarry<T> c;
 #pragma unroll
   for (int j = 0; j < R::K - 1; ++j)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) c.up2[j][a] = c.mid[j][a] = c.up1[j][a] = make_float2(0.f, 0.f);
+    for (int a = 0; a < 3; ++a) c.up2[j][a] = c.mid[j][a] = c.up1[j][a] = RollPair<T>::of(make_float2(0.f, 0.f));
   const int x0 = X0 + 2 * lane;
   T* out = B + (long long)Ya * g.pitch + x0;  // the lane's nodes of the next row stored
   const int lo = X0 + K, hi = min(g.nx - K, X0 + K + R::OUT);
