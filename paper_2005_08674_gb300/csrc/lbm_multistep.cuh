@@ -15,7 +15,9 @@
 //       nodes (Sec. 5) included.  The nodes near the edges of a large domain
 //       (its frame) are such tiles, and a small domain is nothing but tiles.
 //
-// Neither waits for another block: what an item needs it computes itself.
+// Neither waits for another block: what an item needs it computes itself.  A
+// domain whose state fits the SMs' shared memory can also stay there for all
+// the steps of a call (resident_kernel); its blocks exchange halos.
 #pragma once
 
 #include "lbm_kernels.cuh"
@@ -89,24 +91,26 @@ __host__ __device__ constexpr size_t tile_bytes(int w, int h) {
   return (size_t)2 * 9 * w * h * sizeof(C);
 }
 
-// `steps` steps of the output nodes `t` (A: step n, B: step n + steps), by a
-// block of NT threads.  Step j is computed on the output rectangle widened by
-// steps - j nodes on each side (clipped at the domain's edges, running past
-// them along a periodic axis), so the last one needs no other tile's results.
-// Sides of the rectangle that lie on an edge are at least two nodes deep:
-// the second-order difference reads the node two further in.
-template <typename T, int MODEL, bool SHIFT, int NT>
-__device__ __forceinline__ void tile_steps(const T* __restrict__ A, T* __restrict__ B, const Geom& g, const Nsbc& p,
-                                           const Rates<typename Store<T>::C>& r, const TileRect& t, int steps,
-                                           typename Store<T>::C* smem) {
+// The region of a tile: its output nodes and `halo` more on each side, cut at
+// the domain's edges and running past them along a periodic axis.
+struct TileRegion {
+  int x0, y0, w, h;
+};
+
+__host__ __device__ inline TileRegion tile_region(int nx, int ny, bool px, bool py, const TileRect& t, int halo) {
+  const int x0 = px || t.x0 > halo ? t.x0 - halo : 0, x1 = px || t.x1 + halo < nx ? t.x1 + halo : nx;
+  const int y0 = py || t.y0 > halo ? t.y0 - halo : 0, y1 = py || t.y1 + halo < ny ? t.y1 + halo : ny;
+  return TileRegion{x0, y0, x1 - x0, y1 - y0};
+}
+
+// The state of the region, from A to shared memory, by a block of NT threads.
+template <typename T, int NT>
+__device__ __forceinline__ void tile_load(const T* __restrict__ A, const Geom& g, const TileRegion& reg,
+                                          typename Store<T>::C* smem) {
   using S = Store<T>;
   using C = typename S::C;
-  const int tid = threadIdx.x;
-  const bool px = p.periodic_x != 0, py = p.periodic_y != 0;
-  const int rx0 = px ? t.x0 - steps : max(t.x0 - steps, 0), rx1 = px ? t.x1 + steps : min(t.x1 + steps, g.nx);
-  const int ry0 = py ? t.y0 - steps : max(t.y0 - steps, 0), ry1 = py ? t.y1 + steps : min(t.y1 + steps, g.ny);
-  const int w = rx1 - rx0, h = ry1 - ry0;
-  const int other = 9 * w * h;  // the two steps' states: smem and smem + other
+  const int tid = threadIdx.x, w = reg.w, rx0 = reg.x0, ry0 = reg.y0;
+  const int other = 9 * w * reg.h;
   // element e of the region's state: population k % 9 of row k / 9, k = e / w
   // (the factor is exact: e w < 2^32).  Asynchronous copies, or eight loads
   // of 16-bit values at once, keep every load of the tile in flight.
@@ -134,122 +138,358 @@ __device__ __forceinline__ void tile_steps(const T* __restrict__ A, T* __restric
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  for (int j = 1; j <= steps; ++j) {
-    const C* __restrict__ src = smem + (j & 1 ? 0 : other);
-    C* __restrict__ dst = smem + (j & 1 ? other : 0);
-    const bool last = j == steps;
-    const int e = steps - j;
-    const int ax = px ? t.x0 - e : max(t.x0 - e, 0), bx = px ? t.x1 + e : min(t.x1 + e, g.nx);
-    const int ay = py ? t.y0 - e : max(t.y0 - e, 0), by = py ? t.y1 + e : min(t.y1 + e, g.ny);
-    // perimeter rows and columns inside the step's rectangle (along a
-    // periodic axis also their images a period away)
-    const int wj = bx - ax, hj = by - ay;
-    int n_rows = 0, n_cols = 0, rows[4], cols[4];
-#pragma unroll
+}
+
+// ---- boundary nodes of a resident tile --------------------------------------
+// Where a quad of lanes finds its boundary node, worked out once per launch:
+// nsbc_edge_nodes, which serves any source, looks its node up and wraps every
+// address anew in each step, half of the instructions of a chain that all
+// the other warps of the block wait for.
+struct EdgeSlot {
+  int x, y;      // may lie past the domain along a periodic axis
+  int at, back;  // the node's population 0 in the region's state; the same of this lane's node b - q n
+  EdgeNode en;   // the node's own coordinates and normal
+  bool any, kp, km, want;  // a node; its pulled pair is known; the lane's node b - q n is needed
+};
+
+// Slot k (a quad) of the perimeter nodes inside the output rectangle widened by e.
+struct EdgeList {
+  int ax, bx, ay, by, n_rows, n_cols, n;
+  bool px, py;
+  __host__ __device__ EdgeList(const TileRect& t, int e, int nx, int ny, bool px_, bool py_) : px(px_), py(py_) {
+    ax = px || t.x0 > e ? t.x0 - e : 0;
+    bx = px || t.x1 + e < nx ? t.x1 + e : nx;
+    ay = py || t.y0 > e ? t.y0 - e : 0;
+    by = py || t.y1 + e < ny ? t.y1 + e : ny;
+    n_rows = n_cols = n = 0;
     for (int k = 0; k < 4; ++k) {
-      const int yk = k == 0 ? 0 : (k == 1 ? g.ny - 1 : (k == 2 ? -1 : g.ny));
-      const int xk = k == 0 ? 0 : (k == 1 ? g.nx - 1 : (k == 2 ? -1 : g.nx));
-      rows[k] = yk;
-      cols[k] = xk;
-      const bool ry = (k < 2 || py) && yk >= ay && yk < by, rx = (k < 2 || px) && xk >= ax && xk < bx;
-      n_rows |= ry << k;  // bit k: row rows[k] lies inside
-      n_cols |= rx << k;
+      const int yk = line(k, ny), xk = line(k, nx);
+      if ((k < 2 || py) && yk >= ay && yk < by) n_rows |= 1 << k, n += bx - ax;
+      if ((k < 2 || px) && xk >= ax && xk < bx) n_cols |= 1 << k, n += by - ay;
     }
-    const int n_per = __popc(n_rows) * wj + __popc(n_cols) * hj;
-    const int edge_slots = (4 * n_per + 31) & ~31;
-    // interior nodes: the rectangle without the edges of non-periodic axes
-    const int ix = px ? ax : max(ax, 1), jx = px ? bx : min(bx, g.nx - 1);
-    const int iy = py ? ay : max(ay, 1), jy = py ? by : min(by, g.ny - 1);
-    const int wi = max(jx - ix, 0), n_int = wi * max(jy - iy, 0);
-    constexpr bool PAIR = std::is_same<C, float>::value;
-    const int n_work = PAIR ? (n_int + 1) >> 1 : n_int;
-    // q / wi = high word of q mul: exact, n_int * wi < 2^32; a width of 1 has no such factor
-    const unsigned mul = wi > 1 ? 0xffffffffu / (unsigned)wi + 1u : 0u;  // ceil(2^32 / wi)
-    for (int u = tid; u < edge_slots + n_work; u += NT) {
-      if (u < edge_slots) {
-        // a boundary node per quad of lanes
-        int k = u >> 2;
-        if (k >= n_per) continue;
-        int x = 0, y = 0;
-        bool found = false, twice = false;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          if (!found && (n_rows >> c & 1)) {
-            if (k < wj) {
-              found = true;
-              x = ax + k;
-              y = rows[c];
-            } else {
-              k -= wj;
-            }
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          if (!found && (n_cols >> c & 1)) {
-            if (k < hj) {
-              found = true;
-              x = cols[c];
-              y = ay + k;
-#pragma unroll
-              for (int d = 0; d < 4; ++d) twice |= (n_rows >> d & 1) && rows[d] == y;  // already taken with its row
-            } else {
-              k -= hj;
-            }
-          }
-        }
-        if (!found || twice) continue;
-        EdgeNode en[1];
-        const bool ok[1] = {true};
-        en[0].x = x < 0 ? x + g.nx : (x >= g.nx ? x - g.nx : x);
-        en[0].y = y < 0 ? y + g.ny : (y >= g.ny ? y - g.ny : y);
-        en[0].nxn = px ? 0 : (en[0].x == 0 ? -1 : (en[0].x == g.nx - 1 ? 1 : 0));
-        en[0].nyn = py ? 0 : (en[0].y == 0 ? -1 : (en[0].y == g.ny - 1 ? 1 : 0));
-        en[0].open = en[0].nxn != 0 || en[0].nyn != 0;
-        const TileState<T> from{const_cast<C*>(src), rx0, ry0, w, g.nx, g.ny, h};
-        if (last)
-          nsbc_edge_nodes<T, MODEL, 1, SHIFT>(from, GlobalDst<T>{B, g.plane, g.pitch}, g, p, r, en, ok, tid & 3);
-        else
-          nsbc_edge_nodes<T, MODEL, 1, SHIFT>(from, TileState<T>{dst, rx0, ry0, w, g.nx, g.ny, h}, g, p, r, en, ok,
-                                              tid & 3);
-        continue;
-      }
-      constexpr int N = PAIR ? 2 : 1;  // two nodes at once in float (paired FP32 instructions)
-      C v[9][N];
-      int at[N], gx[N], gy[N];
-      bool ok[N];
-#pragma unroll
-      for (int k = 0; k < N; ++k) {
-        const int q = u - edge_slots + k * n_work;
-        ok[k] = q < n_int;
-        const int qq = ok[k] ? q : 0;
-        const int row = wi > 1 ? (int)__umulhi(mul, (unsigned)qq) : qq;
-        gy[k] = iy + row;
-        gx[k] = ix + (qq - row * wi);
-        if (px) ok[k] = ok[k] && gx[k] != 0 && gx[k] != g.nx - 1 && gx[k] != -1 && gx[k] != g.nx;
-        if (py) ok[k] = ok[k] && gy[k] != 0 && gy[k] != g.ny - 1 && gy[k] != -1 && gy[k] != g.ny;
-        at[k] = 9 * (gy[k] - ry0) * w + (gx[k] - rx0);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) v[i][k] = src[at[k] + (i - 9 * cy(i)) * w - cx(i)];
-      }
-      collide_nodes<MODEL, SHIFT, PAIR>(v, r, C(S::kScale));
-#pragma unroll
-      for (int k = 0; k < N; ++k) {
-        if (!ok[k]) continue;
-        if (last) {
-          const int x = gx[k] < 0 ? gx[k] + g.nx : (gx[k] >= g.nx ? gx[k] - g.nx : gx[k]);
-          const int y = gy[k] < 0 ? gy[k] + g.ny : (gy[k] >= g.ny ? gy[k] - g.ny : gy[k]);
-          T* o = B + (long long)y * g.pitch + x;
-#pragma unroll
-          for (int i = 0; i < 9; ++i) S::st1r(o + i * g.plane, v[i][k]);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 9; ++i) dst[at[k] + i * w] = stored<T>(v[i][k]);
-        }
-      }
-    }
-    __syncthreads();
   }
+  // the first and last line of an axis, and along a periodic one their images
+  static __host__ __device__ int line(int k, int n) { return k == 0 ? 0 : (k == 1 ? n - 1 : (k == 2 ? -1 : n)); }
+  // node k < n; false where a column's node already came with its row
+  __host__ __device__ bool node(int k, int nx, int ny, int& x, int& y) const {
+    for (int c = 0; c < 4; ++c)
+      if (n_rows >> c & 1) {
+        if (k < bx - ax) {
+          x = ax + k;
+          y = line(c, ny);
+          return true;
+        }
+        k -= bx - ax;
+      }
+    for (int c = 0; c < 4; ++c)
+      if (n_cols >> c & 1) {
+        if (k < by - ay) {
+          x = line(c, nx);
+          y = ay + k;
+          for (int d = 0; d < 4; ++d)
+            if ((n_rows >> d & 1) && line(d, ny) == y) return false;
+          return true;
+        }
+        k -= by - ay;
+      }
+    return false;
+  }
+};
+
+__device__ __forceinline__ EdgeSlot edge_slot(const EdgeList& list, int u, const TileRegion& reg, const Geom& g,
+                                              const Nsbc& p) {
+  EdgeSlot s;
+  const int q = u & 3;
+  s.x = s.y = 0;
+  s.any = (u >> 2) < list.n && list.node(u >> 2, g.nx, g.ny, s.x, s.y);
+  s.en.x = s.x < 0 ? s.x + g.nx : (s.x >= g.nx ? s.x - g.nx : s.x);
+  s.en.y = s.y < 0 ? s.y + g.ny : (s.y >= g.ny ? s.y - g.ny : s.y);
+  s.en.nxn = list.px ? 0 : (s.en.x == 0 ? -1 : (s.en.x == g.nx - 1 ? 1 : 0));
+  s.en.nyn = list.py ? 0 : (s.en.y == 0 ? -1 : (s.en.y == g.ny - 1 ? 1 : 0));
+  s.en.open = s.en.nxn != 0 || s.en.nyn != 0;
+  const QuadPair pr = quad_pair(q);
+  auto known = [&](int x, int y) {
+    return (list.px || (x >= 0 && x < g.nx)) && (list.py || (y >= 0 && y < g.ny));
+  };
+  s.kp = known(s.x - pr.cx, s.y - pr.cy);
+  s.km = known(s.x + pr.cx, s.y + pr.cy);
+  s.want = s.en.open && q <= p.order;
+  const bool split = p.corner == 1 && s.en.nxn != 0 && s.en.nyn != 0;  // the vertical edge's normal first
+  s.at = 9 * (s.y - reg.y0) * reg.w + s.x - reg.x0;
+  s.back = s.at - q * (9 * (split ? 0 : s.en.nyn) * reg.w + s.en.nxn);
+  return s;
+}
+
+// A node's results: to the next state in shared memory, and to device memory
+// at the end or where a neighbour tile's halo takes the node.
+template <typename T>
+struct EdgeDst {
+  using C = typename Store<T>::C;
+  C* s;  // population 0
+  int w;
+  T* b;
+  long long plane;
+  bool to_s, to_b;
+  __device__ __forceinline__ void st(int i, int, int, C v) const {
+    const T t = Store<T>::cvt(v);
+    if (to_s) s[i * w] = Store<T>::ld1s(&t);
+    if (to_b) Store<T>::st1(b + i * plane, v);
+  }
+};
+
+// nsbc_edge_nodes on a node of the region's state src (the same operations in
+// the same order); `from` is the state for the second pass of a corner.
+template <typename T, int MODEL, bool SHIFT>
+__device__ __forceinline__ void tile_edge(const typename Store<T>::C* __restrict__ src, const TileState<T>& from,
+                                          int w, const EdgeDst<T>& to, const Geom& g, const Nsbc& p,
+                                          const Rates<typename Store<T>::C>& r, const EdgeSlot& s, int q) {
+  using C = typename Store<T>::C;
+  const unsigned quad = 0xFu << ((threadIdx.x & 31) & ~3);
+  const QuadPair pr = quad_pair(q);
+  auto ld = [&](int o) { return Store<T>::kScale == 1 ? src[o] : src[o] * C(1.0 / Store<T>::kScale); };
+  const C hp = s.kp ? ld(s.at + (pr.ip - 9 * pr.cy) * w - pr.cx) : C(0);
+  const C hm = s.km ? ld(s.at + (pr.im + 9 * pr.cy) * w + pr.cx) : C(0);
+  const C h0 = ld(s.at);
+  C v[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) v[i] = s.want ? ld(s.back + i * w) : C(0);
+  const bool corner = s.en.nxn != 0 && s.en.nyn != 0, split = p.corner == 1 && corner;
+  Predicted<C> mine =
+      quad_predict<T, SHIFT>(v, far_of(r.z), quad, q < 3 ? q : 0, corner && !split, predict_of<C>(p));
+  if (split)
+    mine = predicted_mean(mine, corner_second_prediction<T, SHIFT>(from, s.en.x, s.en.y - q * s.en.nyn, far_of(r.z),
+                                                                  quad, q, predict_of<C>(p)));
+  const C mcq = predicted_value(mine);
+  C mc[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) mc[c] = __shfl_sync(quad, mcq, c, 4);
+  quad_finish<T, MODEL, SHIFT>(to, g, p, r, s.en, pr, q, quad, hp, hm, h0, s.kp, s.km, mc, true);
+}
+
+constexpr int kRowSlack = 72;  // elements
+
+// One step of a tile, src -> dst (region states in shared memory), by a block
+// of NT threads: computed on the output rectangle widened by e nodes on each
+// side (clipped at the domain's edges, running past them along a periodic
+// axis).  last: the step's output nodes go to B and nothing to dst.  Sides of
+// the rectangle that lie on an edge are at least two nodes deep: the
+// second-order difference reads the node two further in.
+template <typename T, int MODEL, bool SHIFT, int NT>
+__device__ __forceinline__ void tile_step(const typename Store<T>::C* __restrict__ src,
+                                          typename Store<T>::C* __restrict__ dst, T* __restrict__ B, const Geom& g,
+                                          const Nsbc& p, const Rates<typename Store<T>::C>& r, const TileRect& t,
+                                          const TileRegion& reg, int e, bool last) {
+  using S = Store<T>;
+  using C = typename S::C;
+  const int tid = threadIdx.x, w = reg.w, h = reg.h, rx0 = reg.x0, ry0 = reg.y0;
+  const bool px = p.periodic_x != 0, py = p.periodic_y != 0;
+  const int ax = px ? t.x0 - e : max(t.x0 - e, 0), bx = px ? t.x1 + e : min(t.x1 + e, g.nx);
+  const int ay = py ? t.y0 - e : max(t.y0 - e, 0), by = py ? t.y1 + e : min(t.y1 + e, g.ny);
+  // perimeter rows and columns inside the step's rectangle (along a
+  // periodic axis also their images a period away)
+  const int wj = bx - ax, hj = by - ay;
+  int n_rows = 0, n_cols = 0, rows[4], cols[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int yk = k == 0 ? 0 : (k == 1 ? g.ny - 1 : (k == 2 ? -1 : g.ny));
+    const int xk = k == 0 ? 0 : (k == 1 ? g.nx - 1 : (k == 2 ? -1 : g.nx));
+    rows[k] = yk;
+    cols[k] = xk;
+    const bool ry = (k < 2 || py) && yk >= ay && yk < by, rx = (k < 2 || px) && xk >= ax && xk < bx;
+    n_rows |= ry << k;  // bit k: row rows[k] lies inside
+    n_cols |= rx << k;
+  }
+  const int n_per = __popc(n_rows) * wj + __popc(n_cols) * hj;
+  const int edge_slots = (4 * n_per + 31) & ~31;
+  // interior nodes: the rectangle without the edges of non-periodic axes
+  const int ix = px ? ax : max(ax, 1), jx = px ? bx : min(bx, g.nx - 1);
+  const int iy = py ? ay : max(ay, 1), jy = py ? by : min(by, g.ny - 1);
+  const int wi = max(jx - ix, 0), n_int = wi * max(jy - iy, 0);
+  constexpr bool PAIR = std::is_same<C, float>::value;
+  const int n_work = PAIR ? (n_int + 1) >> 1 : n_int;
+  // q / wi = high word of q mul: exact, n_int * wi < 2^32; a width of 1 has no such factor
+  const unsigned mul = wi > 1 ? 0xffffffffu / (unsigned)wi + 1u : 0u;  // ceil(2^32 / wi)
+  for (int u = tid; u < edge_slots + n_work; u += NT) {
+    if (u < edge_slots) {
+      // a boundary node per quad of lanes
+      int k = u >> 2;
+      if (k >= n_per) continue;
+      int x = 0, y = 0;
+      bool found = false, twice = false;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (!found && (n_rows >> c & 1)) {
+          if (k < wj) {
+            found = true;
+            x = ax + k;
+            y = rows[c];
+          } else {
+            k -= wj;
+          }
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (!found && (n_cols >> c & 1)) {
+          if (k < hj) {
+            found = true;
+            x = cols[c];
+            y = ay + k;
+#pragma unroll
+            for (int d = 0; d < 4; ++d) twice |= (n_rows >> d & 1) && rows[d] == y;  // already taken with its row
+          } else {
+            k -= hj;
+          }
+        }
+      }
+      if (!found || twice) continue;
+      EdgeNode en[1];
+      const bool ok[1] = {true};
+      en[0].x = x < 0 ? x + g.nx : (x >= g.nx ? x - g.nx : x);
+      en[0].y = y < 0 ? y + g.ny : (y >= g.ny ? y - g.ny : y);
+      en[0].nxn = px ? 0 : (en[0].x == 0 ? -1 : (en[0].x == g.nx - 1 ? 1 : 0));
+      en[0].nyn = py ? 0 : (en[0].y == 0 ? -1 : (en[0].y == g.ny - 1 ? 1 : 0));
+      en[0].open = en[0].nxn != 0 || en[0].nyn != 0;
+      const TileState<T> from{const_cast<C*>(src), rx0, ry0, w, g.nx, g.ny, h};
+      const TileState<T> to{dst, rx0, ry0, w, g.nx, g.ny, h};
+      const GlobalDst<T> out{B, g.plane, g.pitch};
+      if (last)
+        nsbc_edge_nodes<T, MODEL, 1, SHIFT>(from, out, g, p, r, en, ok, tid & 3);
+      else
+        nsbc_edge_nodes<T, MODEL, 1, SHIFT>(from, to, g, p, r, en, ok, tid & 3);
+      continue;
+    }
+    constexpr int N = PAIR ? 2 : 1;  // two nodes at once in float (paired FP32 instructions)
+    C v[9][N];
+    int at[N], gx[N], gy[N];
+    bool ok[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const int q = u - edge_slots + k * n_work;
+      ok[k] = q < n_int;
+      const int qq = ok[k] ? q : 0;
+      const int row = wi > 1 ? (int)__umulhi(mul, (unsigned)qq) : qq;
+      gy[k] = iy + row;
+      gx[k] = ix + (qq - row * wi);
+      if (px) ok[k] = ok[k] && gx[k] != 0 && gx[k] != g.nx - 1 && gx[k] != -1 && gx[k] != g.nx;
+      if (py) ok[k] = ok[k] && gy[k] != 0 && gy[k] != g.ny - 1 && gy[k] != -1 && gy[k] != g.ny;
+      at[k] = 9 * (gy[k] - ry0) * w + (gx[k] - rx0);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) v[i][k] = src[at[k] + (i - 9 * cy(i)) * w - cx(i)];
+    }
+    collide_nodes<MODEL, SHIFT, PAIR>(v, r, C(S::kScale));
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      if (!ok[k]) continue;
+      if (last) {
+        const int x = gx[k] < 0 ? gx[k] + g.nx : (gx[k] >= g.nx ? gx[k] - g.nx : gx[k]);
+        const int y = gy[k] < 0 ? gy[k] + g.ny : (gy[k] >= g.ny ? gy[k] - g.ny : gy[k]);
+        T* o = B + (long long)y * g.pitch + x;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) S::st1r(o + i * g.plane, v[i][k]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) dst[at[k] + i * w] = stored<T>(v[i][k]);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// One step of a resident tile, as tile_step.  Beside it, the last step of a
+// round (e = 0) writes the nodes nearer than `ring` to a side that has a
+// neighbour to B as well.  list: the perimeter nodes of the round's widest
+// step, `mine` this thread's slot of it.
+template <typename T, int MODEL, bool SHIFT, int NT>
+__device__ __forceinline__ void resident_step(const typename Store<T>::C* __restrict__ src,
+                                              typename Store<T>::C* __restrict__ dst, T* __restrict__ B,
+                                              const Geom& g, const Nsbc& p, const Rates<typename Store<T>::C>& r,
+                                              const TileRect& t, const TileRegion& reg, int e, bool last, int ring,
+                                              const CellConst<float2>& cell, const EdgeList& list,
+                                              const EdgeSlot& mine) {
+  using S = Store<T>;
+  using C = typename S::C;
+  const int tid = threadIdx.x, w = reg.w, rx0 = reg.x0, ry0 = reg.y0;
+  const bool px = p.periodic_x != 0, py = p.periodic_y != 0;
+  const int ax = px ? t.x0 - e : max(t.x0 - e, 0), bx = px ? t.x1 + e : min(t.x1 + e, g.nx);
+  const int ay = py ? t.y0 - e : max(t.y0 - e, 0), by = py ? t.y1 + e : min(t.y1 + e, g.ny);
+  // output nodes [cx0, cx1) x [cy0, cy1): no neighbour takes them
+  const int cx0 = px || t.x0 > 0 ? t.x0 + ring : t.x0, cx1 = px || t.x1 < g.nx ? t.x1 - ring : t.x1;
+  const int cy0 = py || t.y0 > 0 ? t.y0 + ring : t.y0, cy1 = py || t.y1 < g.ny ? t.y1 - ring : t.y1;
+  auto publish = [&](int x, int y) { return e == 0 && !(x >= cx0 && x < cx1 && y >= cy0 && y < cy1); };
+  auto edge = [&](const EdgeSlot& s) {
+    if (!s.any || s.x < ax || s.x >= bx || s.y < ay || s.y >= by) return;
+    tile_edge<T, MODEL, SHIFT>(src, TileState<T>{const_cast<C*>(src), rx0, ry0, w, g.nx, g.ny, reg.h}, w,
+                               EdgeDst<T>{dst + s.at, w, B + (long long)s.en.y * g.pitch + s.en.x, g.plane, !last,
+                                          last || publish(s.x, s.y)},
+                               g, p, r, s, tid & 3);
+  };
+#pragma unroll 1
+  for (int u = tid; u < 4 * list.n; u += NT) edge(u == tid ? mine : edge_slot(list, u, reg, g, p));
+  // interior nodes: the rectangle without the edges of non-periodic axes
+  const int ix = px ? ax : max(ax, 1), jx = px ? bx : min(bx, g.nx - 1);
+  const int iy = py ? ay : max(ay, 1), jy = py ? by : min(by, g.ny - 1);
+  const int wi = max(jx - ix, 0);
+  // A warp takes 64 columns of a row, two nodes 32 apart per lane, so that
+  // a row costs one address per population; the warps the boundary leaves
+  // free take the rows where there are enough of them.  (Lanes past the
+  // row read what follows it in shared memory, kRowSlack at the end, and
+  // store nothing.)
+  constexpr int NW = NT / 32;
+  const int lane = tid & 31, busy = (4 * list.n + 31) >> 5, skip = 2 * busy <= NW ? busy : 0;
+  const int chunks = (wi + 63) >> 6, tasks = chunks * max(jy - iy, 0);
+  const bool pub = e == 0;
+  for (int q = (tid >> 5) - skip; q < tasks; q += NW - skip) {
+    if (q < 0) break;
+    const int chunk = chunks == 1 ? 0 : q / (jy - iy), y = iy + q - chunk * (jy - iy);
+    const int x = ix + 64 * chunk + lane;
+    const int at = 9 * (y - ry0) * w + (x - rx0);
+    float2 f[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const C* o = src + at + (i - 9 * cy(i)) * w - cx(i);
+      f[i] = make_float2(o[0], o[32]);
+    }
+    collide<MODEL, SHIFT>(f, r, C(S::kScale), cell);
+    auto inside = [&](int xk) {
+      return xk < jx && !(px && (xk == 0 || xk == g.nx - 1 || xk == -1 || xk == g.nx)) &&
+             !(py && (y == 0 || y == g.ny - 1 || y == -1 || y == g.ny));
+    };
+    const bool ok[2] = {inside(x), inside(x + 32)};
+    if (!last) {
+      C* o = dst + at;
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        if (ok[0]) o[i * w] = stored<T>(f[i].x);
+        if (ok[1]) o[i * w + 32] = stored<T>(f[i].y);
+      }
+    }
+    if (last || pub) {  // e = 0: no coordinate lies past the domain
+      T* o = B + (long long)y * g.pitch + x;
+      const bool out[2] = {ok[0] && (last || publish(x, y)), ok[1] && (last || publish(x + 32, y))};
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        if (out[0]) S::st1r(o + i * g.plane, f[i].x);
+        if (out[1]) S::st1r(o + i * g.plane + 32, f[i].y);
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// `steps` steps of the output nodes `t` (A: step n, B: step n + steps), by a
+// block of NT threads: step j is computed on the output rectangle widened by
+// steps - j nodes, so the last one needs no other tile's results.
+template <typename T, int MODEL, bool SHIFT, int NT>
+__device__ __forceinline__ void tile_steps(const T* __restrict__ A, T* __restrict__ B, const Geom& g, const Nsbc& p,
+                                           const Rates<typename Store<T>::C>& r, const TileRect& t, int steps,
+                                           typename Store<T>::C* smem) {
+  const TileRegion reg = tile_region(g.nx, g.ny, p.periodic_x != 0, p.periodic_y != 0, t, steps);
+  const int other = 9 * reg.w * reg.h;  // the two steps' states: smem and smem + other
+  tile_load<T, NT>(A, g, reg, smem);
+  for (int j = 1; j <= steps; ++j)
+    tile_step<T, MODEL, SHIFT, NT>(smem + (j & 1 ? 0 : other), smem + (j & 1 ? other : 0), B, g, p, r, t, reg,
+                                   steps - j, j == steps);
 }
 
 // ---------------------------------------------------------------------------
@@ -687,6 +927,183 @@ inline TilePlan plan_tiles(int nx, int ny, bool f64, bool px, bool py, int sms) 
         const double us = (t_launch + waves * block) / steps;
         if (us < best.us) best = TilePlan{gx, gy, steps, (int)smem, us};
       }
+  return best;
+}
+
+// ---------------------------------------------------------------------------
+// A domain that stays on chip: gx x gy tiles, a block each, all resident at
+// once (cooperative launch), hold the state in shared memory for all the
+// steps of a launch.  Every `halo` steps a block writes the nodes its
+// neighbours' halos take to device memory, raises its flag, waits for the
+// flags of its (up to 8) neighbours and reads its own halo.  Rounds write B
+// and A in turn: a block writes a buffer again two rounds later, when every
+// neighbour has raised the flag of the round between, so has read the first.
+// What bounds it: the boundary nodes' chain of operations, about 1 us a step in
+// the blocks that hold an edge, while the others wait for them in the
+// exchange, itself 1.6 us a round.  So rounds are long (the halo is computed
+// twice rather than exchanged), the boundary's lookups are made once, and its
+// warps are left out of the rows.  Microseconds a step against the forms of
+// one launch per step or per tile plan: 128^2 channel (MRT) 2.4 against 2.7,
+// 300^2 f32 2.3 against 2.8, 613 x 377 f16 3.5 against 4.0.  In double the FP64 pipe is the bound and the boundary blocks'
+// share of it the longest: 200^2 12.5 against 9.1, so it is not built.
+// ---------------------------------------------------------------------------
+constexpr int kFlagStride = 8;  // a flag per 32 bytes
+
+// The halo of a tile's region (the region without the tile), element by
+// element: first the whole rows above and below, then the sides of the rows
+// between.
+struct TileHalo {
+  int w, tw, th, top, left;      // region width, tile, rows above, columns beside
+  int cols, n_rows, n;           // columns of a row between; elements of the whole rows, of all
+  unsigned mul_w, mul_c;         // e / w and e / cols as high words (exact: e w < 2^32)
+  __host__ __device__ TileHalo(const TileRect& t, const TileRegion& reg)
+      : w(reg.w), tw(t.x1 - t.x0), th(t.y1 - t.y0), top(t.y0 - reg.y0), left(t.x0 - reg.x0) {
+    cols = w - tw;
+    n_rows = 9 * (reg.h - th) * w;
+    n = n_rows + 9 * th * cols;
+    mul_w = 0xffffffffu / (unsigned)w + 1u;
+    mul_c = cols > 1 ? 0xffffffffu / (unsigned)cols + 1u : 0u;
+  }
+  // element e < n: population i of region node (lx, ly)
+  __host__ __device__ void at(int e, int& i, int& lx, int& ly) const {
+    const bool row = e < n_rows;
+    if (!row) e -= n_rows;
+    const int k = row || cols > 1 ? (int)((unsigned long long)(unsigned)e * (row ? mul_w : mul_c) >> 32) : e;
+    lx = e - k * (row ? w : cols);
+    ly = k / 9;
+    i = k - 9 * ly;
+    if (row) {
+      if (ly >= top) ly += th;
+    } else {
+      if (lx >= left) lx += tw;
+      ly += top;
+    }
+  }
+};
+
+// from device memory, past the L1 cache
+template <typename T, int NT>
+__device__ __forceinline__ void tile_halo(const T* B, const Geom& g, const TileHalo& halo, const TileRegion& reg,
+                                          typename Store<T>::C* dst) {
+  using S = Store<T>;
+  constexpr int Q = 6;  // loads in flight per thread
+  for (int e0 = threadIdx.x; e0 < halo.n; e0 += Q * NT) {
+    T v[Q];
+    int at[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      at[q] = -1;
+      if (e0 + q * NT >= halo.n) continue;
+      int i, lx, ly;
+      halo.at(e0 + q * NT, i, lx, ly);
+      at[q] = (9 * ly + i) * reg.w + lx;
+      int x = reg.x0 + lx, y = reg.y0 + ly;
+      x = x < 0 ? x + g.nx : (x >= g.nx ? x - g.nx : x);
+      y = y < 0 ? y + g.ny : (y >= g.ny ? y - g.ny : y);
+      const T* src = B + i * g.plane + (long long)y * g.pitch + x;
+      v[q] = in_bounds(src, sizeof(T)) ? __ldcg(src) : T(0.f);
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (at[q] >= 0) dst[at[q]] = S::ld1s(&v[q]);
+  }
+}
+
+// flags[block]: rounds whose outer nodes the block has written (zero at
+// launch).  A wait that gives up sets err[2] and ends its block; so, in turn,
+// do the blocks that wait for it.
+template <typename T, int MODEL, bool SHIFT>
+__global__ void __launch_bounds__(kTileThreads)
+    resident_kernel(T* A, T* B, Geom g, Nsbc p, Rates<typename Store<T>::C> r, int gx, int gy, int halo, int steps,
+                    unsigned* flags, int* err) {
+  using C = typename Store<T>::C;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  C* smem = reinterpret_cast<C*>(smem_raw);
+  const int ty = blockIdx.x / gx, tx = blockIdx.x - ty * gx, tid = threadIdx.x;
+  const TileRect t{(int)((unsigned)g.nx * tx / gx), (int)((unsigned)g.ny * ty / gy),
+                   (int)((unsigned)g.nx * (tx + 1) / gx), (int)((unsigned)g.ny * (ty + 1) / gy)};
+  const bool px = p.periodic_x != 0, py = p.periodic_y != 0;
+  const TileRegion reg = tile_region(g.nx, g.ny, px, py, t, halo);
+  const int other = 9 * reg.w * reg.h;
+  const TileHalo halo_of(t, reg);
+  const CellConst<float2> cell = cell_const<MODEL, false, float2>(r, C(Store<T>::kScale));
+  const EdgeList list(t, halo - 1, g.nx, g.ny, px, py);
+  const EdgeSlot slot = edge_slot(list, tid, reg, g, p);
+  // thread k < 9 waits for the neighbour (k % 3 - 1, k / 3 - 1)
+  const unsigned* theirs = nullptr;
+  if (tid < 9 && tid != 4) {
+    int nx = tx + tid % 3 - 1, ny = ty + tid / 3 - 1;
+    if (px) nx = nx < 0 ? gx - 1 : (nx == gx ? 0 : nx);
+    if (py) ny = ny < 0 ? gy - 1 : (ny == gy ? 0 : ny);
+    if (nx >= 0 && nx < gx && ny >= 0 && ny < gy) theirs = flags + (ny * gx + nx) * kFlagStride;
+  }
+  tile_load<T, kTileThreads>(A, g, reg, smem);
+  int at = 0;  // where the newest state is: smem + at
+  for (unsigned round = 1;; ++round) {
+    const int k = min(halo, steps);
+    steps -= k;
+    for (int j = 1; j <= k; ++j) {
+      resident_step<T, MODEL, SHIFT, kTileThreads>(smem + at, smem + (other - at), round & 1 ? B : A, g, p, r, t, reg,
+                                                     k - j, steps == 0 && j == k, halo, cell, list,
+                                                     slot);
+      at = other - at;
+    }
+    if (steps == 0) return;
+    // the block's stores are ordered before the flag by the step's barrier and this fence
+    if (tid == 0) {
+      __threadfence();
+      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flags + blockIdx.x * kFlagStride), "r"(round)
+                   : "memory");
+    }
+    bool late = false;
+    if (theirs) {
+      unsigned seen = 0;
+      const long long t0 = clock64();
+      for (;;) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(theirs) : "memory");
+        if ((int)(seen - round) >= 0) break;
+        if (clock64() - t0 > kTmaWaitCycles) {
+          late = true;
+          break;
+        }
+      }
+    }
+    if (__syncthreads_or(late)) {
+      if (tid == 0) atomicExch(&err[2], 1);
+      return;
+    }
+    tile_halo<T, kTileThreads>(round & 1 ? B : A, g, halo_of, reg, smem + at);
+    __syncthreads();
+  }
+}
+
+// Host: the tiles and the halo of a resident domain, by a model of a round;
+// steps = 0 where the state does not fit the SMs' shared memory.
+inline TilePlan plan_resident(int nx, int ny, bool px, bool py, int sms) {
+  // microseconds: a round's exchange, halo node, step (the boundary's chain of operations), row of 64 nodes,
+  // boundary node (of a corner tile; both lines of a periodic axis)
+  const double t_round = 2.6, t_halo = 0.7e-3, t_step = 0.9, t_row = 0.025, t_edge = 0.01;
+  TilePlan best;
+  for (int halo = 1; halo <= 8; ++halo) {
+    const int side = std::max(4, halo);  // a halo reaches no further than the next tile
+    for (int gx = 1; gx <= sms && nx / gx >= side; ++gx)
+      for (int gy = 1; gx * gy <= sms && ny / gy >= side; ++gy) {
+        const int tw = (nx + gx - 1) / gx, th = (ny + gy - 1) / gy;
+        const int w = px || gx > 2 ? tw + 2 * halo : (gx == 2 ? tw + halo : tw);
+        const int h = py || gy > 2 ? th + 2 * halo : (gy == 2 ? th + halo : th);
+        if ((px && w > nx) || (py && h > ny)) continue;
+        const size_t smem = tile_bytes<float>(w, h) + kRowSlack * sizeof(float);
+        if (smem > kTileRoom) continue;
+        double us = t_round + t_halo * ((double)w * h - (double)tw * th);
+        for (int j = 1; j <= halo; ++j) {
+          const double c = (double)(halo - j) / halo;  // of the halo that step j still covers
+          const double wj = tw + (w - tw) * c, hj = th + (h - th) * c;
+          const double edge = (px || gx == 1 ? 2 : 1) * hj + (py || gy == 1 ? 2 : 1) * wj;
+          us += t_step + t_row * (int)((wj + 63) / 64) * hj + t_edge * edge;
+        }
+        if (us / halo < best.us) best = TilePlan{gx, gy, halo, (int)smem, us / halo};
+      }
+  }
   return best;
 }
 

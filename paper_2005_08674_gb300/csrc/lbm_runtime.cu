@@ -88,8 +88,12 @@ constexpr int kNsbcThreads = 128;
 // where pick_form() draws the lines
 constexpr long long kPassNodes32 = 1200000, kPassNodes16 = 2800000, kTileNodes = 110000, kFusedNodes = 800000;
 constexpr long long kTileCells = 1 << 21;  // largest domain the autotuner tries as tiles
+// steps of a launch of the resident kernel: below, the flags' clearing and the
+// cooperative launch (about 20 us together, against 0.4 us saved per step)
+// outweigh what it saves; the upper bound keeps a launch to some 20 ms
+constexpr int kResidentMin = 64, kResidentMax = 4096;
 
-// How lbm_step launches steps: the bulk and NSBC kernel pair, both in one
+// How lbm_step launches steps, where it does not keep the domain resident: the bulk and NSBC kernel pair, both in one
 // launch, the staged kernel, the multi-step pass, or tiles.
 enum class Form { Pair, Fused, Staged, Pass, Tiles };
 
@@ -139,6 +143,8 @@ struct lbm {
   // tiles (small domains): several steps per launch of tile_kernel
   bool tiles = false;
   int tl_gx = 0, tl_gy = 0, tl_steps = 0, tl_smem = 0;
+  // the domain as resident tiles (resident_kernel): halo 0 where it does not fit
+  int rs_gx = 0, rs_gy = 0, rs_halo = 0, rs_smem = 0;
   // no launch form was asked for: lbm_step takes the one pick_form() names
   bool form_auto = true;
   Form form = Form::Pair;  // what prepare_form() settled on
@@ -562,6 +568,76 @@ void enqueue_macros_rows(const lbm_t* h, double* d_rho, double* d_ux, double* d_
   });
 }
 
+// ---- a domain that stays on chip for many steps ------------------------------
+template <typename T>
+int resident_prepare(lbm_t* h) {
+  h->rs_halo = 0;
+  int coop = 0;
+  LBM_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
+  if (!coop) return LBM_OK;
+  const lbmk::TilePlan p = lbmk::plan_resident(h->nx, h->ny, h->nsbc.periodic_x, h->nsbc.periodic_y,
+                                               std::min(h->sms, kReduceBlocks));
+  if (p.steps == 0) return LBM_OK;
+  cudaError_t e = cudaSuccess;
+  int per_sm = 1;
+  for (const void* k :
+       {(const void*)lbmk::resident_kernel<T, 0, false>, (const void*)lbmk::resident_kernel<T, 0, true>,
+        (const void*)lbmk::resident_kernel<T, 1, false>, (const void*)lbmk::resident_kernel<T, 1, true>}) {
+    int blocks = 0;
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbmk::kTileRoom);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k, lbmk::kTileThreads, p.smem);
+    per_sm = std::min(per_sm, blocks);
+  }
+  if (e != cudaSuccess)
+    return fail(LBM_ECUDA, "resident tiles: %d bytes of shared memory refused: %s", p.smem, cudaGetErrorString(e));
+  if (per_sm < 1) return LBM_OK;
+  h->rs_gx = p.gx;
+  h->rs_gy = p.gy;
+  h->rs_halo = p.steps;
+  h->rs_smem = p.smem;
+  return LBM_OK;
+}
+
+// `steps` steps in one launch, from buffer `from`; the state is then in buffer
+// from ^ (rounds & 1).  The blocks wait for one another: a cooperative launch,
+// which starts all of them or none.  Their flags (zeroed before each launch)
+// lie in the scratch area, which nothing else uses while steps run.
+template <typename T>
+cudaError_t launch_resident(lbm_t* h, int from, int steps, cudaStream_t s) {
+  using C = typename lbmk::Store<T>::C;
+  T *A = static_cast<T*>(h->buf[from]), *B = static_cast<T*>(h->buf[1 - from]);
+  lbmk::Geom g = geom(h);
+  lbmk::Nsbc p = h->nsbc;
+  lbmk::Rates<C> r = rates<C>(h);
+  int gx = h->rs_gx, gy = h->rs_gy, halo = h->rs_halo;
+  unsigned* flags = reinterpret_cast<unsigned*>(scratch_partials(h));
+  int* err = sched(h);
+  cudaError_t e =
+      cudaMemsetAsync(flags, 0, (size_t)gx * gy * lbmk::kFlagStride * sizeof(unsigned), s);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&A, &B, &g, &p, &r, &gx, &gy, &halo, &steps, &flags, &err};
+  with_shift(h, [&](auto zc) {
+    constexpr bool Z = decltype(zc)::value;
+    const void* k = h->collision == 1 ? (const void*)lbmk::resident_kernel<T, 1, Z>
+                                      : (const void*)lbmk::resident_kernel<T, 0, Z>;
+    e = cudaLaunchCooperativeKernel(k, dim3(gx * gy), dim3(lbmk::kTileThreads), args, h->rs_smem, s);
+  });
+  return e;
+}
+
+int enqueue_resident(lbm_t* h, int steps) {
+  cudaError_t e = cudaSuccess;
+  dispatch(h->storage, [&](auto tag) {
+    using T = decltype(tag);
+    if constexpr (!std::is_same<T, double>::value) e = launch_resident<T>(h, h->cur, steps, h->stream);
+  });
+  if (e != cudaSuccess) return fail(LBM_ECUDA, "resident tiles: launch failed: %s", cudaGetErrorString(e));
+  h->cur ^= (steps + h->rs_halo - 1) / h->rs_halo & 1;
+  return LBM_OK;
+}
+
 // The launch form lbm_step takes when none was asked for, by size and storage
 // (microseconds per step on a GB300, BGK):
 //   nodes            200^2   300^2   400^2   600^2  1024^2  1200^2  1700^2  2048^2  4096^2
@@ -604,6 +680,17 @@ int prepare_form(lbm_t* h) {
         rc = pass_prepare<T>(h);
       }
     });
+  h->rs_halo = 0;
+  // above kTileNodes the MRT and the shifted collision cost the tiles' rows what
+  // the launches cost the one-step form (400^2 MRT in a stream, 200 steps: 741
+  // against 730 us), plain BGK does not (613 x 377 f16, 100 steps: 402 against 440)
+  const bool plain = h->collision == 0 && !zshift(h).on;
+  if (rc == LBM_OK && !h->profiling && h->storage != LBM_F64 && tiles_ok(h) &&
+      (plain || (long long)h->nx * h->ny <= kTileNodes) && (h->form_auto ? h->form != Form::Pass : h->form == Form::Tiles))
+    dispatch(h->storage, [&](auto tag) {
+      using T = decltype(tag);
+      if constexpr (!std::is_same<T, double>::value) rc = resident_prepare<T>(h);
+    });
   h->form_ready = rc == LBM_OK;
   return rc;
 }
@@ -643,7 +730,9 @@ void enqueue_step(const lbm_t* h, int from, cudaStream_t s, bool fork) {
       launch_staged<T>(h, a, b, s);
       return;
     }
-    if (h->form == Form::Fused) {
+    // (a step that no graph overlaps: one launch instead of the pair's two in
+    // a row, 9.2 against about 12 us at 1024^2 f32)
+    if (h->form == Form::Fused || (h->form == Form::Pair && h->form_auto && !fork)) {
       launch_fused<T>(h, a, b, s);
       return;
     }
@@ -1019,6 +1108,12 @@ int lbm_step(lbm_t* h, int32_t n) {
   if (rc) return rc;
   const int per = steps_per_launch(h);
   int left = n;
+  while (h->rs_halo && left >= kResidentMin) {
+    const int take = std::min(left, kResidentMax);
+    rc = enqueue_resident(h, take);
+    if (rc) return rc;
+    left -= take;
+  }
   if (!h->profiling && per == 1 && left >= kGraphSteps) {
     if (!h->graph[h->cur]) {
       rc = capture_graph(h, h->cur);
@@ -1475,11 +1570,18 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
     h->tiles = tiles;
     drop_graphs(h);
     if (prepare_form(h) == LBM_OK) {
-      const int per = steps_per_launch(h), launches = std::max(4, reps / per);
-      for (int k = 0; k < 2; ++k) enqueue_launch(h, k & 1, per, h->stream, false);
+      const int cur = h->cur, per = h->rs_halo ? 64 : steps_per_launch(h), launches = h->rs_halo ? 2 : std::max(4, reps / per);
+      auto launch = [&](int k) {
+        if (h->rs_halo)
+          enqueue_resident(h, per);  // (moves h->cur)
+        else
+          enqueue_launch(h, k & 1, per, h->stream, false);
+      };
+      for (int k = 0; k < 2; ++k) launch(k);
       cudaEventRecord(e0, h->stream);
-      for (int k = 0; k < launches; ++k) enqueue_launch(h, k & 1, per, h->stream, false);
+      for (int k = 0; k < launches; ++k) launch(k);
       cudaEventRecord(e1, h->stream);
+      h->cur = cur;
       float ms = 1e30f;
       if (cudaEventSynchronize(e1) == cudaSuccess) {
         cudaEventElapsedTime(&ms, e0, e1);
