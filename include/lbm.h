@@ -139,7 +139,9 @@ int lbm_get_dims(const lbm_t* h, int32_t* nx, int32_t* ny);
 size_t lbm_buffer_bytes(const lbm_t* h);
 
 /* Bytes of the scratch area: three [ny][nx] double fields (macros) plus
- * reduction partials, rounded to 256 bytes. */
+ * reduction partials, rounded to 256 bytes.  Nothing in it is kept from one
+ * call to the next: handles that take turns may share one area, and the
+ * caller may use it between calls (lbm_step does not touch it). */
 size_t lbm_scratch_bytes(const lbm_t* h);
 
 /* Hand the library caller-owned device memory (e.g. from PyTorch): two

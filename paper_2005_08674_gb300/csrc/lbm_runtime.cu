@@ -149,6 +149,10 @@ struct lbm {
   bool form_auto = true;
   Form form = Form::Pair;  // what prepare_form() settled on
   bool form_ready = false;
+  // work counters and the resident tiles' flags: the library's own memory, as
+  // bound scratch areas may be shared by handles or hold the caller's data
+  // between two calls
+  int* d_sync = nullptr;
   bool sched_clear = false;  // the counters have been zeroed
   int4* d_items = nullptr;
   lbmk::InstDev* d_inst = nullptr;
@@ -176,12 +180,14 @@ double* scratch_field(lbm_t* h, int c) {
 }
 double* scratch_partials(lbm_t* h) { return scratch_field(h, 3); }
 double* scratch_out(lbm_t* h) { return scratch_partials(h) + kReduceBlocks * 4; }
-// work counter, warps or blocks done, give-up flag of the kernels that claim
-// work: the last bytes of the area, which its rounding to 256 bytes leaves
-constexpr size_t kScratchTail = (kReduceBlocks * 4 + 4) * sizeof(double);
-static_assert((kScratchTail + 255) / 256 * 256 - kScratchTail >= 16, "no room for the counters");
-int* sched(const lbm_t* h) {
-  return reinterpret_cast<int*>(static_cast<char*>(h->scratch) + lbm_scratch_bytes(h) - 16);
+// d_sync: work counter, warps or blocks done and give-up flag of the kernels
+// that claim work, then the flags of the resident tiles, one per block.
+constexpr size_t kSyncFlags = 256;
+constexpr int kResidentBlocks = 512;
+constexpr size_t kSyncBytes = kSyncFlags + (size_t)kResidentBlocks * lbmk::kFlagStride * sizeof(unsigned);
+int* sched(const lbm_t* h) { return h->d_sync; }
+unsigned* resident_flags(const lbm_t* h) {
+  return reinterpret_cast<unsigned*>(reinterpret_cast<char*>(h->d_sync) + kSyncFlags);
 }
 
 void drop_graphs(lbm_t* h) {
@@ -198,6 +204,7 @@ int ensure_memory(lbm_t* h) {
   if (h->bound) return LBM_OK;
   const size_t bb = lbm_buffer_bytes(h), sb = lbm_scratch_bytes(h);
   LBM_CUDA(cudaGetDevice(&h->device));
+  if (!h->d_sync) LBM_CUDA(cudaMalloc(&h->d_sync, kSyncBytes));
   LBM_CUDA(cudaMalloc(&h->buf[0], bb));
   LBM_CUDA(cudaMalloc(&h->buf[1], bb));
   LBM_CUDA(cudaMalloc(&h->scratch, sb));
@@ -576,7 +583,7 @@ int resident_prepare(lbm_t* h) {
   LBM_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
   if (!coop) return LBM_OK;
   const lbmk::TilePlan p = lbmk::plan_resident(h->nx, h->ny, h->nsbc.periodic_x, h->nsbc.periodic_y,
-                                               std::min(h->sms, kReduceBlocks));
+                                               std::min(h->sms, kResidentBlocks));
   if (p.steps == 0) return LBM_OK;
   cudaError_t e = cudaSuccess;
   int per_sm = 1;
@@ -602,8 +609,7 @@ int resident_prepare(lbm_t* h) {
 
 // `steps` steps in one launch, from buffer `from`; the state is then in buffer
 // from ^ (rounds & 1).  The blocks wait for one another: a cooperative launch,
-// which starts all of them or none.  Their flags (zeroed before each launch)
-// lie in the scratch area, which nothing else uses while steps run.
+// which starts all of them or none.  Their flags are zeroed before each launch.
 template <typename T>
 cudaError_t launch_resident(lbm_t* h, int from, int steps, cudaStream_t s) {
   using C = typename lbmk::Store<T>::C;
@@ -612,7 +618,7 @@ cudaError_t launch_resident(lbm_t* h, int from, int steps, cudaStream_t s) {
   lbmk::Nsbc p = h->nsbc;
   lbmk::Rates<C> r = rates<C>(h);
   int gx = h->rs_gx, gy = h->rs_gy, halo = h->rs_halo;
-  unsigned* flags = reinterpret_cast<unsigned*>(scratch_partials(h));
+  unsigned* flags = resident_flags(h);
   int* err = sched(h);
   cudaError_t e =
       cudaMemsetAsync(flags, 0, (size_t)gx * gy * lbmk::kFlagStride * sizeof(unsigned), s);
@@ -879,6 +885,7 @@ void lbm_destroy(lbm_t* h) {
     cudaFree(h->scratch);
   }
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
+  if (h->d_sync) cudaFree(h->d_sync);
   if (h->d_items) cudaFree(h->d_items);
   if (h->d_inst) cudaFree(h->d_inst);
   if (h->d_shift) cudaFree(h->d_shift);
@@ -1039,6 +1046,7 @@ int lbm_bind(lbm_t* h, void* dev_a, void* dev_b, void* dev_scratch) {
   for (void* p : {dev_a, dev_b, dev_scratch})
     if (reinterpret_cast<uintptr_t>(p) % 256) return fail(LBM_EINVAL, "lbm_bind: pointers must be 256-byte aligned");
   LBM_CUDA(cudaGetDevice(&h->device));
+  if (!h->d_sync) LBM_CUDA(cudaMalloc(&h->d_sync, kSyncBytes));
   h->buf[0] = dev_a;
   h->buf[1] = dev_b;
   h->scratch = dev_scratch;
