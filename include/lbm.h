@@ -289,13 +289,23 @@ int32_t lbm_get_fused(const lbm_t* h);
  * and lbm_set_fused turn it off; lbm_autotune times it against the other
  * forms.  LBM_EINVAL when enabling it on an f64 handle, a handle with a
  * periodic axis or fewer than 8 x 8 nodes.  A bounded wait that gives up makes
- * lbm_status report LBM_ETIMEOUT.  No device memory of its own.
+ * lbm_status report LBM_ETIMEOUT.
  * lbm_get_twostep: 1 if on, 0 if off, LBM_EINVAL for NULL. */
 int lbm_set_twostep(lbm_t* h, int32_t enable);
 int32_t lbm_get_twostep(const lbm_t* h);
-/* LBM_ETIMEOUT if a bounded wait of the staged kernel gave up (the state is
- * then not valid), else LBM_OK; synchronises the stream. */
+/* The steps of the staged form, of a pass and of a resident domain wait, each
+ * wait for a bounded time (about a second), inside their kernels.  After one
+ * that gave up the state is not valid: lbm_status and every other call that
+ * waits for the stream and hands out results (lbm_get_macros,
+ * lbm_get_populations, lbm_save_state, lbm_reduce, lbm_reduce_noalloc) return
+ * LBM_ETIMEOUT until lbm_init*, lbm_set_populations or lbm_load_state sets a
+ * new state; lbm_step and lbm_get_macros_device, which do not wait, cannot
+ * tell.  lbm_status: LBM_ETIMEOUT then, else LBM_OK; synchronises the stream. */
 int lbm_status(lbm_t* h);
+/* SM clock cycles after which the blocks of a resident domain give up waiting
+ * for one another, 0 .. 4e9 (default 2e9, about a second); with 0 a wait that
+ * is not over at the first look gives up.  LBM_EINVAL outside that range. */
+int lbm_set_wait_limit(lbm_t* h, int64_t cycles);
 
 /* Time every compiled bulk launch shape and prefetch distance (as the
  * kernel pair and as the fused one-launch step), the staged kernel with 3 and
@@ -335,7 +345,7 @@ int lbm_tune_cache_stats(int64_t* hits, int64_t* misses);
  * no counterpart; this is a library service.
  * Same arguments, results, synchronisation and return codes as lbm_reduce,
  * and the same kernels, but the partial sums live in a fixed device array
- * inside the library (131,104 bytes, held by every GPU that loads the
+ * inside the library (131,112 bytes, held by every GPU that loads the
  * library until the process exits) instead of the handle's scratch area; the
  * call makes no cudaMalloc, cudaFree or other allocating call.
  * The array holds the partial sums of at most 4096 blocks; the reduction
@@ -475,9 +485,9 @@ int lbm_partition_instances(int32_t count, const int64_t* cells, int32_t ranks, 
 
 /* Failure-detection check of the bounded device-side waits: one block waits
  * on an mbarrier that nothing arrives on (the waits of the shared-memory
- * paths), then on a device counter that nothing increments (the two-step
- * pass's wait for its first-frame chunks); each gives up after budget_cycles
- * SM clock cycles (at most 4e9), and the kernel returns normally.  Returns
+ * paths), then on a flag that nothing raises (the wait of a resident domain's
+ * blocks for one another); each gives up after budget_cycles SM clock cycles
+ * (at most 4e9), and the kernel returns normally.  Returns
  * LBM_ETIMEOUT when both waits gave up (the expected outcome), LBM_OK if
  * either did not, LBM_ECUDA on a CUDA error.  Allocates and frees two ints of
  * device memory; synchronises. */

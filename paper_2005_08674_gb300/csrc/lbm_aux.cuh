@@ -15,15 +15,17 @@ namespace lbmk {
 // (forming it in float measurably changed the 16-bit runs' reflection
 // figures).  The stored value is the deviation from the far-field
 // equilibrium (Shift).  Grid: x over the pitch, blockIdx.y striding over the
-// rows.
+// rows.  sync (null, or with the first rows): the four work counters and
+// flags, zeroed for the steps that follow.
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void init_kernel(T* __restrict__ A, T* __restrict__ A2, Geom g, Shift<double> zd,
                             const double* __restrict__ rho, const double* __restrict__ ux,
-                            const double* __restrict__ uy, int y0, int y1) {
+                            const double* __restrict__ uy, int y0, int y1, int* __restrict__ sync) {
   using S = Store<T>;
   using C = typename S::C;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (sync && x < 4 && blockIdx.y == 0) sync[x] = 0;
   if (x >= g.pitch) return;
   for (int y = y0 + (int)blockIdx.y; y < y1; y += (int)gridDim.y) {
     double e[9];
@@ -181,9 +183,12 @@ __global__ void __launch_bounds__(NT) reduce_kernel(const T* __restrict__ A, Geo
   }
 }
 
+// The sums of the partials, and whether a wait of the steps before gave up
+// (out[4] unless gave_up is null, so that it comes to the host with the sums).
 template <int NT>
 __global__ void __launch_bounds__(NT) reduce_finish(const double* __restrict__ partials, int nblocks,
-                                                    double* __restrict__ out) {
+                                                    double* __restrict__ out, const int* __restrict__ gave_up) {
+  if (gave_up && threadIdx.x == 0) out[4] = *gave_up ? 1.0 : 0.0;
   __shared__ double smem[NT / 32];
   for (int c = 0; c < 4; ++c) {
     double s = 0.0;

@@ -232,8 +232,9 @@ __global__ void __launch_bounds__(BX) batch_step_kernel(const T* __restrict__ A,
 // next tile is in flight while the current one is collided, so the bytes in
 // flight are bounded by shared memory, not by registers.
 // ---------------------------------------------------------------------------
-// A wait on a barrier nothing ever arrives on must give up after its budget;
-// *flag = 1 if it did (the kernel then returns normally), 2 otherwise.
+// A wait on a barrier nothing ever arrives on, then one on a flag that nothing
+// raises (flag[1], zero): each must give up after its budget.  flag[0] = 1 if
+// both did (the kernel then returns normally), 2 otherwise.
 __global__ void wait_selftest_kernel(long long budget, int* flag) {
   __shared__ __align__(8) uint64_t bar;
   if (threadIdx.x == 0) {
@@ -241,7 +242,11 @@ __global__ void wait_selftest_kernel(long long budget, int* flag) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (threadIdx.x == 0) *flag = !mbar_wait(&bar, 0u, budget) ? 1 : 2;
+  if (threadIdx.x == 0) {
+    const bool a = mbar_wait(&bar, 0u, budget);
+    const bool b = lbmk::flag_wait(reinterpret_cast<const unsigned*>(flag + 1), 1u, budget);
+    flag[0] = !a && !b ? 1 : 2;
+  }
 }
 
 // The whole step of every instance in ONE persistent launch: blocks take
@@ -950,7 +955,7 @@ int lbm_batch_init(lbm_batch_t* b, int32_t k, const double* rho, const double* u
     lbmk::init_kernel<T><<<lbmk::rows_grid(d.pitch, d.ny), 256, 0, b->stream>>>(
         static_cast<T*>(b->pool[0]) + d.off, static_cast<T*>(b->pool[1]) + d.off, inst_geom(d),
         lbmk::far_field_shift(d.m0),
-        bscratch(b, 0), bscratch(b, 1), bscratch(b, 2), 0, d.ny);
+        bscratch(b, 0), bscratch(b, 1), bscratch(b, 2), 0, d.ny, nullptr);
   });
   rc = batch_check_launch();
   if (rc) return rc;
@@ -1055,7 +1060,7 @@ int lbm_batch_unstable_nodes(lbm_batch_t* b, int32_t k, int64_t* count) {
         lbmk::shift_as<typename lbmk::Store<T>::C>(lbmk::far_field_shift(d.m0)),
         ref, d.m0[0], d.m0[1], d.m0[2], partials);
   });
-  lbmk::reduce_finish<256><<<1, 256, 0, b->stream>>>(partials, blocks, out);
+  lbmk::reduce_finish<256><<<1, 256, 0, b->stream>>>(partials, blocks, out, nullptr);
   int rc = batch_check_launch();
   if (rc) return rc;
   double h[4];
@@ -1309,9 +1314,9 @@ int lbm_partition_instances(int32_t count, const int64_t* cells, int32_t ranks, 
 int lbm_wait_selftest(int64_t budget_cycles) {
   if (budget_cycles <= 0 || budget_cycles > 4000000000LL)
     return bfail(LBM_EINVAL, "lbm_wait_selftest: budget %lld outside (0, 4e9] cycles", (long long)budget_cycles);
-  int* d = nullptr;
-  BATCH_CUDA(cudaMalloc(&d, sizeof(int)));
-  cudaError_t e = cudaMemset(d, 0, sizeof(int));
+  int* d = nullptr;  // the result, and a flag that stays 0
+  BATCH_CUDA(cudaMalloc(&d, 2 * sizeof(int)));
+  cudaError_t e = cudaMemset(d, 0, 2 * sizeof(int));
   int h = 0;
   if (e == cudaSuccess) {
     wait_selftest_kernel<<<1, 32>>>(budget_cycles, d);

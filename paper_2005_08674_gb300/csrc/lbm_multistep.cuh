@@ -785,29 +785,34 @@ __device__ __forceinline__ bool roll_item(const T* __restrict__ A, T* __restrict
   const CellConst<float2> k = cell_const<MODEL, kPinConst && !SHIFT, float2>(r, float(Store<T>::kScale));
   const T* mine = ring + 2 * lane;
   int slot = 0;
-  auto wait = [&](int sl) {
-    const bool done = mbar_wait(&bar[sl], (phase >> sl) & 1u);
-    phase ^= 1u << sl;
-    if (__all_sync(0xffffffffu, done)) return true;
-    if (lane == 0) atomicExch(&err[2], 1);
-    return false;
-  };
   auto next = [](int sl) { return sl + 1 == R::DEPTH ? 0 : sl + 1; };
   int s = s0;
+  // Row `row` has arrived; else the item ends, once the copies still in flight
+  // into the ring have (or have been waited for as long again).
+  auto wait = [&](int sl, int row) {
+    if (__all_sync(0xffffffffu, mbar_wait(&bar[sl], (phase >> sl) & 1u))) {
+      phase ^= 1u << sl;
+      return true;
+    }
+    if (lane == 0) atomicExch(&err[2], 1);
+    const int last = min(s1, max(s0 + R::DEPTH - 1, row + R::DEPTH - 3));  // newest row staged
+    for (; row <= last; ++row, sl = next(sl)) mbar_wait(&bar[sl], (phase >> sl) & 1u);
+    return false;
+  };
   for (;;) {
     if (K == R::K && s >= s0 + 2 * R::K) {
 #pragma unroll 1
       for (; s < s1; s += 2) {
-        if (!wait(slot)) return false;
+        if (!wait(slot, s)) return false;
         roll_row<true, T, MODEL, SHIFT>(stage, out, g, r, K, x0, s0, s, s1, slot, mine, lo, hi, whole, some, c, k);
         slot = next(slot);
-        if (!wait(slot)) return false;
+        if (!wait(slot, s + 1)) return false;
         roll_row<true, T, MODEL, SHIFT>(stage, out, g, r, K, x0, s0, s + 1, s1, slot, mine, lo, hi, whole, some, c, k);
         slot = next(slot);
       }
     }
     if (s > s1) break;
-    if (!wait(slot)) return false;
+    if (!wait(slot, s)) return false;
     if (s >= s0 + 2)
       roll_row<false, T, MODEL, SHIFT>(stage, out, g, r, K, x0, s0, s, s1, slot, mine, lo, hi, whole, some, c, k);
     slot = next(slot);
@@ -823,7 +828,8 @@ __device__ __forceinline__ bool roll_item(const T* __restrict__ A, T* __restrict
 // band b; items come as all strips of a band side by side, the bands in waves
 // (wave k: bands k, k + n_waves, ...), so that the lines neighbouring strips
 // share and the rows a band restarts on are read from L2.  The last warp out
-// resets the counters.  A wait that gives up sets sched[2].
+// resets the counters.  A warp whose wait gave up sets sched[2] and takes no
+// more items, but counts as out, so the next pass starts from zero again.
 template <typename T, int MODEL, bool SHIFT>
 __global__ void __launch_bounds__(kRollThreads, Roll<T>::BLOCKS)
     pass_kernel(const T* __restrict__ A, T* __restrict__ B, Geom g, Nsbc p, Rates<typename Store<T>::C> r,
@@ -859,7 +865,7 @@ __global__ void __launch_bounds__(kRollThreads, Roll<T>::BLOCKS)
     if (b >= n_bands) continue;
     const int Ya = steps + b * band, Yb = min(Ya + band, g.ny - steps);
     if (Ya >= Yb) continue;
-    if (!roll_item<T, MODEL, SHIFT>(A, B, g, r, steps, strip * R::OUT, Ya, Yb, ring, bar, phase, lane, sched)) return;
+    if (!roll_item<T, MODEL, SHIFT>(A, B, g, r, steps, strip * R::OUT, Ya, Yb, ring, bar, phase, lane, sched)) break;
   }
   if (lane == 0) {
     __threadfence();
@@ -1009,13 +1015,25 @@ __device__ __forceinline__ void tile_halo(const T* B, const Geom& g, const TileH
   }
 }
 
+// Whether *flag reaches `want` before `limit` SM clock cycles have passed (it
+// is looked at once in any case).
+__device__ __forceinline__ bool flag_wait(const unsigned* flag, unsigned want, long long limit) {
+  const long long t0 = clock64();
+  for (;;) {
+    unsigned seen;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
+    if ((int)(seen - want) >= 0) return true;
+    if (clock64() - t0 >= limit) return false;
+  }
+}
+
 // flags[block]: rounds whose outer nodes the block has written (zero at
-// launch).  A wait that gives up sets err[2] and ends its block; so, in turn,
-// do the blocks that wait for it.
+// launch).  A wait that gives up after `limit` cycles sets err[2] and ends its
+// block; so, in turn, do the blocks that wait for it.
 template <typename T, int MODEL, bool SHIFT>
 __global__ void __launch_bounds__(kTileThreads)
     resident_kernel(T* A, T* B, Geom g, Nsbc p, Rates<typename Store<T>::C> r, int gx, int gy, int halo, int steps,
-                    unsigned* flags, int* err) {
+                    unsigned* flags, long long limit, int* err) {
   using C = typename Store<T>::C;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   C* smem = reinterpret_cast<C*>(smem_raw);
@@ -1055,20 +1073,7 @@ __global__ void __launch_bounds__(kTileThreads)
       asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flags + blockIdx.x * kFlagStride), "r"(round)
                    : "memory");
     }
-    bool late = false;
-    if (theirs) {
-      unsigned seen = 0;
-      const long long t0 = clock64();
-      for (;;) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(theirs) : "memory");
-        if ((int)(seen - round) >= 0) break;
-        if (clock64() - t0 > kTmaWaitCycles) {
-          late = true;
-          break;
-        }
-      }
-    }
-    if (__syncthreads_or(late)) {
+    if (__syncthreads_or(theirs && !flag_wait(theirs, round, limit))) {
       if (tid == 0) atomicExch(&err[2], 1);
       return;
     }
@@ -1171,7 +1176,7 @@ __global__ void __launch_bounds__(kRollThreads, Roll<T>::BLOCKS)
     const int Ya = max(w.z, steps), Yb = min(w.w, d.ny - steps);
     if (Ya >= Yb) continue;
     if (!roll_item<T, MODEL, SHIFT>(A + d.off, B + d.off, g, r, steps, w.y, Ya, Yb, ring, bar, phase, lane, sched))
-      return;
+      break;
   }
   if (lane == 0) {
     __threadfence();

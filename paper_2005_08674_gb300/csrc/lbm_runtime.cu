@@ -153,7 +153,8 @@ struct lbm {
   // bound scratch areas may be shared by handles or hold the caller's data
   // between two calls
   int* d_sync = nullptr;
-  bool sched_clear = false;  // the counters have been zeroed
+  bool waited = false;            // steps since the state was set hold bounded waits
+  long long wait_limit = lbmk::kTmaWaitCycles;  // of the resident tiles (lbm_set_wait_limit)
   int4* d_items = nullptr;
   lbmk::InstDev* d_inst = nullptr;
   void* d_shift = nullptr;  // the far field's storage shift in the compute type (staged kernel)
@@ -174,7 +175,7 @@ lbmk::Geom geom(const lbm_t* h) { return lbmk::Geom{h->nx, h->ny, h->pitch, h->p
 
 size_t macro_bytes(const lbm_t* h) { return round_up((size_t)h->nx * h->ny * sizeof(double), 256); }
 
-// scratch layout: rho | ux | uy (each macro_bytes) | partials | out[4]
+// scratch layout: rho | ux | uy (each macro_bytes) | partials | out[5]
 double* scratch_field(lbm_t* h, int c) {
   return reinterpret_cast<double*>(static_cast<char*>(h->scratch) + c * macro_bytes(h));
 }
@@ -217,12 +218,21 @@ int ensure_memory(lbm_t* h) {
   return LBM_OK;
 }
 
-// Zero the work counters once the memory is there (each launch that uses them
-// leaves them at zero).
+// A new state starts from clear work counters and a clear give-up flag, in
+// stream order (lbm_init*: init_kernel does it).
 int clear_sched(lbm_t* h) {
-  if (h->sched_clear) return LBM_OK;
   LBM_CUDA(cudaMemsetAsync(sched(h), 0, 4 * sizeof(int), h->stream));
-  h->sched_clear = true;
+  h->waited = false;
+  return LBM_OK;
+}
+
+// The end of a call that waits for the stream: LBM_ETIMEOUT if a wait of the
+// steps before gave up, the state then not being one.
+int sync_checked(lbm_t* h, cudaStream_t s, const char* who) {
+  int flag = 0;
+  if (h->waited) LBM_CUDA(cudaMemcpyAsync(&flag, sched(h) + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
+  LBM_CUDA(cudaStreamSynchronize(s));
+  if (flag) return fail(LBM_ETIMEOUT, "%s: a bounded wait of a step kernel gave up", who);
   return LBM_OK;
 }
 
@@ -562,7 +572,8 @@ void enqueue_init_rows(const lbm_t* h, const double* d_rho, const double* d_ux, 
   dispatch(h->storage, [&](auto tag) {
     using T = decltype(tag);
     lbmk::init_kernel<T><<<lbmk::rows_grid(h->pitch, y1 - y0), 256, 0, h->stream>>>(
-        static_cast<T*>(h->buf[0]), static_cast<T*>(h->buf[1]), geom(h), zshift(h), d_rho, d_ux, d_uy, y0, y1);
+        static_cast<T*>(h->buf[0]), static_cast<T*>(h->buf[1]), geom(h), zshift(h), d_rho, d_ux, d_uy, y0, y1,
+        y0 == 0 ? sched(h) : nullptr);
   });
 }
 
@@ -619,11 +630,12 @@ cudaError_t launch_resident(lbm_t* h, int from, int steps, cudaStream_t s) {
   lbmk::Rates<C> r = rates<C>(h);
   int gx = h->rs_gx, gy = h->rs_gy, halo = h->rs_halo;
   unsigned* flags = resident_flags(h);
+  long long limit = h->wait_limit;
   int* err = sched(h);
   cudaError_t e =
       cudaMemsetAsync(flags, 0, (size_t)gx * gy * lbmk::kFlagStride * sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
-  void* args[] = {&A, &B, &g, &p, &r, &gx, &gy, &halo, &steps, &flags, &err};
+  void* args[] = {&A, &B, &g, &p, &r, &gx, &gy, &halo, &steps, &flags, &limit, &err};
   with_shift(h, [&](auto zc) {
     constexpr bool Z = decltype(zc)::value;
     const void* k = h->collision == 1 ? (const void*)lbmk::resident_kernel<T, 1, Z>
@@ -640,6 +652,7 @@ int enqueue_resident(lbm_t* h, int steps) {
     if constexpr (!std::is_same<T, double>::value) e = launch_resident<T>(h, h->cur, steps, h->stream);
   });
   if (e != cudaSuccess) return fail(LBM_ECUDA, "resident tiles: launch failed: %s", cudaGetErrorString(e));
+  h->waited = true;
   h->cur ^= (steps + h->rs_halo - 1) / h->rs_halo & 1;
   return LBM_OK;
 }
@@ -1037,7 +1050,7 @@ int lbm_set_stream(lbm_t* h, void* cuda_stream) {
 size_t lbm_buffer_bytes(const lbm_t* h) { return h ? (size_t)9 * h->plane * h->elt : 0; }
 
 size_t lbm_scratch_bytes(const lbm_t* h) {
-  return h ? 3 * macro_bytes(h) + round_up((kReduceBlocks * 4 + 4) * sizeof(double), 256) : 0;
+  return h ? 3 * macro_bytes(h) + round_up((kReduceBlocks * 4 + 5) * sizeof(double), 256) : 0;
 }
 
 int lbm_bind(lbm_t* h, void* dev_a, void* dev_b, void* dev_scratch) {
@@ -1062,8 +1075,7 @@ int lbm_init_device(lbm_t* h, const double* d_rho, const double* d_ux, const dou
   int rc = ensure_memory(h);
   if (rc) return rc;
   h->cur = 0;
-  rc = clear_sched(h);
-  if (rc) return rc;
+  h->waited = false;
   enqueue_init_rows(h, d_rho, d_ux, d_uy, 0, h->ny);
   rc = check_launch();
   if (rc) return rc;
@@ -1078,8 +1090,8 @@ int lbm_init(lbm_t* h, const double* rho, const double* ux, const double* uy) {
   int rc = ensure_memory(h);
   if (rc) return rc;
   rc = ensure_streams(h);
-  if (!rc) rc = clear_sched(h);
   if (rc) return rc;
+  h->waited = false;
   // the copy of row chunk c (side stream, copy engine) overlaps the
   // initialisation of chunk c - 1 (the handle's stream)
   const double* src[3] = {rho, ux, uy};
@@ -1115,6 +1127,7 @@ int lbm_step(lbm_t* h, int32_t n) {
   if (!rc) rc = ensure_staged(h);
   if (rc) return rc;
   const int per = steps_per_launch(h);
+  if (n > 0 && (h->form == Form::Pass || h->form == Form::Staged)) h->waited = true;
   int left = n;
   while (h->rs_halo && left >= kResidentMin) {
     const int take = std::min(left, kResidentMax);
@@ -1206,8 +1219,7 @@ int lbm_get_macros(lbm_t* h, double* rho, double* ux, double* uy) {
   if (rc) return rc;
   LBM_CUDA(cudaEventRecord(h->ev_join, h->side));  // later work on the handle's stream waits for the copies
   LBM_CUDA(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
-  LBM_CUDA(cudaStreamSynchronize(h->side));
-  return LBM_OK;
+  return sync_checked(h, h->side, "lbm_get_macros");
 }
 
 int lbm_get_populations(lbm_t* h, double* f) {
@@ -1225,7 +1237,7 @@ int lbm_get_populations(lbm_t* h, double* f) {
     LBM_CUDA(cudaMemcpyAsync(f + i * n, scratch_field(h, 0), n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     LBM_CUDA(cudaStreamSynchronize(h->stream));
   }
-  return LBM_OK;
+  return sync_checked(h, h->stream, "lbm_get_populations");
 }
 
 int lbm_set_populations(lbm_t* h, const double* f) {
@@ -1287,9 +1299,8 @@ int lbm_save_state(lbm_t* h, void* host, size_t bytes, int64_t* steps) {
   std::memcpy(host, &hd, sizeof hd);
   LBM_CUDA(cudaMemcpyAsync(static_cast<char*>(host) + sizeof hd, h->buf[h->cur], lbm_buffer_bytes(h),
                            cudaMemcpyDeviceToHost, h->stream));
-  LBM_CUDA(cudaStreamSynchronize(h->stream));
   if (steps) *steps = h->steps;
-  return LBM_OK;
+  return sync_checked(h, h->stream, "lbm_save_state");
 }
 
 int lbm_load_state(lbm_t* h, const void* host, size_t bytes) {
@@ -1340,11 +1351,15 @@ int lbm_reduce(lbm_t* h, const double* ref_rho, const double* ref_ux, const doub
         static_cast<const T*>(h->buf[h->cur]), geom(h), lbmk::shift_as<typename lbmk::Store<T>::C>(zshift(h)), ref,
         h->nsbc.m0[0], h->nsbc.m0[1], h->nsbc.m0[2], scratch_partials(h));
   });
-  lbmk::reduce_finish<kReduceThreads><<<1, kReduceThreads, 0, h->stream>>>(scratch_partials(h), blocks, scratch_out(h));
+  lbmk::reduce_finish<kReduceThreads><<<1, kReduceThreads, 0, h->stream>>>(scratch_partials(h), blocks, scratch_out(h),
+                                                                         sched(h) + 2);
   int rc = check_launch();
   if (rc) return rc;
-  LBM_CUDA(cudaMemcpyAsync(out, scratch_out(h), 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  double sums[5];
+  LBM_CUDA(cudaMemcpyAsync(sums, scratch_out(h), sizeof sums, cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(cudaStreamSynchronize(h->stream));
+  std::memcpy(out, sums, 4 * sizeof(double));
+  if (sums[4] != 0.0) return fail(LBM_ETIMEOUT, "lbm_reduce: a bounded wait of a step kernel gave up");
   if (out[3] > 0.0) return fail(LBM_EUNSTABLE, "lbm_reduce: %.0f nodes with non-finite or non-positive density", out[3]);
   return LBM_OK;
 }
@@ -1448,11 +1463,14 @@ int32_t lbm_get_twostep(const lbm_t* h) { return h ? (h->twostep ? 1 : 0) : LBM_
 
 int lbm_status(lbm_t* h) {
   if (!h) return fail(LBM_EINVAL, "lbm_status: NULL handle");
-  if (!h->sched_clear) return LBM_OK;
-  int flag = 0;
-  LBM_CUDA(cudaMemcpyAsync(&flag, sched(h) + 2, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  LBM_CUDA(cudaStreamSynchronize(h->stream));
-  if (flag) return fail(LBM_ETIMEOUT, "lbm_status: a bounded wait of a step kernel gave up");
+  return sync_checked(h, h->stream, "lbm_status");
+}
+
+int lbm_set_wait_limit(lbm_t* h, int64_t cycles) {
+  if (!h) return fail(LBM_EINVAL, "lbm_set_wait_limit: NULL handle");
+  if (cycles < 0 || cycles > 4000000000LL)
+    return fail(LBM_EINVAL, "lbm_set_wait_limit: %lld outside [0, 4e9] cycles", (long long)cycles);
+  h->wait_limit = cycles;
   return LBM_OK;
 }
 
@@ -1664,7 +1682,7 @@ namespace {
 // blocks: the grid is min(ny, kNoAllocMaxBlocks), one block per row up to that.
 constexpr int kNoAllocThreads = kReduceThreads;
 constexpr int kNoAllocMaxBlocks = 4096;
-constexpr int kNoAllocDoubles = kNoAllocMaxBlocks * 4 + 4;  // partials + out[4]: 131,104 bytes
+constexpr int kNoAllocDoubles = kNoAllocMaxBlocks * 4 + 5;  // partials + out[5]: 131,112 bytes
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
 
@@ -1718,11 +1736,14 @@ extern "C" int lbm_reduce_noalloc(lbm_t* h, const double* ref_rho, const double*
         static_cast<const T*>(h->buf[h->cur]), geom(h), lbmk::shift_as<typename lbmk::Store<T>::C>(zshift(h)), ref,
         h->nsbc.m0[0], h->nsbc.m0[1], h->nsbc.m0[2], partials);
   });
-  lbmk::reduce_finish<kNoAllocThreads><<<1, kNoAllocThreads, 0, h->stream>>>(partials, blocks, d_out);
+  lbmk::reduce_finish<kNoAllocThreads><<<1, kNoAllocThreads, 0, h->stream>>>(partials, blocks, d_out, sched(h) + 2);
   rc = check_launch();
   if (rc) return rc;
-  LBM_CUDA(cudaMemcpyAsync(out, d_out, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  double sums[5];
+  LBM_CUDA(cudaMemcpyAsync(sums, d_out, sizeof sums, cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(cudaStreamSynchronize(h->stream));
+  std::memcpy(out, sums, 4 * sizeof(double));
+  if (sums[4] != 0.0) return fail(LBM_ETIMEOUT, "lbm_reduce_noalloc: a bounded wait of a step kernel gave up");
   if (out[3] > 0.0)
     return fail(LBM_EUNSTABLE, "lbm_reduce_noalloc: %.0f nodes with non-finite or non-positive density", out[3]);
   return LBM_OK;

@@ -72,6 +72,7 @@ _SIGS = {
     "lbm_set_twostep": (ctypes.c_int, [_vp, _i32]),
     "lbm_get_twostep": (ctypes.c_int32, [_vp]),
     "lbm_status": (ctypes.c_int, [_vp]),
+    "lbm_set_wait_limit": (ctypes.c_int, [_vp, ctypes.c_int64]),
     "lbm_reduce_noalloc": (ctypes.c_int, [_vp, _vp, _vp, _vp, _i32, _dp]),
     "lbm_set_tune_cache": (ctypes.c_int, [ctypes.c_char_p]),
     "lbm_tune_cache_stats": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]),
@@ -368,6 +369,10 @@ def lbm_get_twostep(h) -> int:
 
 def lbm_status(h):
     return _check(_L.lbm_status(h))
+
+
+def lbm_set_wait_limit(h, cycles: int):
+    return _check(_L.lbm_set_wait_limit(h, int(cycles)))
 
 
 def lbm_profile(h, enable: bool):
