@@ -1463,6 +1463,7 @@ int32_t lbm_get_twostep(const lbm_t* h) { return h ? (h->twostep ? 1 : 0) : LBM_
 
 int lbm_status(lbm_t* h) {
   if (!h) return fail(LBM_EINVAL, "lbm_status: NULL handle");
+  if (!h->initialised) return LBM_OK;  // nothing has run
   return sync_checked(h, h->stream, "lbm_status");
 }
 
