@@ -169,7 +169,10 @@ int lbm_init_device(lbm_t* h, const double* d_rho, const double* d_ux, const dou
  * about 400,000 nodes, 110,000 with MRT or a mean flow) run in one cooperative launch that keeps it there.  All
  * forms give the same bits.  Forms of one step are replayed from a CUDA graph of a
  * fixed number of steps captured on first use (and recaptured after
- * lbm_set_nsbc / lbm_set_stream); everything else is launched directly. */
+ * lbm_set_nsbc / lbm_set_stream); everything else is launched directly.
+ * In a stream that the caller is capturing, after a first step outside it, an
+ * even n leaves the state in the buffer it started from, so that the caller's
+ * graph can be replayed. */
 int lbm_step(lbm_t* h, int32_t n);
 
 /* Number of steps taken since the last lbm_init* / lbm_set_populations. */

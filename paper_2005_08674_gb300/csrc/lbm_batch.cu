@@ -40,6 +40,7 @@
 #include "lbm_tune_cache.h"
 
 int lbm_internal_fail(int code, const char* msg);
+bool lbm_internal_capturing(cudaStream_t s);
 // the autotuner cache of lbm_runtime.cu (lbm_set_tune_cache)
 std::string lbm_internal_tune_path();
 std::string lbm_internal_tune_key(const char* kind, int storage, int model, bool shift,
@@ -983,8 +984,13 @@ int lbm_batch_step(lbm_batch_t* b, int32_t n) {
     rc = build_passes(b);
     if (rc) return rc;
   }
+  // a caller's graph, as in lbm_step: no graph of ours in it, and an even number
+  // of steps leaves the state in its pool
+  const bool captured = lbm_internal_capturing(b->stream);
+  long long launches = passes ? ((long long)n + lbmk::kPassSteps - 1) / lbmk::kPassSteps : n;
+  launches += (launches ^ n) & 1;
   int left = n;
-  if (left >= kBatchGraphSteps) {
+  if (!captured && left >= kBatchGraphSteps) {
     if (!b->graph[b->cur]) {
       cudaGraph_t g = nullptr;
       BATCH_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
@@ -1007,6 +1013,8 @@ int lbm_batch_step(lbm_batch_t* b, int32_t n) {
   while (passes && left >= 2) {
     int take = std::min(lbmk::kPassSteps, left);
     if (left - take == 1 && take > 2) --take;  // five are three and two: a pass takes two steps at least
+    if (captured) take = (int)((left + launches - 1) / launches--);
+    if (take == 1) break;
     enqueue_batch_pass(b, b->cur, take, b->stream);
     b->cur ^= 1;
     left -= take;

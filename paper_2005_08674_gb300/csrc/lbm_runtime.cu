@@ -836,6 +836,22 @@ int enqueue_launch_profiled(lbm_t* h, int from, int steps) {
   return LBM_OK;
 }
 
+}  // namespace
+
+// Shared with the batched mode: the caller is capturing this stream into a
+// graph of its own.
+bool lbm_internal_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (!s) return false;  // the legacy stream cannot be
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return st == cudaStreamCaptureStatusActive;
+}
+
+namespace {
+
 int check_launch() {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LBM_ECUDA, "kernel launch failed: %s", cudaGetErrorString(e));
@@ -1127,15 +1143,22 @@ int lbm_step(lbm_t* h, int32_t n) {
   if (!rc) rc = ensure_staged(h);
   if (rc) return rc;
   const int per = steps_per_launch(h);
+  // A caller's graph is replayed on the buffers it was captured with, so an
+  // even number of steps must leave the state in the buffer it came from, as
+  // single steps do: as many launches as that takes (and none of the graphs
+  // below, which a capture does not take).
+  const bool captured = lbm_internal_capturing(h->stream);
+  long long launches = ((long long)n + per - 1) / per;
+  launches += (launches ^ n) & 1;
   if (n > 0 && (h->form == Form::Pass || h->form == Form::Staged)) h->waited = true;
   int left = n;
-  while (h->rs_halo && left >= kResidentMin) {
+  while (!captured && h->rs_halo && left >= kResidentMin) {
     const int take = std::min(left, kResidentMax);
     rc = enqueue_resident(h, take);
     if (rc) return rc;
     left -= take;
   }
-  if (!h->profiling && per == 1 && left >= kGraphSteps) {
+  if (!captured && !h->profiling && per == 1 && left >= kGraphSteps) {
     if (!h->graph[h->cur]) {
       rc = capture_graph(h, h->cur);
       if (rc) return rc;
@@ -1151,6 +1174,7 @@ int lbm_step(lbm_t* h, int32_t n) {
     if (h->form == Form::Pass && left - take == 1 && take > 2) --take;
     // the last tile launches share what is left evenly
     if (h->form == Form::Tiles) take = (left + (left + per - 1) / per - 1) / ((left + per - 1) / per);
+    if (captured) take = (int)((left + launches - 1) / launches--);
     if (!h->profiling)
       enqueue_launch(h, h->cur, take, h->stream, false);
     else
