@@ -645,12 +645,20 @@ cudaError_t launch_resident(lbm_t* h, int from, int steps, cudaStream_t s) {
   return e;
 }
 
+// Where the launch is refused -- a stream that may use too few SMs for all
+// blocks at once -- the domain is not kept resident any more (rs_halo = 0)
+// until the form is settled anew, and the caller takes the steps otherwise.
 int enqueue_resident(lbm_t* h, int steps) {
   cudaError_t e = cudaSuccess;
   dispatch(h->storage, [&](auto tag) {
     using T = decltype(tag);
     if constexpr (!std::is_same<T, double>::value) e = launch_resident<T>(h, h->cur, steps, h->stream);
   });
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaGetLastError();
+    h->rs_halo = 0;
+    return LBM_OK;
+  }
   if (e != cudaSuccess) return fail(LBM_ECUDA, "resident tiles: launch failed: %s", cudaGetErrorString(e));
   h->waited = true;
   h->cur ^= (steps + h->rs_halo - 1) / h->rs_halo & 1;
@@ -1156,7 +1164,7 @@ int lbm_step(lbm_t* h, int32_t n) {
     const int take = std::min(left, kResidentMax);
     rc = enqueue_resident(h, take);
     if (rc) return rc;
-    left -= take;
+    if (h->rs_halo) left -= take;
   }
   if (!captured && !h->profiling && per == 1 && left >= kGraphSteps) {
     if (!h->graph[h->cur]) {
@@ -1621,14 +1629,17 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
     h->tiles = tiles;
     drop_graphs(h);
     if (prepare_form(h) == LBM_OK) {
-      const int cur = h->cur, per = h->rs_halo ? 64 : steps_per_launch(h), launches = h->rs_halo ? 2 : std::max(4, reps / per);
+      const int cur = h->cur;
+      if (h->rs_halo) enqueue_resident(h, kResidentMin);  // (moves h->cur; finds out whether it is launched at all)
+      const bool resident = h->rs_halo != 0;
+      const int per = resident ? kResidentMin : steps_per_launch(h), launches = resident ? 2 : std::max(4, reps / per);
       auto launch = [&](int k) {
-        if (h->rs_halo)
-          enqueue_resident(h, per);  // (moves h->cur)
+        if (resident)
+          enqueue_resident(h, per);
         else
           enqueue_launch(h, k & 1, per, h->stream, false);
       };
-      for (int k = 0; k < 2; ++k) launch(k);
+      for (int k = 0; k < (resident ? 1 : 2); ++k) launch(k);
       cudaEventRecord(e0, h->stream);
       for (int k = 0; k < launches; ++k) launch(k);
       cudaEventRecord(e1, h->stream);
