@@ -161,7 +161,8 @@ int lbm_init(lbm_t* h, const double* rho, const double* ux, const double* uy);
 int lbm_init_device(lbm_t* h, const double* d_rho, const double* d_ux, const double* d_uy);
 
 /* Advance n >= 0 steps, asynchronously on the stream.  Until lbm_set_launch,
- * lbm_set_fused, lbm_set_staged, lbm_set_twostep or lbm_autotune chooses, the
+ * lbm_set_fused, lbm_set_staged, lbm_set_twostep, lbm_set_tiles or lbm_autotune
+ * chooses, the
  * launch form goes by size and storage: several steps per launch on small
  * domains (tiles in shared memory) and on large ones (the pass of
  * lbm_set_twostep), one launch or the kernel pair per step between; 64 steps
@@ -296,6 +297,25 @@ int32_t lbm_get_fused(const lbm_t* h);
  * lbm_get_twostep: 1 if on, 0 if off, LBM_EINVAL for NULL. */
 int lbm_set_twostep(lbm_t* h, int32_t enable);
 int32_t lbm_get_twostep(const lbm_t* h);
+/* Tiles: several steps per launch of blocks that each hold a tile of the domain
+ * and a halo in shared memory; 64 steps or more of an f32, f16 or bf16 domain
+ * that fits the SMs' shared memory as a whole go out as one cooperative launch
+ * of blocks that exchange halos (the domain stays resident), if the stream
+ * takes it.  Bit-identical to the kernel pair.  enable != 0 turns it on (and
+ * the other forms off); the setters of the other forms turn it off.
+ * LBM_EINVAL when enabling it below 8 x 8 nodes, above 2^21, or where no tiling
+ * fits (very long and narrow domains). */
+int lbm_set_tiles(lbm_t* h, int32_t enable);
+/* How lbm_step launches the next steps, as set, as lbm_autotune chose or as it
+ * picks itself: the form, the most steps one of its launches takes, and the
+ * number of steps in a call from which on the domain stays resident (0: never).
+ * LBM_EINVAL for a NULL argument, LBM_ESTATE before lbm_bind or lbm_init*. */
+#define LBM_FORM_PAIR 0   /* bulk and NSBC kernels */
+#define LBM_FORM_FUSED 1  /* both in one launch (lbm_set_fused) */
+#define LBM_FORM_STAGED 2 /* lbm_set_staged */
+#define LBM_FORM_PASS 3   /* lbm_set_twostep */
+#define LBM_FORM_TILES 4  /* lbm_set_tiles */
+int lbm_get_form(lbm_t* h, int32_t* form, int32_t* steps_per_launch, int32_t* resident_from);
 /* The steps of the staged form, of a pass and of a resident domain wait, each
  * wait for a bounded time (about a second), inside their kernels.  After one
  * that gave up the state is not valid: lbm_status and every other call that
@@ -316,8 +336,7 @@ int lbm_set_wait_limit(lbm_t* h, int64_t cycles);
  * CUDA events on the stream) and keep the fastest; the state is restored
  * afterwards (through a temporary device copy from cudaMallocAsync).  Writes
  * the bulk shape, and the time per step in milliseconds of the winner, to
- * the optional outputs; lbm_get_staged / lbm_get_fused tell whether the
- * staged or the fused form won. */
+ * the optional outputs; lbm_get_form tells which form won. */
 int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_rows, double* ms_per_step);
 
 /* Autotuner cache (a library service; the paper has no counterpart).  With

@@ -95,7 +95,8 @@ constexpr int kResidentMin = 64, kResidentMax = 4096;
 
 // How lbm_step launches steps, where it does not keep the domain resident: the bulk and NSBC kernel pair, both in one
 // launch, the staged kernel, the multi-step pass, or tiles.
-enum class Form { Pair, Fused, Staged, Pass, Tiles };
+enum class Form { Pair = LBM_FORM_PAIR, Fused = LBM_FORM_FUSED, Staged = LBM_FORM_STAGED, Pass = LBM_FORM_PASS,
+                  Tiles = LBM_FORM_TILES };
 
 // launch shapes compiled for the bulk kernel: threads per block along x
 constexpr int kShapesBX[] = {64, 128, 256, 512};
@@ -140,7 +141,7 @@ struct lbm {
   // bands per wave, waves and persistent grid, and the device's SM count
   bool twostep = false;
   int ts_strips = 0, ts_bands = 0, ts_band = 0, ts_wave_bands = 0, ts_waves = 0, ts_grid = 0, sms = 0;
-  // tiles (small domains): several steps per launch of tile_kernel
+  // tiles (lbm_set_tiles; small domains): several steps per launch of tile_kernel
   bool tiles = false;
   int tl_gx = 0, tl_gy = 0, tl_steps = 0, tl_smem = 0;
   // the domain as resident tiles (resident_kernel): halo 0 where it does not fit
@@ -489,10 +490,17 @@ void launch_tiles(const lbm_t* h, const void* a, void* b, int steps, cudaStream_
   });
 }
 
+lbmk::TilePlan tile_plan(const lbm_t* h) {
+  return lbmk::plan_tiles(h->nx, h->ny, h->storage == LBM_F64, h->nsbc.periodic_x, h->nsbc.periodic_y, h->sms);
+}
+
 template <typename T>
 int tiles_prepare(lbm_t* h) {
-  lbmk::TilePlan p = lbmk::plan_tiles(h->nx, h->ny, h->storage == LBM_F64, h->nsbc.periodic_x, h->nsbc.periodic_y, h->sms);
-  if (p.steps == 0) return fail(LBM_EINVAL, "tiles: no plan");
+  const lbmk::TilePlan p = tile_plan(h);
+  if (p.steps == 0) {  // the edges were changed since lbm_set_tiles, and no tiling serves these
+    h->form = Form::Pair;
+    return LBM_OK;
+  }
   h->tl_gx = p.gx;
   h->tl_gy = p.gy;
   h->tl_steps = p.steps;
@@ -682,15 +690,19 @@ Form pick_form(const lbm_t* h) {
   return nodes <= kFusedNodes ? Form::Fused : Form::Pair;
 }
 
+int device_sms(lbm_t* h) {
+  if (h->sms) return LBM_OK;
+  int sms = 0;
+  LBM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+  h->sms = sms;
+  return LBM_OK;
+}
+
 // The form of the next steps, its grid and its kernels' attributes (nothing
 // is allocated).
 int prepare_form(lbm_t* h) {
   if (h->form_ready) return LBM_OK;
-  if (!h->sms) {
-    int sms = 0;
-    LBM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-    h->sms = sms;
-  }
+  if (int rc = device_sms(h)) return rc;
   h->form = h->form_auto ? (h->profiling ? Form::Pair : pick_form(h))
             : h->staged                ? Form::Staged
             : h->fused                 ? Form::Fused
@@ -713,7 +725,8 @@ int prepare_form(lbm_t* h) {
   // against 730 us), plain BGK does not (613 x 377 f16, 100 steps: 402 against 440)
   const bool plain = h->collision == 0 && !zshift(h).on;
   if (rc == LBM_OK && !h->profiling && h->storage != LBM_F64 && tiles_ok(h) &&
-      (plain || (long long)h->nx * h->ny <= kTileNodes) && (h->form_auto ? h->form != Form::Pass : h->form == Form::Tiles))
+      (h->form_auto ? h->form != Form::Pass && (plain || (long long)h->nx * h->ny <= kTileNodes)
+                    : h->form == Form::Tiles))
     dispatch(h->storage, [&](auto tag) {
       using T = decltype(tag);
       if constexpr (!std::is_same<T, double>::value) rc = resident_prepare<T>(h);
@@ -1491,6 +1504,36 @@ int lbm_set_twostep(lbm_t* h, int32_t enable) {
   return LBM_OK;
 }
 
+int lbm_set_tiles(lbm_t* h, int32_t enable) {
+  if (!h) return fail(LBM_EINVAL, "lbm_set_tiles: NULL handle");
+  if (enable) {
+    int rc = device_sms(h);
+    if (rc) return rc;
+    if (!tiles_ok(h) || (long long)h->nx * h->ny > kTileCells || tile_plan(h).steps == 0)
+      return fail(LBM_EINVAL, "lbm_set_tiles: needs 8 x 8 to %lld nodes that tiles in shared memory can cover", kTileCells);
+  }
+  h->tiles = enable != 0;
+  h->form_auto = false;
+  if (h->tiles) {
+    h->staged = 0;
+    h->fused = false;
+    h->twostep = false;
+  }
+  drop_graphs(h);
+  return LBM_OK;
+}
+
+int lbm_get_form(lbm_t* h, int32_t* form, int32_t* steps_per_launch, int32_t* resident_from) {
+  if (!h || !form || !steps_per_launch || !resident_from) return fail(LBM_EINVAL, "lbm_get_form: NULL argument");
+  if (!h->bound) return fail(LBM_ESTATE, "lbm_get_form: no memory yet (lbm_bind or lbm_init first)");
+  int rc = prepare_form(h);
+  if (rc) return rc;
+  *form = (int32_t)h->form;
+  *steps_per_launch = ::steps_per_launch(h);
+  *resident_from = h->rs_halo ? kResidentMin : 0;
+  return LBM_OK;
+}
+
 int32_t lbm_get_twostep(const lbm_t* h) { return h ? (h->twostep ? 1 : 0) : LBM_EINVAL; }
 
 int lbm_status(lbm_t* h) {
@@ -1628,7 +1671,7 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
     h->twostep = !tiles;
     h->tiles = tiles;
     drop_graphs(h);
-    if (prepare_form(h) == LBM_OK) {
+    if (prepare_form(h) == LBM_OK && h->form == (tiles ? Form::Tiles : Form::Pass)) {
       const int cur = h->cur;
       if (h->rs_halo) enqueue_resident(h, kResidentMin);  // (moves h->cur; finds out whether it is launched at all)
       const bool resident = h->rs_halo != 0;

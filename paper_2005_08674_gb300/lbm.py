@@ -72,6 +72,8 @@ _SIGS = {
     "lbm_set_twostep": (ctypes.c_int, [_vp, _i32]),
     "lbm_get_twostep": (ctypes.c_int32, [_vp]),
     "lbm_status": (ctypes.c_int, [_vp]),
+    "lbm_set_tiles": (ctypes.c_int, [_vp, _i32]),
+    "lbm_get_form": (ctypes.c_int, [_vp, _i32p, _i32p, _i32p]),
     "lbm_set_wait_limit": (ctypes.c_int, [_vp, ctypes.c_int64]),
     "lbm_reduce_noalloc": (ctypes.c_int, [_vp, _vp, _vp, _vp, _i32, _dp]),
     "lbm_set_tune_cache": (ctypes.c_int, [ctypes.c_char_p]),
@@ -371,6 +373,20 @@ def lbm_status(h):
     return _check(_L.lbm_status(h))
 
 
+def lbm_set_tiles(h, enable: bool):
+    return _check(_L.lbm_set_tiles(h, int(bool(enable))))
+
+
+FORMS = ("pair", "fused", "staged", "pass", "tiles")
+
+
+def lbm_get_form(h):
+    """(form, most steps per launch, steps of a call from which the domain stays resident or 0)."""
+    form, per, res = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
+    _check(_L.lbm_get_form(h, ctypes.byref(form), ctypes.byref(per), ctypes.byref(res)))
+    return FORMS[form.value], per.value, res.value
+
+
 def lbm_set_wait_limit(h, cycles: int):
     return _check(_L.lbm_set_wait_limit(h, int(cycles)))
 
@@ -546,6 +562,16 @@ class Simulation:
     @property
     def twostep(self) -> bool:
         return lbm_get_twostep(self.h) == 1
+
+    def set_tiles(self, enable=True):
+        """Several steps per launch on tiles in shared memory (see lbm_set_tiles)."""
+        lbm_set_tiles(self.h, enable)
+        return self
+
+    @property
+    def form(self):
+        """(form, most steps per launch, steps from which the domain stays resident): see lbm_get_form."""
+        return lbm_get_form(self.h)
 
     def status(self):
         """Raises LbmError(LBM_ETIMEOUT) if a bounded device-side wait gave up."""

@@ -1,0 +1,95 @@
+"""Each launch form, asked for and known to have run, against the kernel pair bit by
+bit: tiles on every storage (double among them), resident domains, and the form
+lbm_step picks by itself, which lbm_get_form names."""
+import json
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+NSBC = ["nsbc"] * 4
+VELOCITY = [("velocity", 0.03, 0.01), "nsbc", "nsbc", ("velocity", 0.0, -0.02)]
+CHANNEL = [("velocity", 0.05, 0.0), "nsbc", "periodic", "periodic"]
+PERIODIC = ["periodic"] * 4
+SETTINGS = [("bgk", NSBC, (0.0, 0.0), 1, 0), ("mrt", VELOCITY, (0.05, 0.01), 2, 1), ("mrt", CHANNEL, (0.05, 0.0), 1, 0),
+            ("bgk", PERIODIC, (0.0, 0.0), 1, 0)]
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    from paper_2005_08674_gb300 import build
+    build.build()
+    from paper_2005_08674_gb300 import lbm as m
+    return m
+
+
+def _runs(lbm, nx, ny, storage, setting, choose, steps):
+    """Populations of the kernel pair and of the form `choose` asks for, and that form."""
+    model, edges, far, order, corner = setting
+    rng = np.random.default_rng(nx + ny)
+    f = [b + 1e-3 * rng.standard_normal((ny, nx)) for b in (1.0, far[0], far[1])]
+    out = []
+    for pair in (True, False):
+        with lbm.Simulation(nx, ny, 0.6, storage=storage, mrt_rates=(1.4, 1.4, 1.2), farfield_u=far, collision=model,
+                            edges=edges, grad_order=order, corner_mode=corner, beta=0.1) as s:
+            s.init(*f)
+            if pair:
+                s.set_launch(128, 1, 0)
+            else:
+                choose(s)
+            form = s.form
+            for n in steps:
+                s.step(n)
+            s.status()
+            out.append(s.populations())
+    return out[0], out[1], form
+
+
+@pytest.mark.parametrize("nx,ny", [(8, 8), (9, 13), (64, 40), (131, 75), (257, 9), (200, 201)])
+@pytest.mark.parametrize("storage", ["f64", "f32", "f16", "bf16"])
+@pytest.mark.parametrize("setting", SETTINGS)
+def test_tiles_equal_pair(lbm, nx, ny, storage, setting):
+    ref, got, form = _runs(lbm, nx, ny, storage, setting, lambda s: s.set_tiles(), (1, 2, 3, 7, 16, 29))
+    assert form[0] == "tiles" and form[1] >= 1
+    assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("nx,ny", [(8, 8), (17, 200), (128, 128), (401, 399), (500, 610)])
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("setting", SETTINGS)
+def test_resident_tiles_equal_pair(lbm, nx, ny, storage, setting):
+    ref, got, form = _runs(lbm, nx, ny, storage, setting, lambda s: s.set_tiles(), (64, 70, 63, 5))
+    assert form[0] == "tiles" and form[2] == 64
+    assert np.array_equal(got, ref)
+
+
+def test_tiles_refused(lbm):
+    for nx, ny in ((7, 9), (9, 7), (2048, 1025), (65536, 32)):
+        with lbm.Simulation(nx, ny, 0.6) as s:
+            with pytest.raises(lbm.LbmError):
+                s.set_tiles()
+
+
+def test_form_follows_the_setters(lbm):
+    with lbm.Simulation(300, 300, 0.6) as s:
+        for choose, form, per in ((lambda: s.set_launch(128, 1, 0), "pair", 1), (s.set_fused, "fused", 1),
+                                  (lambda: s.set_staged(3), "staged", 1), (s.set_twostep, "pass", 4),
+                                  (lambda: s.set_twostep(False), "pair", 1)):
+            choose()
+            assert s.form == (form, per, 0)
+
+
+def test_forms_in_bounds():
+    """No form of several steps makes an access that the bounds-checked build rejects."""
+    from paper_2005_08674_gb300 import build
+    build.build(check=True)
+    r = subprocess.run([sys.executable, os.path.join(HERE, "checked_forms.py")], capture_output=True, text=True,
+                       timeout=900, env=dict(os.environ, LBM_CHECKED="1"))
+    assert r.returncode == 0, r.stderr[-2000:]
+    out = json.loads(r.stdout.strip().splitlines()[-1])
+    assert out["checked"] and out["rejected"] == 0, out
