@@ -163,12 +163,12 @@ int lbm_init_device(lbm_t* h, const double* d_rho, const double* d_ux, const dou
 /* Advance n >= 0 steps, asynchronously on the stream.  Until lbm_set_launch,
  * lbm_set_fused, lbm_set_staged, lbm_set_twostep, lbm_set_tiles or lbm_autotune
  * chooses, the
- * launch form goes by size and storage: several steps per launch on small
- * domains (tiles in shared memory) and on large ones (the pass of
- * lbm_set_twostep), one launch or the kernel pair per step between; 64 steps
- * or more of a domain whose state fits the SMs' shared memory (f32, f16, bf16;
- * about 400,000 nodes, 110,000 with MRT or a mean flow) run in one cooperative launch that keeps it there.  All
- * forms give the same bits.  Forms of one step are replayed from a CUDA graph of a
+ * launch form goes by size, shape, edges and storage (lbm_get_form names it):
+ * several steps per launch on small domains (tiles in shared memory) and on
+ * large ones (the pass of lbm_set_twostep), one launch or the kernel pair per
+ * step between; 64 steps or more of a domain whose state fits the SMs' shared
+ * memory (f32, f16, bf16; up to about 400,000 nodes) run in one cooperative
+ * launch that keeps it there.  All forms give the same bits.  Forms of one step are replayed from a CUDA graph of a
  * fixed number of steps captured on first use (and recaptured after
  * lbm_set_nsbc / lbm_set_stream); everything else is launched directly.
  * In a stream that the caller is capturing, after a first step outside it, an

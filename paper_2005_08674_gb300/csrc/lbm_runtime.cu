@@ -87,6 +87,8 @@ constexpr int kReduceBlocks = 1216;  // 8 x 152 SMs
 constexpr int kNsbcThreads = 128;
 // where pick_form() draws the lines
 constexpr long long kPassNodes32 = 1200000, kPassNodes16 = 2800000, kTileNodes = 110000, kFusedNodes = 800000;
+constexpr long long kTileNodesEdge = 32000, kTileNodesEdge16 = 20000, kResidentNodesPeriodic = 5000;
+constexpr int kPassRows32 = 80, kPassRows16 = 320;
 constexpr long long kTileCells = 1 << 21;  // largest domain the autotuner tries as tiles
 // steps of a launch of the resident kernel: below, the flags' clearing and the
 // cooperative launch (about 20 us together, against 0.4 us saved per step)
@@ -673,6 +675,33 @@ int enqueue_resident(lbm_t* h, int steps) {
   return LBM_OK;
 }
 
+// A domain several times wider than high: rows are where the forms of one step
+// are at their best and tiles at their worst; and the other way round.
+bool wide(const lbm_t* h) { return h->nx > 4 * h->ny; }
+bool tall(const lbm_t* h) { return h->ny > 4 * h->nx; }
+bool thin_f32(const lbm_t* h) {
+  return h->storage == LBM_F32 && h->nx < 64 && (long long)h->nx * h->ny > kTileNodes;
+}
+
+// Tiles as lbm_step's own choice, against one launch per step.  Tiles compute
+// the nodes on both lines of a periodic axis with the boundary's quads and
+// twice, and hold 16-bit states as floats.  Microseconds a step, tiles / one
+// launch:
+//   open, f32     320^2 2.91 / 2.95  2000 x 50 2.9 / 2.7   6000 x 16 3.7 / 2.8
+//   open, f16     128^2 2.5 / 2.6    200^2 2.9 / 2.6       320^2 3.7 / 3.1
+//   one axis      f32 160^2 2.4 / 2.5, 200^2 2.7 / 2.6     f16 160^2 2.9 / 2.7
+//   both axes     f32 16^2 2.4 / 2.0, 64^2 2.2 / 2.1, 200^2 3.0 / 2.3
+//   tall          f16 100 x 1000 3.6 / 4.2, 8 x 13000 8.7 / 31
+bool tiles_serve(const lbm_t* h) {
+  if (h->storage == LBM_F64 || !tiles_ok(h) || wide(h)) return false;
+  const int axes = (h->nsbc.periodic_x != 0) + (h->nsbc.periodic_y != 0);
+  const long long most = axes == 2   ? 0
+                         : tall(h)   ? kTileNodes
+                         : h->elt == 2 ? (axes ? kTileNodesEdge16 : kTileNodesEdge)
+                                       : (axes ? kTileNodesEdge : kTileNodes);
+  return (long long)h->nx * h->ny <= most;
+}
+
 // The launch form lbm_step takes when none was asked for, by size and storage
 // (microseconds per step on a GB300, BGK):
 //   nodes            200^2   300^2   400^2   600^2  1024^2  1200^2  1700^2  2048^2  4096^2
@@ -682,12 +711,38 @@ int enqueue_resident(lbm_t* h, int steps) {
 //   f16   one launch                  4.0     5.6     7.4    11.0    19.8    28.5     107
 //         pass                        6.8     7.5    11.5    14.3    19.2    23.6      75
 // A pass is a chain of rows, so it needs enough of them to fill the chip; a
-// tile's halo grows with the steps it takes.
+// tile's halo grows with the steps it takes.  The frame of a pass costs a node
+// of the perimeter about 40 times an inner one in f32 (a pass / the pair:
+// 65536 x 20 33 / 18, x 48 42 / 40, x 96 57 / 74, 20000 x 64 15.8 / 12.8,
+// x 100 17.4 / 21.6), more in 16 bits (65536 x 96 62 / 46, x 160 76 / 70,
+// 20000 x 250 35 / 33, 5000 x 600 18.5 / 19.5): wide domains of few rows do
+// without.  Narrow ones of many rows do not: the pair's rows are short there
+// (20 x 65536 f32 43 / 115), and below 64 columns one launch loses to the pair
+// as well where there are enough rows (4 x 40000 f32 56 / 52; in f64 and 16
+// bits it wins, 419 / 377 and 90 / 93).
 Form pick_form(const lbm_t* h) {
   const long long nodes = (long long)h->nx * h->ny;
-  if (pass_ok(h) && nodes >= (h->elt == 4 ? kPassNodes32 : kPassNodes16)) return Form::Pass;
-  if (h->storage != LBM_F64 && tiles_ok(h) && nodes <= kTileNodes) return Form::Tiles;
-  return nodes <= kFusedNodes ? Form::Fused : Form::Pair;
+  const bool f32 = h->elt == 4;
+  if (pass_ok(h) && nodes >= (f32 ? kPassNodes32 : kPassNodes16) &&
+      (h->ny >= (f32 ? kPassRows32 : kPassRows16) || h->ny >= h->nx))
+    return Form::Pass;
+  if (tiles_serve(h)) return Form::Tiles;
+  return nodes <= kFusedNodes && !thin_f32(h) ? Form::Fused : Form::Pair;
+}
+
+// The domain resident as lbm_step's own choice (calls of kResidentMin steps or
+// more), against one launch per step; microseconds a step, resident / one
+// launch:
+//   open, BGK at rest   620^2 f32 4.9 / 5.0   613 x 377 f16 3.4 / 3.7   1200 x 300 f16 4.6 / 4.0
+//   open, otherwise     320^2 MRT f32 3.25 / 3.26, 400^2 3.6 / 3.4   1000 x 100 3.3 / 3.0
+//   one periodic axis   160^2 f32 2.4 / 2.6, 240^2 2.7 / 2.6; MRT 160^2 3.0 / 2.9, 200^2 3.2 / 2.9
+//   both                64^2 1.8 / 2.1, MRT 2.1 / 2.2; 128^2 2.2 / 2.1, MRT 2.7 / 2.2
+bool resident_serves(const lbm_t* h) {
+  const long long nodes = (long long)h->nx * h->ny;
+  const bool plain = h->collision == 0 && !zshift(h).on;
+  const int axes = (h->nsbc.periodic_x != 0) + (h->nsbc.periodic_y != 0);
+  if (axes) return nodes <= (axes == 2 ? kResidentNodesPeriodic : kTileNodesEdge);
+  return nodes <= (wide(h) && !plain ? kTileNodesEdge : kTileNodes) || (plain && !wide(h));
 }
 
 int device_sms(lbm_t* h) {
@@ -720,13 +775,8 @@ int prepare_form(lbm_t* h) {
       }
     });
   h->rs_halo = 0;
-  // above kTileNodes the MRT and the shifted collision cost the tiles' rows what
-  // the launches cost the one-step form (400^2 MRT in a stream, 200 steps: 741
-  // against 730 us), plain BGK does not (613 x 377 f16, 100 steps: 402 against 440)
-  const bool plain = h->collision == 0 && !zshift(h).on;
   if (rc == LBM_OK && !h->profiling && h->storage != LBM_F64 && tiles_ok(h) &&
-      (h->form_auto ? h->form != Form::Pass && (plain || (long long)h->nx * h->ny <= kTileNodes)
-                    : h->form == Form::Tiles))
+      (h->form_auto ? h->form != Form::Pass && resident_serves(h) : h->form == Form::Tiles))
     dispatch(h->storage, [&](auto tag) {
       using T = decltype(tag);
       if constexpr (!std::is_same<T, double>::value) rc = resident_prepare<T>(h);
@@ -772,7 +822,7 @@ void enqueue_step(const lbm_t* h, int from, cudaStream_t s, bool fork) {
     }
     // (a step that no graph overlaps: one launch instead of the pair's two in
     // a row, 9.2 against about 12 us at 1024^2 f32)
-    if (h->form == Form::Fused || (h->form == Form::Pair && h->form_auto && !fork)) {
+    if (h->form == Form::Fused || (h->form == Form::Pair && h->form_auto && !fork && !thin_f32(h))) {
       launch_fused<T>(h, a, b, s);
       return;
     }

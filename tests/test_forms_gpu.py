@@ -93,3 +93,30 @@ def test_forms_in_bounds():
     assert r.returncode == 0, r.stderr[-2000:]
     out = json.loads(r.stdout.strip().splitlines()[-1])
     assert out["checked"] and out["rejected"] == 0, out
+
+
+CASES = [
+    # open squares, one and two periodic axes
+    (128, 128, "f32", "bgk", NSBC, "tiles", True), (300, 300, "f32", "mrt", NSBC, "tiles", True),
+    (300, 300, "f16", "bgk", NSBC, "fused", True), (128, 128, "f32", "mrt", CHANNEL, "tiles", True),
+    (300, 300, "f32", "bgk", CHANNEL, "fused", False), (64, 64, "f32", "bgk", PERIODIC, "fused", True),
+    (300, 300, "f32", "bgk", PERIODIC, "fused", False), (500, 500, "f16", "bgk", PERIODIC, "fused", False),
+    (500, 500, "f32", "bgk", NSBC, "fused", True), (500, 500, "f32", "mrt", NSBC, "fused", False),
+    (200, 200, "f64", "bgk", NSBC, "fused", False),
+    # wide ones of few rows and their transposes
+    (13000, 8, "f32", "bgk", NSBC, "fused", True), (13000, 8, "f32", "mrt", NSBC, "fused", False),
+    (13000, 8, "f16", "bgk", CHANNEL, "fused", False), (8, 13000, "f32", "bgk", NSBC, "tiles", True),
+    (8, 13000, "f16", "bgk", NSBC, "tiles", True), (3, 3, "f32", "bgk", NSBC, "fused", False),
+    (65536, 20, "f32", "bgk", NSBC, "pair", False), (20, 65536, "f32", "bgk", NSBC, "pass", False),
+    (65536, 48, "f16", "bgk", NSBC, "pair", False), (48, 65536, "f16", "bgk", NSBC, "pass", False),
+    (20000, 100, "f32", "bgk", NSBC, "pass", False), (4, 40000, "f32", "bgk", NSBC, "pair", False),
+    # large ones
+    (1024, 1024, "f32", "bgk", NSBC, "pair", False), (1201, 1003, "f32", "bgk", NSBC, "pass", False),
+    (1801, 1600, "f16", "bgk", NSBC, "pass", False), (1500, 1500, "f32", "bgk", CHANNEL, "pair", False)]
+
+
+@pytest.mark.parametrize("nx,ny,storage,model,edges,form,resident", CASES)
+def test_picked_form(lbm, nx, ny, storage, model, edges, form, resident):
+    """The form lbm_step picks by itself: each one where it is the faster."""
+    with lbm.Simulation(nx, ny, 0.6, storage=storage, collision=model, edges=edges) as s:
+        assert s.form[0] == form and (s.form[2] > 0) == resident
