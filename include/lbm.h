@@ -476,13 +476,17 @@ int lbm_batch_set_launch(lbm_batch_t* b, int32_t threads_x, int32_t rows, int32_
  * four steps (graphs of 16 steps), of two or three where fewer are left, and
  * for a lone step one batched step of the launch shape set.  enable != 0 turns
  * it on; lbm_batch_set_launch turns it off; a batch for which neither was
- * called takes passes when it is stored in f32 and has a million nodes or
- * more (lbm_batch_get_twostep then still reports 0).  lbm_batch_autotune times
- * it against the other forms.  LBM_EINVAL when enabling it on f64 storage,
+ * called takes passes when it is stored in f32, has a million nodes or more
+ * and 34 or more to each node of its instances' perimeters
+ * (lbm_batch_get_twostep then still reports 0; lbm_batch_passes tells).
+ * lbm_batch_autotune times it against the other forms.  LBM_EINVAL when enabling it on f64 storage,
  * with a periodic axis, or with an instance smaller than 8 x 8.
  * lbm_batch_get_twostep: 1 on, 0 off, LBM_EINVAL for NULL. */
 int lbm_batch_set_twostep(lbm_batch_t* b, int32_t enable);
 int32_t lbm_batch_get_twostep(const lbm_batch_t* b);
+/* Whether lbm_batch_step takes its next steps in passes, as set or by itself:
+ * 1 or 0, LBM_EINVAL for NULL.  Host-only. */
+int32_t lbm_batch_passes(const lbm_batch_t* b);
 /* Time every compiled tile shape, grid size, prefetch setting and split, the
  * shared-memory paths and the multi-step pass, on the batch's own state
  * (restored afterwards, through a temporary device copy from

@@ -96,6 +96,7 @@ struct lbm_batch {
   std::vector<double> tau;
   long long pool_elems = 0;
   long long cells = 0;
+  long long perimeter = 0;  // nodes of all instances' perimeters, corners twice
   size_t max_cells = 0;
   lbmk::Nsbc nsbc{};
   int collision = 0;
@@ -621,12 +622,23 @@ bool batch_pass_ok(const lbm_batch_t* b) {
 // Whether the next steps are taken in passes: as asked for, else f32 batches
 // of kPassCells nodes or more (us a step, staged / pass: 0.34 M nodes 8.7 /
 // 9.1, 2.1 M 30 / 21, 3.9 M 53 / 37, 13.9 M 157 / 85; f16 13.9 M 95 / 104:
-// the 16-bit pass is bound by instructions, not by the traffic it saves).
-constexpr long long kPassCells = 1000000;
+// the 16-bit pass is bound by instructions, not by the traffic it saves) with
+// kPassInner nodes to each node of a perimeter or more, as a frame's tiles
+// compute every node several times (staged / pass, BGK and MRT, 1.2 .. 2 M
+// nodes: 8^2 at 3.5 to a perimeter node 112 / 348 and 132 / 422, 64^2 at 16
+// 24 / 29 and 26 / 34, 128^2 at 32 20.0 / 20.0 and 21 / 23, uneven ones at
+// 35.5 34 / 27 and 35 / 32, 160^2 at 40 19 / 15 and 20 / 19).
+constexpr long long kPassCells = 1000000, kPassInner = 34;
 bool batch_passes(const lbm_batch_t* b) {
-  const bool want = b->form_auto ? b->storage == LBM_F32 && b->cells >= kPassCells : b->twostep;
+  const bool want = b->form_auto ? b->storage == LBM_F32 && b->cells >= kPassCells &&
+                                       b->cells >= kPassInner * b->perimeter
+                                 : b->twostep;
   return want && batch_pass_ok(b);
 }
+// Two steps left go singly below this size, or with few nodes to the perimeter
+// (us, a pass of two / two staged steps: 1.0 M nodes 31 / 29, 1.2 M in 200^2
+// 39 / 37, 2.0 M in 1000^2 48 / 51, 2.0 M uneven at 35.5 78 / 74).
+constexpr long long kPassOfTwoCells = 1500000, kPassOfTwoInner = 45;
 
 // Work lists of the multi-step pass, largest instance first: rolling items in
 // bands of rows, all strips of a band side by side; frame tiles.  The items
@@ -824,6 +836,7 @@ lbm_batch_t* lbm_batch_create(int32_t count, const lbm_instance_desc* descs, int
     b->inst.push_back(d);
     b->tau.push_back(s.tau);
     b->cells += (long long)s.nx * s.ny;
+    b->perimeter += 2LL * (s.nx + s.ny);
     b->max_cells = std::max(b->max_cells, (size_t)s.nx * s.ny);
   }
   b->pool_elems = off;
@@ -1015,6 +1028,9 @@ int lbm_batch_step(lbm_batch_t* b, int32_t n) {
     if (left - take == 1 && take > 2) --take;  // five are three and two: a pass takes two steps at least
     if (captured) take = (int)((left + launches - 1) / launches--);
     if (take == 1) break;
+    if (take == 2 && !captured && b->form_auto &&
+        (b->cells < kPassOfTwoCells || b->cells < kPassOfTwoInner * b->perimeter))
+      break;
     enqueue_batch_pass(b, b->cur, take, b->stream);
     b->cur ^= 1;
     left -= take;
@@ -1119,6 +1135,8 @@ int lbm_batch_set_twostep(lbm_batch_t* b, int32_t enable) {
   drop_batch_graphs(b);
   return LBM_OK;
 }
+
+int32_t lbm_batch_passes(const lbm_batch_t* b) { return b ? (batch_passes(b) ? 1 : 0) : LBM_EINVAL; }
 
 int32_t lbm_batch_get_twostep(const lbm_batch_t* b) { return b ? (b->twostep ? 1 : 0) : LBM_EINVAL; }
 

@@ -99,6 +99,7 @@ _SIGS = {
     "lbm_batch_autotune": (ctypes.c_int, [_vp, _i32p, _i32p, _i32p, _i32p, _i32p, _i32p, _dp]),
     "lbm_batch_set_twostep": (ctypes.c_int, [_vp, _i32]),
     "lbm_batch_get_twostep": (ctypes.c_int32, [_vp]),
+    "lbm_batch_passes": (ctypes.c_int32, [_vp]),
     "lbm_batch_status": (ctypes.c_int, [_vp]),
     "lbm_wait_selftest": (ctypes.c_int, [ctypes.c_int64]),
     "lbm_partition_instances": (ctypes.c_int, [_i32, ctypes.POINTER(ctypes.c_int64), _i32, _i32p]),
@@ -687,6 +688,10 @@ def lbm_batch_get_twostep(b) -> int:
     return int(_L.lbm_batch_get_twostep(b))
 
 
+def lbm_batch_passes(b) -> int:
+    return int(_L.lbm_batch_passes(b))
+
+
 def lbm_partition_instances(cells, ranks: int):
     """Rank of each instance for a node-balanced split over `ranks` (see lbm.h)."""
     n = len(cells)
@@ -786,3 +791,8 @@ class Batch:
     @property
     def twostep(self) -> bool:
         return lbm_batch_get_twostep(self.b) == 1
+
+    @property
+    def passes(self) -> bool:
+        """Whether the next steps are taken in passes (see lbm_batch_passes)."""
+        return lbm_batch_passes(self.b) == 1
