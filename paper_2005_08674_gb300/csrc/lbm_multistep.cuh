@@ -907,24 +907,37 @@ struct TilePlan {
   double us = 1e30;  // per step
 };
 
+// The largest piece of a side of n nodes in 1 .. most pieces of 4 or more.
+struct TileCuts {
+  int most = 0, size[65];
+  explicit TileCuts(int n) {
+    for (int g = 1; g <= 64 && n / g >= 4; ++g) size[most = g] = (n + g - 1) / g;
+  }
+};
+
 inline TilePlan plan_tiles(int nx, int ny, bool f64, bool px, bool py, int sms) {
   // microseconds, measured: launch, load per node, step, node, boundary node
   const double t_launch = 2.0, t_load = f64 ? 1.4e-3 : 0.7e-3, t_step = f64 ? 0.9 : 0.35;
   const double t_node = f64 ? 15e-3 : 0.45e-3, t_edge = f64 ? 100e-3 : 3e-3;
   const size_t elt = f64 ? 8 : 4, room = kTileRoom;
   TilePlan best;
+  const TileCuts cx(nx), cy(ny);
   for (int steps : {1, 2, 3, 4, 5, 6, 8, 10, 12})
-    for (int gx = 1; gx <= 64 && nx / gx >= 4; ++gx)
-      for (int gy = 1; gy <= 64 && ny / gy >= 4; ++gy) {
-        if (gx * gy > 8 * sms) break;
-        const int tw = (nx + gx - 1) / gx, th = (ny + gy - 1) / gy;
-        const int w = px || gx > 2 ? tw + 2 * steps : (gx == 2 ? tw + steps : tw);
-        const int h = py || gy > 2 ? th + 2 * steps : (gy == 2 ? th + steps : th);
-        if ((px && w > nx) || (py && h > ny)) continue;
+    for (int gx = 1; gx <= cx.most; ++gx) {
+      const int tw = cx.size[gx], w = px || gx > 2 ? tw + 2 * steps : (gx == 2 ? tw + steps : tw);
+      if (px && w > nx) continue;
+      for (int gy = 1, waves = 1; gy <= cy.most && gx * gy <= 8 * sms; ++gy) {
+        while (gx * gy > waves * sms) ++waves;
+        const int th = cy.size[gy], h = py || gy > 2 ? th + 2 * steps : (gy == 2 ? th + steps : th);
+        if (py && h > ny) continue;
         const size_t smem = 2 * 9 * (size_t)w * h * elt;
         if (smem > room) continue;
-        const int waves = (gx * gy + sms - 1) / sms;
         double block = 0.8 + t_load * w * h;
+        // no less than steps on the tile alone: most candidates end here, so that a plan takes microseconds
+        if ((t_launch + waves * (block + steps * (t_step + t_node * tw * th + t_edge * std::max(tw, th)))) *
+                (1.0 - 1e-9) >
+            best.us * steps)
+          continue;
         for (int j = 1; j <= steps; ++j) {
           const double c = (double)(steps - j) / steps;  // of the halo that step j still covers
           const double wj = tw + (w - tw) * c, hj = th + (h - th) * c;
@@ -933,6 +946,7 @@ inline TilePlan plan_tiles(int nx, int ny, bool f64, bool px, bool py, int sms) 
         const double us = (t_launch + waves * block) / steps;
         if (us < best.us) best = TilePlan{gx, gy, steps, (int)smem, us};
       }
+    }
   return best;
 }
 
@@ -1100,6 +1114,9 @@ inline TilePlan plan_resident(int nx, int ny, bool px, bool py, int sms) {
         const size_t smem = tile_bytes<float>(w, h) + kRowSlack * sizeof(float);
         if (smem > kTileRoom) continue;
         double us = t_round + t_halo * ((double)w * h - (double)tw * th);
+        // no less than `halo` steps on the tile alone, as in plan_tiles
+        if ((us + halo * (t_step + t_row * ((tw + 63) / 64) * th + t_edge * (tw + th))) * (1.0 - 1e-9) > best.us * halo)
+          continue;
         for (int j = 1; j <= halo; ++j) {
           const double c = (double)(halo - j) / halo;  // of the halo that step j still covers
           const double wj = tw + (w - tw) * c, hj = th + (h - th) * c;

@@ -151,7 +151,7 @@ struct lbm {
   // no launch form was asked for: lbm_step takes the one pick_form() names
   bool form_auto = true;
   Form form = Form::Pair;  // what prepare_form() settled on
-  bool form_ready = false;
+  bool form_ready = false, rs_ready = false;
   // work counters and the resident tiles' flags: the library's own memory, as
   // bound scratch areas may be shared by handles or hold the caller's data
   // between two calls
@@ -508,9 +508,11 @@ int tiles_prepare(lbm_t* h) {
   h->tl_steps = p.steps;
   h->tl_smem = p.smem;
   cudaError_t e = cudaSuccess;
-  for (const void* k : {(const void*)lbmk::tile_kernel<T, 0, false>, (const void*)lbmk::tile_kernel<T, 0, true>,
-                        (const void*)lbmk::tile_kernel<T, 1, false>, (const void*)lbmk::tile_kernel<T, 1, true>})
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbmk::kTileRoom);
+  with_shift(h, [&](auto zc) {
+    constexpr bool Z = decltype(zc)::value;
+    const void* k = h->collision == 1 ? (const void*)lbmk::tile_kernel<T, 1, Z> : (const void*)lbmk::tile_kernel<T, 0, Z>;
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbmk::kTileRoom);
+  });
   if (e != cudaSuccess)
     return fail(LBM_ECUDA, "tiles: %d bytes of shared memory refused: %s", (int)lbmk::kTileRoom, cudaGetErrorString(e));
   return LBM_OK;
@@ -598,8 +600,17 @@ void enqueue_macros_rows(const lbm_t* h, double* d_rho, double* d_ux, double* d_
 
 // ---- a domain that stays on chip for many steps ------------------------------
 template <typename T>
+const void* resident_kernel_for(const lbm_t* h) {
+  const void* k = nullptr;
+  with_shift(h, [&](auto zc) {
+    constexpr bool Z = decltype(zc)::value;
+    k = h->collision == 1 ? (const void*)lbmk::resident_kernel<T, 1, Z> : (const void*)lbmk::resident_kernel<T, 0, Z>;
+  });
+  return k;
+}
+
+template <typename T>
 int resident_prepare(lbm_t* h) {
-  h->rs_halo = 0;
   int coop = 0;
   LBM_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
   if (!coop) return LBM_OK;
@@ -607,17 +618,10 @@ int resident_prepare(lbm_t* h) {
                                                std::min(h->sms, kResidentBlocks));
   if (p.steps == 0) return LBM_OK;
   cudaError_t e = cudaSuccess;
-  int per_sm = 1;
-  for (const void* k :
-       {(const void*)lbmk::resident_kernel<T, 0, false>, (const void*)lbmk::resident_kernel<T, 0, true>,
-        (const void*)lbmk::resident_kernel<T, 1, false>, (const void*)lbmk::resident_kernel<T, 1, true>}) {
-    int blocks = 0;
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbmk::kTileRoom);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k, lbmk::kTileThreads, p.smem);
-    per_sm = std::min(per_sm, blocks);
-  }
+  int per_sm = 0;
+  const void* k = resident_kernel_for<T>(h);
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lbmk::kTileRoom);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, lbmk::kTileThreads, p.smem);
   if (e != cudaSuccess)
     return fail(LBM_ECUDA, "resident tiles: %d bytes of shared memory refused: %s", p.smem, cudaGetErrorString(e));
   if (per_sm < 1) return LBM_OK;
@@ -646,13 +650,8 @@ cudaError_t launch_resident(lbm_t* h, int from, int steps, cudaStream_t s) {
       cudaMemsetAsync(flags, 0, (size_t)gx * gy * lbmk::kFlagStride * sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
   void* args[] = {&A, &B, &g, &p, &r, &gx, &gy, &halo, &steps, &flags, &limit, &err};
-  with_shift(h, [&](auto zc) {
-    constexpr bool Z = decltype(zc)::value;
-    const void* k = h->collision == 1 ? (const void*)lbmk::resident_kernel<T, 1, Z>
-                                      : (const void*)lbmk::resident_kernel<T, 0, Z>;
-    e = cudaLaunchCooperativeKernel(k, dim3(gx * gy), dim3(lbmk::kTileThreads), args, h->rs_smem, s);
-  });
-  return e;
+  return cudaLaunchCooperativeKernel(resident_kernel_for<T>(h), dim3(gx * gy), dim3(lbmk::kTileThreads), args,
+                                     h->rs_smem, s);
 }
 
 // Where the launch is refused -- a stream that may use too few SMs for all
@@ -775,13 +774,23 @@ int prepare_form(lbm_t* h) {
       }
     });
   h->rs_halo = 0;
-  if (rc == LBM_OK && !h->profiling && h->storage != LBM_F64 && tiles_ok(h) &&
+  h->rs_ready = false;
+  h->form_ready = rc == LBM_OK;
+  return rc;
+}
+
+// Whether the domain can stay resident (rs_halo); settled after the form, when
+// a call first has steps enough for it.
+int prepare_resident(lbm_t* h) {
+  if (h->rs_ready) return LBM_OK;
+  int rc = LBM_OK;
+  if (!h->profiling && h->storage != LBM_F64 && tiles_ok(h) &&
       (h->form_auto ? h->form != Form::Pass && resident_serves(h) : h->form == Form::Tiles))
     dispatch(h->storage, [&](auto tag) {
       using T = decltype(tag);
       if constexpr (!std::is_same<T, double>::value) rc = resident_prepare<T>(h);
     });
-  h->form_ready = rc == LBM_OK;
+  h->rs_ready = rc == LBM_OK;
   return rc;
 }
 
@@ -1211,6 +1220,7 @@ int lbm_step(lbm_t* h, int32_t n) {
   if (!h->initialised) return fail(LBM_ESTATE, "lbm_step: call lbm_init first");
   int rc = ensure_streams(h);
   if (!rc) rc = prepare_form(h);
+  if (!rc && n >= kResidentMin) rc = prepare_resident(h);
   if (!rc) rc = ensure_staged(h);
   if (rc) return rc;
   const int per = steps_per_launch(h);
@@ -1577,6 +1587,7 @@ int lbm_get_form(lbm_t* h, int32_t* form, int32_t* steps_per_launch, int32_t* re
   if (!h || !form || !steps_per_launch || !resident_from) return fail(LBM_EINVAL, "lbm_get_form: NULL argument");
   if (!h->bound) return fail(LBM_ESTATE, "lbm_get_form: no memory yet (lbm_bind or lbm_init first)");
   int rc = prepare_form(h);
+  if (!rc) rc = prepare_resident(h);
   if (rc) return rc;
   *form = (int32_t)h->form;
   *steps_per_launch = ::steps_per_launch(h);
@@ -1721,7 +1732,8 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
     h->twostep = !tiles;
     h->tiles = tiles;
     drop_graphs(h);
-    if (prepare_form(h) == LBM_OK && h->form == (tiles ? Form::Tiles : Form::Pass)) {
+    if (prepare_form(h) == LBM_OK && prepare_resident(h) == LBM_OK &&
+        h->form == (tiles ? Form::Tiles : Form::Pass)) {
       const int cur = h->cur;
       if (h->rs_halo) enqueue_resident(h, kResidentMin);  // (moves h->cur; finds out whether it is launched at all)
       const bool resident = h->rs_halo != 0;
