@@ -156,6 +156,8 @@ struct lbm {
   // bound scratch areas may be shared by handles or hold the caller's data
   // between two calls
   int* d_sync = nullptr;
+  int sync_slot = -1;
+  bool moved = false;  // to another stream, with a state
   bool waited = false;            // steps since the state was set hold bounded waits
   long long wait_limit = lbmk::kTmaWaitCycles;  // of the resident tiles (lbm_set_wait_limit)
   int4* d_items = nullptr;
@@ -185,10 +187,51 @@ double* scratch_field(lbm_t* h, int c) {
 double* scratch_partials(lbm_t* h) { return scratch_field(h, 3); }
 double* scratch_out(lbm_t* h) { return scratch_partials(h) + kReduceBlocks * 4; }
 // d_sync: work counter, warps or blocks done and give-up flag of the kernels
-// that claim work, then the flags of the resident tiles, one per block.
+// that claim work, then the flags of the resident tiles, one per block.  A
+// handle's area is a slot of an array that the library holds on each device
+// (344 KB), as an allocation would cost a new handle's first steps 90 us; more
+// handles than slots have one allocated.  The address is looked up each time:
+// it does not survive a reset of the device.  What an earlier owner left in a
+// slot is cleared with the first state.
 constexpr size_t kSyncFlags = 256;
-constexpr int kResidentBlocks = 512;
+constexpr int kResidentBlocks = 160, kSyncSlots = 64, kSyncDevices = 64;
 constexpr size_t kSyncBytes = kSyncFlags + (size_t)kResidentBlocks * lbmk::kFlagStride * sizeof(unsigned);
+static __device__ __align__(256) unsigned char g_sync_area[kSyncSlots * kSyncBytes];
+std::mutex g_sync_mutex;
+uint64_t g_sync_used[kSyncDevices] = {};
+static_assert(kSyncSlots == 64 && kSyncBytes % 256 == 0, "a bit per slot");
+
+int take_sync(lbm_t* h) {
+  if (h->d_sync) return LBM_OK;
+  if (h->device >= 0 && h->device < kSyncDevices) {
+    void* base = nullptr;
+    LBM_CUDA(cudaGetSymbolAddress(&base, g_sync_area));
+    std::lock_guard<std::mutex> lock(g_sync_mutex);
+    uint64_t& used = g_sync_used[h->device];
+    for (int k = 0; k < kSyncSlots; ++k)
+      if (!(used >> k & 1)) {
+        used |= 1ull << k;
+        h->sync_slot = k;
+        h->d_sync = reinterpret_cast<int*>(static_cast<char*>(base) + k * kSyncBytes);
+        return LBM_OK;
+      }
+  }
+  LBM_CUDA(cudaMalloc(&h->d_sync, kSyncBytes));
+  return LBM_OK;
+}
+
+// (the handle's streams have been waited for)
+void give_sync(lbm_t* h) {
+  if (h->sync_slot >= 0) {
+    std::lock_guard<std::mutex> lock(g_sync_mutex);
+    g_sync_used[h->device] &= ~(1ull << h->sync_slot);
+  } else if (h->d_sync) {
+    cudaFree(h->d_sync);
+  }
+  h->sync_slot = -1;
+  h->d_sync = nullptr;
+}
+
 int* sched(const lbm_t* h) { return h->d_sync; }
 unsigned* resident_flags(const lbm_t* h) {
   return reinterpret_cast<unsigned*>(reinterpret_cast<char*>(h->d_sync) + kSyncFlags);
@@ -208,7 +251,7 @@ int ensure_memory(lbm_t* h) {
   if (h->bound) return LBM_OK;
   const size_t bb = lbm_buffer_bytes(h), sb = lbm_scratch_bytes(h);
   LBM_CUDA(cudaGetDevice(&h->device));
-  if (!h->d_sync) LBM_CUDA(cudaMalloc(&h->d_sync, kSyncBytes));
+  if (int rc = take_sync(h)) return rc;
   LBM_CUDA(cudaMalloc(&h->buf[0], bb));
   LBM_CUDA(cudaMalloc(&h->buf[1], bb));
   LBM_CUDA(cudaMalloc(&h->scratch, sb));
@@ -982,7 +1025,8 @@ lbm_t* lbm_create(int32_t nx, int32_t ny, double tau, double farfield_rho, const
 
 void lbm_destroy(lbm_t* h) {
   if (!h) return;
-  if (h->stream || h->cap) cudaStreamSynchronize(h->stream);
+  if (h->stream || h->cap || h->bound) cudaStreamSynchronize(h->stream);
+  if (h->moved) cudaDeviceSynchronize();  // steps on an earlier stream may still use the handle's slot
   drop_graphs(h);
   if (h->bound) {
     lbmk::check_remove(h->buf[0]);
@@ -994,7 +1038,7 @@ void lbm_destroy(lbm_t* h) {
     cudaFree(h->scratch);
   }
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
-  if (h->d_sync) cudaFree(h->d_sync);
+  give_sync(h);
   if (h->d_items) cudaFree(h->d_items);
   if (h->d_inst) cudaFree(h->d_inst);
   if (h->d_shift) cudaFree(h->d_shift);
@@ -1139,6 +1183,7 @@ int lbm_set_precision(lbm_t* h, int32_t storage) {
 
 int lbm_set_stream(lbm_t* h, void* cuda_stream) {
   if (!h) return fail(LBM_EINVAL, "lbm_set_stream: NULL handle");
+  h->moved |= h->initialised && h->stream != static_cast<cudaStream_t>(cuda_stream);
   h->stream = static_cast<cudaStream_t>(cuda_stream);
   return LBM_OK;
 }
@@ -1155,7 +1200,7 @@ int lbm_bind(lbm_t* h, void* dev_a, void* dev_b, void* dev_scratch) {
   for (void* p : {dev_a, dev_b, dev_scratch})
     if (reinterpret_cast<uintptr_t>(p) % 256) return fail(LBM_EINVAL, "lbm_bind: pointers must be 256-byte aligned");
   LBM_CUDA(cudaGetDevice(&h->device));
-  if (!h->d_sync) LBM_CUDA(cudaMalloc(&h->d_sync, kSyncBytes));
+  if (int rc = take_sync(h)) return rc;
   h->buf[0] = dev_a;
   h->buf[1] = dev_b;
   h->scratch = dev_scratch;
