@@ -907,11 +907,15 @@ struct TilePlan {
   double us = 1e30;  // per step
 };
 
-// The largest piece of a side of n nodes in 1 .. most pieces of 4 or more.
+// The largest piece of a side of n nodes in 1 .. most pieces of 4 or more, and
+// the fewest pieces (from three on) that are no larger than those of g.
 struct TileCuts {
-  int most = 0, size[65];
+  int most = 0, size[65], fewest[65];
   explicit TileCuts(int n) {
-    for (int g = 1; g <= 64 && n / g >= 4; ++g) size[most = g] = (n + g - 1) / g;
+    for (int g = 1; g <= 64 && n / g >= 4; ++g) {
+      size[most = g] = (n + g - 1) / g;
+      fewest[g] = g > 3 && size[g] == size[g - 1] ? fewest[g - 1] : g;
+    }
   }
 };
 
@@ -926,14 +930,21 @@ inline TilePlan plan_tiles(int nx, int ny, bool f64, bool px, bool py, int sms) 
     for (int gx = 1; gx <= cx.most; ++gx) {
       const int tw = cx.size[gx], w = px || gx > 2 ? tw + 2 * steps : (gx == 2 ? tw + steps : tw);
       if (px && w > nx) continue;
-      for (int gy = 1, waves = 1; gy <= cy.most && gx * gy <= 8 * sms; ++gy) {
-        while (gx * gy > waves * sms) ++waves;
+      // From three rows of tiles on, more rows in the same number of waves
+      // cost less: only the fewest rows with the smallest tiles of 1 .. 8
+      // waves can win (a plan then takes tens of microseconds).
+      for (int c = -1; c <= 8; ++c) {
+        const int top = std::min(cy.most, c * sms / gx);
+        if (c > 0 && top < 3) continue;
+        const int gy = c <= 0 ? c + 2 : cy.fewest[top];
+        if (gy > cy.most || gx * gy > 8 * sms) continue;
+        const int waves = (gx * gy + sms - 1) / sms;
         const int th = cy.size[gy], h = py || gy > 2 ? th + 2 * steps : (gy == 2 ? th + steps : th);
         if (py && h > ny) continue;
         const size_t smem = 2 * 9 * (size_t)w * h * elt;
         if (smem > room) continue;
         double block = 0.8 + t_load * w * h;
-        // no less than steps on the tile alone: most candidates end here, so that a plan takes microseconds
+        // no less than steps on the tile alone: most candidates end here
         if ((t_launch + waves * (block + steps * (t_step + t_node * tw * th + t_edge * std::max(tw, th)))) *
                 (1.0 - 1e-9) >
             best.us * steps)
