@@ -138,8 +138,11 @@ __device__ __forceinline__ void bulk_row(const T* __restrict__ A, T* __restrict_
 }
 
 // f32: 64 registers (32 resident warps); at 72 (28 warps), which the compiler
-// takes if left free, a 1024^2 step loses 3 %.
-template <typename T, int BX, int MODEL, bool SHIFT = false>
+// takes if left free, a 1024^2 step loses 3 %.  PF: the L2 prefetch is compiled
+// in; without it the f32 BGK kernel keeps a value in a register that it spills
+// otherwise (us a step of the pair: 1024^2 9.07 -> 8.80, 1400^2 19.9 -> 19.3,
+// 4 x 40000 50.9 -> 46.4).
+template <typename T, int BX, int MODEL, bool SHIFT = false, bool PF = true>
 __global__ void __launch_bounds__(BX, sizeof(T) == 4 && !SHIFT ? 1024 / BX : 0)
     bulk_kernel(const T* __restrict__ A, T* __restrict__ B, Geom g, Rates<typename Store<T>::C> rates, int rows, int pf) {
   constexpr int V = Store<T>::V;
@@ -147,8 +150,9 @@ __global__ void __launch_bounds__(BX, sizeof(T) == 4 && !SHIFT ? 1024 / BX : 0)
   const int x0 = (blockIdx.x * BX + threadIdx.x) * V;
   const int y_begin = 1 + blockIdx.y * rows;
   const int y_end = min(y_begin + rows, g.ny - 1);
-  const unsigned pf_bytes = warp_segment_bytes<T>(g, x0 - lane * V);
-  for (int y = y_begin; y < y_end; ++y) bulk_row<T, MODEL, SHIFT>(A, B, g, rates, y, x0, lane, pf, pf_bytes);
+  const unsigned pf_bytes = PF ? warp_segment_bytes<T>(g, x0 - lane * V) : 0u;
+  for (int y = y_begin; y < y_end; ++y)
+    bulk_row<T, MODEL, SHIFT>(A, B, g, rates, y, x0, lane, PF ? pf : 0, pf_bytes);
 }
 
 // ---------------------------------------------------------------------------

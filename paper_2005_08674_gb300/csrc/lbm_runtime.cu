@@ -328,9 +328,13 @@ void launch_bulk_bx(const lbm_t* h, const void* a, void* b, int rows, cudaStream
   dim3 grid((nvec + BX - 1) / BX, (h->ny - 2 + rows - 1) / rows);
   with_shift(h, [&](auto zc) {
     constexpr bool Z = decltype(zc)::value;
+    constexpr bool PF = !std::is_same<T, float>::value || Z;  // without the prefetch: f32 at rest
     if (h->collision == 1)
       lbmk::bulk_kernel<T, BX, 1, Z><<<grid, BX, 0, s>>>(static_cast<const T*>(a), static_cast<T*>(b), geom(h),
                                                         rates<C>(h), rows, h->pf);
+    else if (h->pf == 0)
+      lbmk::bulk_kernel<T, BX, 0, Z, PF><<<grid, BX, 0, s>>>(static_cast<const T*>(a), static_cast<T*>(b), geom(h),
+                                                            rates<C>(h), rows, 0);
     else
       lbmk::bulk_kernel<T, BX, 0, Z><<<grid, BX, 0, s>>>(static_cast<const T*>(a), static_cast<T*>(b), geom(h),
                                                         rates<C>(h), rows, h->pf);
@@ -760,8 +764,8 @@ bool tiles_serve(const lbm_t* h) {
 // 20000 x 250 35 / 33, 5000 x 600 18.5 / 19.5): wide domains of few rows do
 // without.  Narrow ones of many rows do not: the pair's rows are short there
 // (20 x 65536 f32 43 / 115), and below 64 columns one launch loses to the pair
-// as well where there are enough rows (4 x 40000 f32 56 / 52; in f64 and 16
-// bits it wins, 419 / 377 and 90 / 93).
+// as well where there are enough rows (one launch / the pair, 4 x 40000: f32
+// 57 / 46; in f64 and 16 bits it wins, 377 / 418 and 90 / 93).
 Form pick_form(const lbm_t* h) {
   const long long nodes = (long long)h->nx * h->ny;
   const bool f32 = h->elt == 4;

@@ -120,3 +120,15 @@ def test_picked_form(lbm, nx, ny, storage, model, edges, form, resident):
     """The form lbm_step picks by itself: each one where it is the faster."""
     with lbm.Simulation(nx, ny, 0.6, storage=storage, collision=model, edges=edges) as s:
         assert s.form[0] == form and (s.form[2] > 0) == resident
+
+
+@pytest.mark.parametrize("bx", [64, 128, 256, 512])
+@pytest.mark.parametrize("nx,ny", [(3, 3), (5, 7), (257, 9), (131, 75), (517, 40)])
+def test_pair_with_and_without_prefetch(lbm, nx, ny, bx):
+    """f32 at rest: the bulk kernel that holds no prefetch against the one that does."""
+    out = []
+    for pf in (0, 1):
+        ref, got, form = _runs(lbm, nx, ny, "f32", SETTINGS[0], lambda s: s.set_launch(bx, 2, pf), (1, 16))
+        assert form[0] == "pair"
+        out += [ref, got]
+    assert all(np.array_equal(out[0], a) for a in out[1:])
