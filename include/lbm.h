@@ -519,11 +519,12 @@ int lbm_partition_instances(int32_t count, const int64_t* cells, int32_t ranks, 
  * device memory; synchronises. */
 int lbm_wait_selftest(int64_t budget_cycles);
 
-/* Per-launch timing.  While enabled, lbm_step launches every step directly
- * (no graph) on the handle's stream with CUDA events around the bulk
- * stream-collide kernel and around the NSBC kernel, which then run one after
- * the other (with the staged kernel: around its one launch per step, counted
- * as the bulk kernel).  lbm_profile resets the record. */
+/* Per-launch timing.  While enabled, lbm_step launches its steps directly (no
+ * graph) on the handle's stream, in the form it uses otherwise (lbm_get_form),
+ * with CUDA events around each launch.  The launches of every form but the
+ * kernel pair -- of one step or of several -- count as bulk launches; the
+ * pair's two kernels run one after the other and count apart.  lbm_profile
+ * resets the record. */
 int lbm_profile(lbm_t* h, int32_t enable);
 
 /* Read and reset the record (synchronises): out[0] = total bulk-kernel

@@ -804,7 +804,7 @@ int device_sms(lbm_t* h) {
 int prepare_form(lbm_t* h) {
   if (h->form_ready) return LBM_OK;
   if (int rc = device_sms(h)) return rc;
-  h->form = h->form_auto ? (h->profiling ? Form::Pair : pick_form(h))
+  h->form = h->form_auto             ? pick_form(h)
             : h->staged                ? Form::Staged
             : h->fused                 ? Form::Fused
             : h->twostep && pass_ok(h) ? Form::Pass
@@ -831,7 +831,7 @@ int prepare_form(lbm_t* h) {
 int prepare_resident(lbm_t* h) {
   if (h->rs_ready) return LBM_OK;
   int rc = LBM_OK;
-  if (!h->profiling && h->storage != LBM_F64 && tiles_ok(h) &&
+  if (h->storage != LBM_F64 && tiles_ok(h) &&
       (h->form_auto ? h->form != Form::Pass && resident_serves(h) : h->form == Form::Tiles))
     dispatch(h->storage, [&](auto tag) {
       using T = decltype(tag);
@@ -928,7 +928,7 @@ int enqueue_step_profiled(lbm_t* h, int from) {
   const void* a = h->buf[from];
   void* b = h->buf[1 - from];
   cudaEvent_t e[4];
-  const bool one = h->staged || h->fused;  // one launch per step
+  const bool one = h->staged || h->form == Form::Fused;  // one launch per step
   int rc = profiled_pair(h, 0, e);
   if (!rc && !one) rc = profiled_pair(h, 1, e + 2);
   if (rc) return rc;
@@ -937,7 +937,7 @@ int enqueue_step_profiled(lbm_t* h, int from) {
     cudaEventRecord(e[0], h->stream);
     if (h->staged)
       launch_staged<T>(h, a, b, h->stream);
-    else if (h->fused)
+    else if (one)
       launch_fused<T>(h, a, b, h->stream);
     else
       launch_bulk<T>(h, a, b, h->bx, h->rows, h->stream);
@@ -1284,9 +1284,19 @@ int lbm_step(lbm_t* h, int32_t n) {
   int left = n;
   while (!captured && h->rs_halo && left >= kResidentMin) {
     const int take = std::min(left, kResidentMax);
+    cudaEvent_t e[2];
+    if (h->profiling) {
+      rc = profiled_pair(h, 0, e);
+      if (rc) return rc;
+      cudaEventRecord(e[0], h->stream);
+    }
     rc = enqueue_resident(h, take);
     if (rc) return rc;
-    if (h->rs_halo) left -= take;
+    if (h->profiling) cudaEventRecord(e[1], h->stream);
+    if (h->rs_halo)
+      left -= take;
+    else if (h->profiling)
+      h->ev_used -= 2;  // refused: nothing was launched between the two
   }
   if (!captured && !h->profiling && per == 1 && left >= kGraphSteps) {
     if (!h->graph[h->cur]) {
@@ -1308,7 +1318,8 @@ int lbm_step(lbm_t* h, int32_t n) {
     if (!h->profiling)
       enqueue_launch(h, h->cur, take, h->stream, false);
     else
-      rc = take > 1 ? enqueue_launch_profiled(h, h->cur, take) : enqueue_step_profiled(h, h->cur);
+      rc = take > 1 || h->form == Form::Tiles ? enqueue_launch_profiled(h, h->cur, take)
+                                              : enqueue_step_profiled(h, h->cur);
     if (rc) return rc;
     h->cur ^= 1;
     left -= take;
@@ -1521,7 +1532,6 @@ int lbm_reduce(lbm_t* h, const double* ref_rho, const double* ref_ux, const doub
 int lbm_profile(lbm_t* h, int32_t enable) {
   if (!h) return fail(LBM_EINVAL, "lbm_profile: NULL handle");
   h->profiling = enable != 0;
-  drop_graphs(h);  // the form lbm_step picks by itself depends on it
   h->ev_used = 0;
   return LBM_OK;
 }
@@ -1701,8 +1711,7 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
   float best = 1e30f;
   int best_bx = h->bx, best_rows = h->rows, best_pf = h->pf, best_staged = h->staged;
   bool best_fused = h->fused, best_twostep = false, best_tiles = false;
-  const bool profiling = h->profiling;
-  h->twostep = h->tiles = h->form_auto = h->profiling = false;
+  h->twostep = h->tiles = h->form_auto = false;
   // whole steps as the graphs run them (NSBC kernel on the forked branch)
   auto time_steps = [&]() -> float {
     h->form_ready = false;
@@ -1821,7 +1830,6 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
   h->fused = best_fused && !best_staged;
   h->twostep = best_twostep;
   h->tiles = best_tiles;
-  h->profiling = profiling;
   drop_graphs(h);
   LBM_CUDA(cudaMemcpyAsync(h->buf[h->cur], backup, bb, cudaMemcpyDeviceToDevice, h->stream));
   LBM_CUDA(cudaFreeAsync(backup, h->stream));
