@@ -1,11 +1,11 @@
 #!/usr/bin/env python
 """D2Q9 + NSBC throughput on one GB300: MLUPS and the HBM roofline.
 
-One "step" is one lattice-Boltzmann time step of the whole domain: either
-the staged step kernel (one producer/consumer launch: interior tiles staged
-into shared memory by bulk copies, and the NSBC perimeter chunks) or the fused
-pull-stream + BGK collide kernel over the interior with the NSBC kernel over
-the perimeter beside it, whichever the autotuner finds faster.  Default workload: 8192 x 8192 nodes, tau 0.55, four Gaussian
+One "step" is one lattice-Boltzmann time step of the whole domain, launched in
+the form that the autotuner finds fastest: several steps per launch (a pass
+over strips and frame tiles, or tiles in shared memory) or one (the staged
+producer/consumer kernel, the fused kernel, or the bulk kernel over the
+interior with the NSBC kernel over the perimeter beside it).  Default workload: 8192 x 8192 nodes, tau 0.55, four Gaussian
 acoustic pulses (amplitude 1e-3, half-width 64) at seeded centres, NSBC on
 all four edges, FP32 shifted storage.
 
@@ -31,9 +31,9 @@ sys.path.insert(0, ROOT)
 
 METRIC = "D2Q9+NSBC MLUPS"
 UNIT = "MLUPS"
-PASS_STEPS = 4  # time steps of one launch of the multi-step pass
 BYTES_PER_CELL = {"f64": 144, "f32": 72, "f16": 36, "bf16": 36}
 CPU_SAMPLE_N = 2048
+E2E_JOBS = 5
 
 
 def parse():
@@ -151,22 +151,32 @@ def kernel_source_sha() -> str:
     return h.hexdigest()[:16]
 
 
-def step_kernel(sim, nx, ny):
+RESIDENT_MAX = 4096  # most steps of one launch of a resident domain
+
+
+def step_kernel(sim, nx, ny, steps):
     """(kernel description, traffic summary file stem, nodes whose state one
-    timed launch reads and writes once) of the kernel that carries the step:
-    the staged kernel updates every node, the bulk kernel the interior (the
-    NSBC kernel the perimeter, beside it); a multi-step pass moves every
-    node's state once for four steps (one launch)."""
-    if sim.twostep:
-        return ("multi-step pass: pass_kernel, one launch per four steps (the nodes at distance 4 or more by warps "
-                "rolling down 64-column strips with the steps in between in registers, the frame as tiles in "
-                "shared memory)", "multistep_traffic", nx * ny)
-    if sim.staged:
+    timed launch reads and writes once, launches that `steps` steps take) of
+    the kernel that carries the step: the bulk kernel updates the interior (the
+    NSBC kernel the perimeter, beside it: two launches a step), every other
+    form all nodes; a launch of several steps moves each node's state once."""
+    form, per, resident_from = sim.form
+    if resident_from and steps >= resident_from:
+        return ("resident_kernel (the domain in shared memory for all steps of a call)", "resident_traffic", nx * ny,
+                -(-steps // RESIDENT_MAX))
+    launches = -(-steps // per)
+    if form == "pass":
+        return (f"multi-step pass: pass_kernel, one launch per {per} steps (the nodes at distance {per} or more by "
+                "warps rolling down 64-column strips with the steps in between in registers, the frame as tiles in "
+                "shared memory)", "multistep_traffic", nx * ny, launches)
+    if form == "tiles":
+        return (f"tile_kernel (tiles in shared memory, {per} steps per launch)", "tile_traffic", nx * ny, launches)
+    if form == "staged":
         return ("batch_ws_kernel (staged step: interior tiles by bulk copies + NSBC chunks, "
-                f"{sim.staged} stages)", "staged_step_traffic", nx * ny)
-    if sim.fused:
-        return "fused_step_kernel (bulk rows + NSBC quads in one launch)", "fused_step_traffic", nx * ny
-    return "bulk_kernel (fused pull-stream + BGK collide)", "bulk_kernel_traffic", (nx - 2) * (ny - 2)
+                f"{sim.staged} stages)", "staged_step_traffic", nx * ny, launches)
+    if form == "fused":
+        return "fused_step_kernel (bulk rows + NSBC quads in one launch)", "fused_step_traffic", nx * ny, launches
+    return ("bulk_kernel (fused pull-stream + BGK collide)", "bulk_kernel_traffic", (nx - 2) * (ny - 2), 2 * launches)
 
 
 def profiled_traffic(stem: str, storage: str, cells: int):
@@ -252,7 +262,7 @@ def aggregate_mlups(cells_per_rank: int, steps: int, ms_max: float, world: int) 
 
 def batch_what(count: int = 256) -> str:
     return (f"{count} instances 64..1024 per side, tau 0.51..0.8, pulses and vortices, "
-            "one persistent launch per step replayed from a CUDA graph")
+            "one launch per step, or per pass of four steps, replayed from a CUDA graph")
 
 
 def shard(cells, rank: int, world: int, partition):
@@ -431,7 +441,8 @@ def run_ours(args, rank, world, local_rank):
     bulk_avg = bulk_ms / max(nb, 1)
     nsbc_avg = nsbc_ms / max(nn, 1)
     peak, peak_kind = measured_peak_gbs()
-    kname, kstem, kcells = step_kernel(sim, w.nx, w.ny)
+    kname, kstem, kcells, _ = step_kernel(sim, w.nx, w.ny, kprof)
+    launches = step_kernel(sim, w.nx, w.ny, args.steps)[3]
     alg_bytes = BYTES_PER_CELL[args.storage] * kcells
     achieved = alg_bytes / (bulk_avg * 1e-3) / 1e9
     traffic = profiled_traffic(kstem, args.storage, kcells)
@@ -443,7 +454,7 @@ def run_ours(args, rank, world, local_rank):
             "warmup": args.warmup, "ms_per_step": ms_max / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": args.storage, "data": "synthetic",
             "config": {"workload": describe(w, args.storage), "nx": w.nx, "ny": w.ny,
-                       "step_kernel": ({"twostep": True} if sim.twostep else
+                       "step_kernel": ({sim.form[0]: True} if sim.form[0] in ("pass", "tiles") else
                                        {"staged_stages": sim.staged} if sim.staged else
                                        {"bulk_threads_x": bx, "bulk_rows": rows, "prefetch_rows": pf,
                                         "fused": sim.fused}),
@@ -459,12 +470,11 @@ def run_ours(args, rank, world, local_rank):
                          "dram_frac": traffic / (bulk_avg * 1e-3) / 1e9 / peak if traffic else None,
                          "kernel": kname,
                          "bytes_per_cell": BYTES_PER_CELL[args.storage], "cells_per_launch": kcells,
-                         "steps_per_launch": PASS_STEPS if sim.twostep else 1,
+                         "steps_per_launch": kprof / max(nb, 1),
                          "avg_launch_ms": bulk_avg, "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)",
                          "nsbc_avg_launch_ms": nsbc_avg if nn else None,
                          "timing": f"per-launch CUDA events over {kprof} steps after the timed region"},
-            "gpu_launches": (-(-args.steps // PASS_STEPS) if sim.twostep else
-                             (1 if sim.staged or sim.fused else 2) * args.steps),
+            "gpu_launches": launches,
             "clocks": clk,
         }
 
@@ -477,22 +487,25 @@ def run_ours(args, rank, world, local_rank):
             t.numpy()[...] = 0.0  # the result buffers exist (and are touched) before the job, like the inputs
         host_in = [t.numpy() for t in pinned[:3]]
         host_out = [t.numpy() for t in pinned[3:]]
-        barrier()
-        t0 = time.perf_counter()
-        lbm.lbm_init(sim.h, *host_in)
-        lbm.lbm_step(sim.h, args.steps)
-        lbm.lbm_get_macros(sim.h, *host_out)
-        t1 = time.perf_counter()
-        barrier()
-        e2e_s = t1 - t0
-        if dist:
-            e2e_s = max_over_ranks(e2e_s, "cuda")
+        # the median of five such jobs: the host link's rate swings by a factor of two and more from job to job
+        jobs = []
+        for _ in range(E2E_JOBS):
+            barrier()
+            t0 = time.perf_counter()
+            lbm.lbm_init(sim.h, *host_in)
+            lbm.lbm_step(sim.h, args.steps)
+            lbm.lbm_get_macros(sim.h, *host_out)
+            t1 = time.perf_counter()
+            barrier()
+            jobs.append(max_over_ranks(t1 - t0, "cuda") if dist else t1 - t0)
+        e2e_s = sorted(jobs)[E2E_JOBS // 2]
         if line is not None:
             nbytes = 3 * cells * 8
             line["e2e"] = {"value": world * cells * args.steps / e2e_s / 1e6, "unit": UNIT,
                            "h2d_bytes_per_step": nbytes / args.steps, "d2h_bytes_per_step": nbytes / args.steps,
-                           "what": "lbm_init (host fields) + lbm_step(steps) + lbm_get_macros (host), wall clock",
-                           "seconds": e2e_s}
+                           "what": "lbm_init (host fields) + lbm_step(steps) + lbm_get_macros (host), wall clock, "
+                                   f"median of {E2E_JOBS} jobs",
+                           "seconds": e2e_s, "seconds_each": jobs}
         del pinned, host_in, host_out
     sim.close()
     del sim
@@ -521,11 +534,11 @@ def run_ours(args, rank, world, local_rank):
             s2.step(min(vsteps, 200))
             bms, bn, _, _ = lbm.lbm_profile_read(s2.h)
             bavg = bms / max(bn, 1)
-            vname, _, vcells = step_kernel(s2, w.nx, w.ny)
+            vname, _, vcells, _ = step_kernel(s2, w.nx, w.ny, min(vsteps, 200))
             gbs = BYTES_PER_CELL[st] * vcells / (bavg * 1e-3) / 1e9
             variants[st] = {"mlups": world * cells * vsteps / (vms * 1e-3) / 1e6, "steps": vsteps,
                             "kernel_gbs": gbs, "kernel_frac": gbs / peak, "kernel": vname,
-                            "bulk_launch": None if (s2.staged or s2.twostep) else [vb, vr, vp]}
+                            "bulk_launch": [vb, vr, vp] if s2.form[0] in ("pair", "fused") else None}
             s2.close()
             del s2
             torch.cuda.empty_cache()
@@ -573,8 +586,7 @@ def run_ours(args, rank, world, local_rank):
             vms = a0.elapsed_time(a1)
             mlups = world * wn.cells * nsteps / (vms * 1e-3) / 1e6
             sizes[f"pulse-{n}"] = {"mlups": mlups, "steps": nsteps, "frac_of_72B_roofline": mlups * 1e6 * 72 / 1e9 / peak,
-                                   "step_kernel": ("twostep" if s4.twostep else f"staged {s4.staged}" if s4.staged
-                                                   else "fused" if s4.fused else "bulk + NSBC pair"),
+                                   "step_kernel": s4.form[0], "resident_from": s4.form[2],
                                    "mb_per_buffer": lbm.lbm_buffer_bytes(s4.h) / 1e6}
             s4.close()
             del s4
