@@ -764,7 +764,10 @@ struct Nsbc {
     kappa = kappa_;
     corner = corner_;
     order = order_;
+    // (settings past the range of float at its end: an infinity would make 0 of a uniform state a NaN)
     auto pair = [](double v) {
+      constexpr double most = 3.4028234663852886e38;
+      v = v > most ? most : (v < -most ? -most : v);
       const float h = (float)v;
       return FloatPair{h, (float)(v - (double)h)};
     };
