@@ -548,7 +548,6 @@ struct Roll {
   static constexpr size_t kSmem = kRing > kTile ? kRing : kTile;
 };
 constexpr int kRollThreads = 32 * 4;
-constexpr bool kPinConst = true;
 
 // this lane's two values of one population at columns 2 lane, 2 lane + 1 of
 // a staged row, in stored units
@@ -782,7 +781,7 @@ __device__ __forceinline__ bool roll_item(const T* __restrict__ A, T* __restrict
   const int lo = X0 + K, hi = min(g.nx - K, X0 + K + R::OUT);
   const bool whole = x0 >= lo && x0 + 2 <= hi;
   const bool some = !whole && x0 + 2 > lo && x0 < hi;
-  const CellConst<float2> k = cell_const<MODEL, kPinConst && !SHIFT, float2>(r, float(Store<T>::kScale));
+  const CellConst<float2> k = cell_const<MODEL, !SHIFT, float2>(r, float(Store<T>::kScale));
   const T* mine = ring + 2 * lane;
   int slot = 0;
   auto next = [](int sl) { return sl + 1 == R::DEPTH ? 0 : sl + 1; };
@@ -975,8 +974,9 @@ inline TilePlan plan_tiles(int nx, int ny, bool f64, bool px, bool py, int sms) 
 // twice rather than exchanged), the boundary's lookups are made once, and its
 // warps are left out of the rows.  Microseconds a step against the forms of
 // one launch per step or per tile plan: 128^2 channel (MRT) 2.4 against 2.7,
-// 300^2 f32 2.3 against 2.8, 613 x 377 f16 3.5 against 4.0.  In double the FP64 pipe is the bound and the boundary blocks'
-// share of it the longest: 200^2 12.5 against 9.1, so it is not built.
+// 320^2 f32 2.6 against 2.9, 613 x 377 f16 3.4 against 3.7.  In double the FP64
+// pipe is the bound and the boundary blocks' share of it the longest: 200^2
+// 12.5 against 9.1, so it is not built.
 // ---------------------------------------------------------------------------
 constexpr int kFlagStride = 8;  // a flag per 32 bytes
 
