@@ -309,6 +309,8 @@ int lbm_set_tiles(lbm_t* h, int32_t enable);
 /* How lbm_step launches the next steps, as set, as lbm_autotune chose or as it
  * picks itself: the form, the most steps one of its launches takes, and the
  * number of steps in a call from which on the domain stays resident (0: never).
+ * (Picked by itself on a small domain, the form of one launch per step leaves
+ * what its graphs of 16 steps do not take, from three steps on, to tiles.)
  * LBM_EINVAL for a NULL argument, LBM_ESTATE before lbm_bind or lbm_init*. */
 #define LBM_FORM_PAIR 0   /* bulk and NSBC kernels */
 #define LBM_FORM_FUSED 1  /* both in one launch (lbm_set_fused) */

@@ -87,7 +87,8 @@ constexpr int kReduceBlocks = 1216;  // 8 x 152 SMs
 constexpr int kNsbcThreads = 128;
 // where pick_form() draws the lines
 constexpr long long kPassNodes32 = 1200000, kPassNodes16 = 2800000, kTileNodes = 110000, kFusedNodes = 800000;
-constexpr long long kTileNodesEdge = 32000, kTileNodesEdge16 = 20000, kResidentNodesPeriodic = 5000;
+constexpr long long kTileNodesEdge = 32000, kTileNodesEdge16 = 20000;
+constexpr long long kResidentNodesPeriodic = 5000, kResidentNodesAxis = 45000, kResidentNodesAxisMrt = 25000;
 constexpr int kPassRows32 = 80, kPassRows16 = 320;
 constexpr long long kTileCells = 1 << 21;  // largest domain the autotuner tries as tiles
 // steps of a launch of the resident kernel: below, the flags' clearing and the
@@ -151,7 +152,7 @@ struct lbm {
   // no launch form was asked for: lbm_step takes the one pick_form() names
   bool form_auto = true;
   Form form = Form::Pair;  // what prepare_form() settled on
-  bool form_ready = false, rs_ready = false;
+  bool form_ready = false, rs_ready = false, tail_ready = false;
   // work counters and the resident tiles' flags: the library's own memory, as
   // bound scratch areas may be shared by handles or hold the caller's data
   // between two calls
@@ -546,10 +547,8 @@ lbmk::TilePlan tile_plan(const lbm_t* h) {
 template <typename T>
 int tiles_prepare(lbm_t* h) {
   const lbmk::TilePlan p = tile_plan(h);
-  if (p.steps == 0) {  // the edges were changed since lbm_set_tiles, and no tiling serves these
-    h->form = Form::Pair;
-    return LBM_OK;
-  }
+  h->tl_steps = 0;
+  if (p.steps == 0) return LBM_OK;
   h->tl_gx = p.gx;
   h->tl_gy = p.gy;
   h->tl_steps = p.steps;
@@ -781,13 +780,14 @@ Form pick_form(const lbm_t* h) {
 // launch:
 //   open, BGK at rest   620^2 f32 4.9 / 5.0   613 x 377 f16 3.4 / 3.7   1200 x 300 f16 4.6 / 4.0
 //   open, otherwise     320^2 MRT f32 3.25 / 3.26, 400^2 3.6 / 3.4   1000 x 100 3.3 / 3.0
-//   one periodic axis   160^2 f32 2.4 / 2.6, 240^2 2.7 / 2.6; MRT 160^2 3.0 / 2.9, 200^2 3.2 / 2.9
+//   one periodic axis   200^2 f32 2.54 / 2.56, bf16 2.3 / 2.7, 240^2 2.7 / 2.6; MRT 160^2 3.0 / 2.9, 200^2 3.2 / 2.9
 //   both                64^2 1.8 / 2.1, MRT 2.1 / 2.2; 128^2 2.2 / 2.1, MRT 2.7 / 2.2
 bool resident_serves(const lbm_t* h) {
   const long long nodes = (long long)h->nx * h->ny;
   const bool plain = h->collision == 0 && !zshift(h).on;
   const int axes = (h->nsbc.periodic_x != 0) + (h->nsbc.periodic_y != 0);
-  if (axes) return nodes <= (axes == 2 ? kResidentNodesPeriodic : kTileNodesEdge);
+  if (axes)
+    return nodes <= (axes == 2 ? kResidentNodesPeriodic : h->collision == 0 ? kResidentNodesAxis : kResidentNodesAxisMrt);
   return nodes <= (wide(h) && !plain ? kTileNodesEdge : kTileNodes) || (plain && !wide(h));
 }
 
@@ -816,13 +816,34 @@ int prepare_form(lbm_t* h) {
       using T = decltype(tag);
       if (h->form == Form::Tiles) {
         rc = tiles_prepare<T>(h);
+        if (h->tl_steps == 0) h->form = Form::Pair;  // the edges were changed since lbm_set_tiles: no tiling serves these
       } else if constexpr (!std::is_same<T, double>::value) {
         rc = pass_prepare<T>(h);
       }
     });
   h->rs_halo = 0;
   h->rs_ready = false;
+  h->tail_ready = h->form == Form::Tiles;
   h->form_ready = rc == LBM_OK;
+  return rc;
+}
+
+// The steps that the graphs of a small domain's one-launch form leave over go
+// out as tiles where there are three or more: launched one by one they take
+// the host 4 us each (calls of five steps, us a step, tiles / one launch: f16
+// 300^2 4.1 / 5.9, 100 x 1000 4.1 / 6.2; of three 5.0 / 5.8 and 5.5 / 6.2, f32
+// 223 x 43 3.4 / 4.2; of two, f16 300^2 6.2 / 5.9).
+constexpr int kTailSteps = 3;
+bool tail_serves(const lbm_t* h) {
+  const long long nodes = (long long)h->nx * h->ny;
+  return h->form_auto && h->form == Form::Fused && h->storage != LBM_F64 && tiles_ok(h) &&
+         nodes <= (wide(h) ? kTileNodesEdge : kTileNodes);
+}
+int prepare_tail(lbm_t* h) {
+  if (h->tail_ready) return LBM_OK;
+  int rc = LBM_OK;
+  dispatch(h->storage, [&](auto tag) { rc = tiles_prepare<decltype(tag)>(h); });
+  h->tail_ready = rc == LBM_OK;
   return rc;
 }
 
@@ -852,11 +873,12 @@ void enqueue_step(const lbm_t* h, int from, cudaStream_t s, bool fork);
 
 // One launch of `steps` steps (the form's own number or fewer) from buffer
 // `from` to 1 - from; the forms of one step take one.
-void enqueue_launch(const lbm_t* h, int from, int steps, cudaStream_t s, bool fork) {
-  if (h->form == Form::Tiles || (h->form == Form::Pass && steps > 1)) {
+// tail: as tiles, whatever the form.
+void enqueue_launch(const lbm_t* h, int from, int steps, cudaStream_t s, bool fork, bool tail) {
+  if (tail || h->form == Form::Tiles || (h->form == Form::Pass && steps > 1)) {
     dispatch(h->storage, [&](auto tag) {
       using T = decltype(tag);
-      if (h->form == Form::Tiles) {
+      if (tail || h->form == Form::Tiles) {
         launch_tiles<T>(h, h->buf[from], h->buf[1 - from], steps, s);
       } else if constexpr (!std::is_same<T, double>::value) {
         launch_pass<T>(h, h->buf[from], h->buf[1 - from], steps, s);
@@ -953,12 +975,12 @@ int enqueue_step_profiled(lbm_t* h, int from) {
 
 // A launch of several steps with an event pair around it (counted as one bulk
 // launch).
-int enqueue_launch_profiled(lbm_t* h, int from, int steps) {
+int enqueue_launch_profiled(lbm_t* h, int from, int steps, bool tail) {
   cudaEvent_t e[2];
   int rc = profiled_pair(h, 0, e);
   if (rc) return rc;
   cudaEventRecord(e[0], h->stream);
-  enqueue_launch(h, from, steps, h->stream, false);
+  enqueue_launch(h, from, steps, h->stream, false, tail);
   cudaEventRecord(e[1], h->stream);
   return LBM_OK;
 }
@@ -1308,18 +1330,25 @@ int lbm_step(lbm_t* h, int32_t n) {
       left -= kGraphSteps;  // kGraphSteps is even: h->cur is unchanged
     }
   }
+  int tail = !captured && left % kGraphSteps >= kTailSteps && tail_serves(h) ? left % kGraphSteps : 0;
+  if (tail) {
+    rc = prepare_tail(h);
+    if (rc) return rc;
+    if (h->tl_steps < 2) tail = 0;
+  }
   while (left > 0) {
-    int take = std::min(per, left);
+    const bool tiles = h->form == Form::Tiles || left <= tail;
+    const int most = tiles ? h->tl_steps : per;
+    int take = std::min(most, left);
     // a pass takes at least two steps: five are three and two, not four and one
     if (h->form == Form::Pass && left - take == 1 && take > 2) --take;
     // the last tile launches share what is left evenly
-    if (h->form == Form::Tiles) take = (left + (left + per - 1) / per - 1) / ((left + per - 1) / per);
+    if (tiles) take = (left + (left + most - 1) / most - 1) / ((left + most - 1) / most);
     if (captured) take = (int)((left + launches - 1) / launches--);
     if (!h->profiling)
-      enqueue_launch(h, h->cur, take, h->stream, false);
+      enqueue_launch(h, h->cur, take, h->stream, false, tiles);
     else
-      rc = take > 1 || h->form == Form::Tiles ? enqueue_launch_profiled(h, h->cur, take)
-                                              : enqueue_step_profiled(h, h->cur);
+      rc = take > 1 || tiles ? enqueue_launch_profiled(h, h->cur, take, tiles) : enqueue_step_profiled(h, h->cur);
     if (rc) return rc;
     h->cur ^= 1;
     left -= take;
@@ -1800,7 +1829,7 @@ int lbm_autotune(lbm_t* h, int32_t* threads_x, int32_t* rows, int32_t* prefetch_
         if (resident)
           enqueue_resident(h, per);
         else
-          enqueue_launch(h, k & 1, per, h->stream, false);
+          enqueue_launch(h, k & 1, per, h->stream, false, false);
       };
       for (int k = 0; k < (resident ? 1 : 2); ++k) launch(k);
       cudaEventRecord(e0, h->stream);

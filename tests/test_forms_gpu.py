@@ -132,3 +132,29 @@ def test_pair_with_and_without_prefetch(lbm, nx, ny, bx):
         assert form[0] == "pair"
         out += [ref, got]
     assert all(np.array_equal(out[0], a) for a in out[1:])
+
+
+@pytest.mark.parametrize("nx,ny,storage,setting", [(300, 300, "f16", SETTINGS[0]), (1000, 30, "f32", SETTINGS[0]),
+                                                   (43, 301, "f16", SETTINGS[3]), (200, 201, "bf16", SETTINGS[2])])
+def test_left_over_steps_as_tiles(lbm, nx, ny, storage, setting):
+    """What the graphs of the one-launch form leave: tiles from three steps on, the same bits."""
+    def choose(s):
+        lbm.lbm_profile(s.h, True)
+
+    def launches(s, n):
+        s.step(n)
+        return lbm.lbm_profile_read(s.h)[1]
+    ref, got, form = _runs(lbm, nx, ny, storage, setting, choose, (1, 3, 4, 5, 15, 16, 20, 31, 4))
+    assert form[0] == "fused"
+    assert np.array_equal(got, ref)
+    ref, got, _ = _runs(lbm, nx, ny, storage, setting, lambda s: None, (1, 3, 4, 5, 15, 16, 20, 31, 4))
+    assert np.array_equal(got, ref)
+    model, edges, far, order, corner = setting
+    with lbm.Simulation(nx, ny, 0.6, storage=storage, mrt_rates=(1.4, 1.4, 1.2), farfield_u=far, collision=model,
+                        edges=edges, grad_order=order, corner_mode=corner) as s:
+        s.init(*[np.full((ny, nx), b) for b in (1.0, far[0], far[1])])
+        lbm.lbm_profile(s.h, True)
+        assert launches(s, 2) == 2
+        assert launches(s, 3) < 3
+        assert launches(s, 15) < 15
+        assert 16 < launches(s, 20) < 20
