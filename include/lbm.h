@@ -479,7 +479,7 @@ int lbm_batch_set_launch(lbm_batch_t* b, int32_t threads_x, int32_t rows, int32_
  * for a lone step one batched step of the launch shape set.  enable != 0 turns
  * it on; lbm_batch_set_launch turns it off; a batch for which neither was
  * called takes passes when it is stored in f32, has a million nodes or more
- * and 34 or more to each node of its instances' perimeters
+ * and 24 or more (MRT: 34) to each node of its instances' perimeters
  * (lbm_batch_get_twostep then still reports 0; lbm_batch_passes tells).
  * lbm_batch_autotune times it against the other forms.  LBM_EINVAL when enabling it on f64 storage,
  * with a periodic axis, or with an instance smaller than 8 x 8.

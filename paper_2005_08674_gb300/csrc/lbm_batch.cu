@@ -623,15 +623,17 @@ bool batch_pass_ok(const lbm_batch_t* b) {
 // of kPassCells nodes or more (us a step, staged / pass: 0.34 M nodes 8.7 /
 // 9.1, 2.1 M 30 / 21, 3.9 M 53 / 37, 13.9 M 157 / 85; f16 13.9 M 95 / 104:
 // the 16-bit pass is bound by instructions, not by the traffic it saves) with
-// kPassInner nodes to each node of a perimeter or more, as a frame's tiles
+// so many nodes to each node of a perimeter or more, as a frame's tiles
 // compute every node several times (staged / pass, BGK and MRT, 1.2 .. 2 M
 // nodes: 8^2 at 3.5 to a perimeter node 112 / 348 and 132 / 422, 64^2 at 16
-// 24 / 29 and 26 / 34, 128^2 at 32 20.0 / 20.0 and 21 / 23, uneven ones at
-// 35.5 34 / 27 and 35 / 32, 160^2 at 40 19 / 15 and 20 / 19).
-constexpr long long kPassCells = 1000000, kPassInner = 34;
+// 24 / 29 and 26 / 34, 80^2 at 20 22.6 / 24.0 and 24 / 29, 96^2 at 24 23.3 /
+// 22.2 and 25 / 27, 128^2 at 32 20.0 / 20.0 and 21 / 23, uneven ones at 35.5
+// 34 / 27 and 35 / 32, 160^2 at 40 19 / 15 and 20 / 19; 5.5 M nodes of 96^2
+// 83 / 79 and 87 / 96).
+constexpr long long kPassCells = 1000000, kPassInner = 24, kPassInnerMrt = 34;
 bool batch_passes(const lbm_batch_t* b) {
   const bool want = b->form_auto ? b->storage == LBM_F32 && b->cells >= kPassCells &&
-                                       b->cells >= kPassInner * b->perimeter
+                                       b->cells >= (b->collision == 1 ? kPassInnerMrt : kPassInner) * b->perimeter
                                  : b->twostep;
   return want && batch_pass_ok(b);
 }
