@@ -388,8 +388,8 @@ int lbm_reduce_noalloc(lbm_t* h, const double* ref_rho, const double* ref_ux, co
 /* ------------------------------------------------------------------------
  * Batched mode: many independent simulations of uneven sizes, each with its
  * own tau and far field, stepped together by ONE persistent kernel launch
- * per step (bulk tiles and NSBC chunks of all instances in one work list),
- * replayed from a CUDA graph.  Storage, collision model and NSBC parameters
+ * per step (bulk tiles and NSBC chunks of all instances in one work list) or
+ * per pass of several steps, replayed from a CUDA graph.  Storage, collision model and NSBC parameters
  * are shared by the batch.  Results per instance are bit-identical to a
  * single-domain handle with the same settings.
  * ------------------------------------------------------------------------ */
@@ -495,8 +495,8 @@ int32_t lbm_batch_passes(const lbm_batch_t* b);
  * cudaMallocAsync) and keep the fastest. */
 int lbm_batch_autotune(lbm_batch_t* b, int32_t* threads_x, int32_t* rows, int32_t* blocks, int32_t* prefetch_rows,
                        int32_t* split, int32_t* tma_tile, double* ms_per_step);
-/* LBM_ETIMEOUT if a staged-tile wait of the shared-memory path gave up since
- * the batch was created (the step then left those tiles untouched); LBM_OK
+/* LBM_ETIMEOUT if a bounded wait of the shared-memory path or of a pass gave up
+ * since the batch was created (the step then left nodes untouched); LBM_OK
  * otherwise.  Synchronises. */
 int lbm_batch_status(lbm_batch_t* b);
 
