@@ -246,7 +246,7 @@ __global__ void wait_selftest_kernel(long long budget, int* flag) {
   __syncthreads();
   if (threadIdx.x == 0) {
     const bool a = mbar_wait(&bar, 0u, budget);
-    const bool b = lbmk::flag_wait(reinterpret_cast<const unsigned*>(flag + 1), 1u, budget);
+    const bool b = lbmk::flag_wait(reinterpret_cast<const unsigned*>(flag + 1), 1u, (unsigned)budget);
     flag[0] = !a && !b ? 1 : 2;
   }
 }

@@ -1041,14 +1041,16 @@ __device__ __forceinline__ void tile_halo(const T* B, const Geom& g, const TileH
 }
 
 // Whether *flag reaches `want` before `limit` SM clock cycles have passed (it
-// is looked at once in any case).
-__device__ __forceinline__ bool flag_wait(const unsigned* flag, unsigned want, long long limit) {
-  const long long t0 = clock64();
+// is looked at once in any case).  32 bits hold limits up to 4e9 cycles, with
+// 0.1 s and more between two looks; in 64 bits the wait cost a resident 128^2
+// channel 0.7 % (489 against 485 us for 200 steps).
+__device__ __forceinline__ bool flag_wait(const unsigned* flag, unsigned want, unsigned limit) {
+  const unsigned t0 = clock();
   for (;;) {
     unsigned seen;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
     if ((int)(seen - want) >= 0) return true;
-    if (clock64() - t0 >= limit) return false;
+    if ((unsigned)clock() - t0 >= limit) return false;
   }
 }
 
@@ -1058,7 +1060,7 @@ __device__ __forceinline__ bool flag_wait(const unsigned* flag, unsigned want, l
 template <typename T, int MODEL, bool SHIFT>
 __global__ void __launch_bounds__(kTileThreads)
     resident_kernel(T* A, T* B, Geom g, Nsbc p, Rates<typename Store<T>::C> r, int gx, int gy, int halo, int steps,
-                    unsigned* flags, long long limit, int* err) {
+                    unsigned* flags, unsigned limit, int* err) {
   using C = typename Store<T>::C;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   C* smem = reinterpret_cast<C*>(smem_raw);

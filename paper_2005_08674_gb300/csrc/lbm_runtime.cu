@@ -160,7 +160,7 @@ struct lbm {
   int sync_slot = -1;
   bool moved = false;  // to another stream, with a state
   bool waited = false;            // steps since the state was set hold bounded waits
-  long long wait_limit = lbmk::kTmaWaitCycles;  // of the resident tiles (lbm_set_wait_limit)
+  unsigned wait_limit = (unsigned)lbmk::kTmaWaitCycles;  // of the resident tiles (lbm_set_wait_limit)
   int4* d_items = nullptr;
   lbmk::InstDev* d_inst = nullptr;
   void* d_shift = nullptr;  // the far field's storage shift in the compute type (staged kernel)
@@ -690,7 +690,7 @@ cudaError_t launch_resident(lbm_t* h, int from, int steps, cudaStream_t s) {
   lbmk::Rates<C> r = rates<C>(h);
   int gx = h->rs_gx, gy = h->rs_gy, halo = h->rs_halo;
   unsigned* flags = resident_flags(h);
-  long long limit = h->wait_limit;
+  unsigned limit = h->wait_limit;
   int* err = sched(h);
   cudaError_t e =
       cudaMemsetAsync(flags, 0, (size_t)gx * gy * lbmk::kFlagStride * sizeof(unsigned), s);
@@ -1695,7 +1695,7 @@ int lbm_set_wait_limit(lbm_t* h, int64_t cycles) {
   if (!h) return fail(LBM_EINVAL, "lbm_set_wait_limit: NULL handle");
   if (cycles < 0 || cycles > 4000000000LL)
     return fail(LBM_EINVAL, "lbm_set_wait_limit: %lld outside [0, 4e9] cycles", (long long)cycles);
-  h->wait_limit = cycles;
+  h->wait_limit = (unsigned)cycles;
   return LBM_OK;
 }
 
